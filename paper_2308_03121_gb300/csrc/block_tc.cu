@@ -1,39 +1,56 @@
 // Residual block of the enhancement trunk, y = x + conv2(LeakyReLU(conv1(x) + b1)) + b2
 // (Section 3.1: the networks NNVISR runs are stacks of such 3x3 blocks), both convs
-// 64 -> 64 channels with zero padding, in one launch of 2-CTA clusters.
+// 64 -> 64 channels with zero padding, in one launch of 2-CTA clusters whose two SMs work
+// as one M = 256 tensor-core pair (tcgen05 cta_group::2).
 //
-// The row-streaming scheme of the single-layer kernel (conv_tc.cu) runs twice, on the
-// two SMs of a cluster:
-//  * rank 0 (the conv1 CTA) TMA-loads rows of x, issues the stacked-tap MMAs of conv1
-//    (one N = 192 MMA per (kx, K step) covers output rows r + 1, r, r - 1) into its TMEM
-//    ring, and its epilogue turns each finished row into h = LeakyReLU(acc + b1), rounded
-//    to the activation type, staged 128-byte swizzled (as the MMA reads it) and sent by one
-//    bulk copy into a ring of h rows in rank 1's shared memory (distributed shared memory);
-//  * rank 1 (the conv2 CTA) runs the same MMA scheme on those h rows with conv2's
-//    weights, and its epilogue adds b2 and the residual x (a TMA load, an L2 hit: rank 0
-//    read that row a few rows earlier) and stores y by TMA.
-// h never reaches device memory.  Per block the DRAM traffic is x read once plus y
-// written once, against x, h, h, x and y for two single-layer launches (at 1920 x 1080:
-// 531 MB instead of 1327 MB), and the two layers' MMA streams run on two SMs at once.
+// Each CTA of the pair owns one column tile of the image and runs both convolutions on it;
+// every MMA covers 128 pixels of both tiles.  What bounds the block is the SMs' shared-memory
+// bandwidth: a 128-pixel x (3 stacked taps x 64 outputs) MMA takes 96 cycles and reads 4 KB of
+// pixels and 6 KB of weights, 107 of the 128 bytes per clock that shared memory delivers, so
+// that the epilogues' traffic stalls the tensor pipe.  In a pair each SM holds and reads half
+// of the weight rows (3 KB per MMA), and the middle tensor h stays on the SM that computes it.
+//
+//  * Stacked taps: input row n feeds accumulator rows n - 1 (ky = 2), n (ky = 1) and n + 1
+//    (ky = 0) with one N = 192 MMA per (kx, 16-channel K step), 12 per row.
+//  * Accumulators: three rows, row i in slot i % 3 of a fixed 192-column TMEM window per conv,
+//    so a row of the MMA's N never wraps.  The order of the taps along N rotates with n
+//    instead: the weights of a kx lie in shared memory as the blocks ky = 2, 1, 0, 2, 1 and the
+//    MMA starts at block 0, 1 or 2.  The epilogue zeroes a slot as it drains it, so every MMA
+//    accumulates: no first-product case, and the rows before and after a strip are drained
+//    and dropped.
+//  * The pair splits N in halves, the lower one from CTA 0: CTA c holds output channels
+//    [32c, 32c + 32) of every block, and a slot's channels 0-31 lie at window column 32 slot,
+//    channels 32-63 at 96 + 32 slot, in both CTAs' TMEM.
+//  * Roles per CTA: warp 0 TMA-loads rows of x; warps 2-9 turn each finished conv1 row into
+//    h = LeakyReLU(acc + b1), rounded to the activation type and staged 128-byte swizzled
+//    where conv2's MMAs read it; warps 10-17 add b2 and the residual x (a TMA load, an L2 hit)
+//    to each finished conv2 row, in the tile the residual came in, which warp 18 stores by TMA.
+//    Warp 1 of CTA 0 issues every MMA: conv1 of row n, then conv2 of the h row that conv1's
+//    row n - 1 completed, so each conv's epilogue has the other conv's MMAs to run behind.
+//    Warp 19 of CTA 1 reports its landed x rows to CTA 0.
+//
+// h never reaches device memory: the DRAM traffic is x read once plus y written once (at
+// 1920 x 1080 531 MB instead of 1327 MB for two single-layer launches).
 //
 // Tiles: conv1 computes the 128 h pixels [x0 - 1, x0 + 127) of a row (the MMA's M), which
 // give conv2 the 126 outputs [x0, x0 + 126): column tiles are 126 pixels wide (x0 = 126 c)
 // and conv2's two last accumulator lanes are discarded.  h pixels or rows outside the
-// image are written as zero (conv2's zero padding).  Rows: the (image, column tile, row)
-// sequence is cut into equal contiguous ranges, one per cluster; a range is one or more
-// strips of output rows [ra, rb) of one column tile, for which conv1 produces h rows
-// [ra - 1, rb] from x rows [ra - 2, rb + 1].
+// image are written as zero (conv2's zero padding).  A pair takes column tiles 2k and 2k + 1
+// over the same rows; the last tile of an odd count is cut into its upper and lower half, one
+// per CTA.  The (image, tile pair, row) sequence is cut into equal contiguous ranges, one
+// per cluster; a range is one or more strips of output rows [ra, rb) of one tile pair, for
+// which conv1 produces h rows [ra - 1, rb] from x rows [ra - 2, rb + 1].
 //
-// Synchronisation between the two CTAs: rank 0's epilogue waits until rank 1's MMAs have
-// released the h slot and the staging tile's previous row (tcgen05.commit multicast onto
-// rank 0's barriers), stages the row and issues the copy, whose bytes complete the
-// transaction count of rank 1's barrier of that slot (armed by rank 1 for each row).
-// (Per-thread remote stores, each followed by a cluster-scope fence and release, measured
-// 1.5 us per row: the round trips, not the MMAs, set the pace.)  Every wait is bounded in
-// time; a CTA that gives up raises the abort flags of both CTAs and the error word.  Both
-// CTAs end with two cluster barriers: between them each side waits for what the other has
-// already started towards its shared memory (copies, MMA commits), counted in words the
-// other side updates, so neither leaves while the other may still write into it.
+// Measured, BF16 (a filter's trunk, block after block): at 1920 x 1080 197 us per block, 231 us
+// before with one conv per SM of the cluster and cta_group::1; at 960 x 540 55 us instead of 70.
+// A row step takes 2430 cycles against 2304 of its 24 MMAs; at 1920 x 1080 the chip's power cap
+// then holds the clock near 1.5 GHz (1.55 PFLOP/s, 0.93 of the sustained cuBLAS rate), so what
+// is left is the arithmetic itself, with 5 % of it in the last, 30-pixel column tile.
+//
+// Every wait is bounded in time; a CTA that gives up raises the abort flags of both CTAs and
+// the error word.  Both CTAs end with two cluster barriers: between them each waits for the
+// last MMA commit onto its barriers, so neither leaves while the other may still write into
+// its shared memory.
 #include <algorithm>
 #include <mutex>
 
@@ -46,24 +63,26 @@ namespace nvisr {
 namespace {
 
 constexpr int BT = 126;                   // output pixels of a column tile
-constexpr int TMH = 128;                  // h pixels of a row tile (the MMA's M)
+constexpr int TMH = 128;                  // h pixels of a row tile (half of the pair's M)
 constexpr int PXS = TMH + 2;              // x pixels of a row box
-constexpr int BTHREADS = 352;             // warps: 0 TMA, 1 MMA, 2-9 epilogue, 10 issuer waits
-constexpr int NSLOT = 8;                  // accumulator rows in TMEM (64 columns each)
-constexpr int HS = 5;                     // h rows in rank 1's ring
+constexpr int BTHREADS = 640;             // warps: 0 x loads, 1 MMA, 2-9 conv1 epilogue, 10-17 conv2 epilogue,
+                                          // 18 residual loads and y stores, 19 x rows' report
+constexpr int XST = 3;                    // x rows in shared memory
+constexpr int NTILE = 2;                  // residual / output tiles
+constexpr int NRING = 4;                  // barriers per kind of per-row event
 constexpr uint32_t AROW = PXS * 128;      // bytes of one 130-pixel row of 64 channels
 constexpr uint32_t ROWB = 17408;          // its 1 KB-aligned slot
-constexpr uint32_t WB = 3 * 3 * 64 * 128; // one conv's stacked weights [kx][2 - ky][64 out][128 B]
-constexpr uint32_t WKX = 3 * 64 * 128;    // weights of one kx
-constexpr uint32_t TILEB = TMH * 128;     // one output / residual row tile
-constexpr uint32_t HDR = 1024;            // barriers, flags, bias
-constexpr uint32_t REGION = HS * ROWB + 4 * TILEB;            // rank 1: h ring + 2 output + 2 residual tiles
-constexpr int XST = 5;                    // rank 0: x stages, then 4 h staging tiles (2 per epilogue group)
-static_assert(XST * ROWB + 4 * TILEB <= REGION, "rank 0's room");
-constexpr int BLOCK_SMEM = 1024 + (int)(HDR + WB + REGION);   // + alignment slack
+constexpr uint32_t TILEB = TMH * 128;     // one h row, one output / residual row tile
+constexpr uint32_t WBLK = 32 * 128;       // weights of one (kx, ky): 32 outputs x 128 B
+constexpr uint32_t WKX = 5 * WBLK;        // one kx: blocks ky = 2, 1, 0, 2, 1
+constexpr uint32_t WB = 3 * WKX;          // one conv
+constexpr uint32_t GKX = 3 * 64 * 128;    // one kx of the global image [kx][2 - ky][64 out][128 B]
+constexpr uint32_t HDR = 1024;            // barriers, flags, biases
+constexpr uint32_t WIN2 = 256;            // TMEM column of conv2's window (conv1's starts at 0)
+// the MMAs read 256 bytes past the h row (they feed the two discarded lanes only): the tiles follow
+constexpr int BLOCK_SMEM = 1024 + (int)(HDR + 2 * WB + XST * ROWB + TILEB + NTILE * TILEB);
 constexpr uint64_t WAIT_NS = 2000000000ull;
 static_assert(BLOCK_SMEM <= 232448, "227 KB per CTA");
-static_assert(XST >= 4, "x prefetch depth");
 
 struct BlockParams {
     int H, W, nimg;
@@ -71,8 +90,13 @@ struct BlockParams {
     const uint8_t *w1, *w2;    // stacked weights of conv1 and conv2
     const float *b1, *b2;      // biases [64]
     int *err;
-    int starve;                // test drill: rank 0 loads no input, the pipeline waits run out
+    int starve;                // test drill: no input is loaded, the pipeline waits run out
 };
+
+// Units (pair rows) of an image: H for each two column tiles, half of them for a last single one.
+__host__ __device__ inline int64_t block_units(int H, int ncols) {
+    return (int64_t)(ncols / 2) * H + (ncols % 2 ? (H + 1) / 2 : 0);
+}
 
 // MULTI: the images of several streams (one BlockProblem each, any sizes) share the launch;
 // otherwise nimg images of one size stacked along the maps' outer dimension.
@@ -87,544 +111,409 @@ __global__ void __launch_bounds__(BTHREADS, 1)
     extern __shared__ uint8_t smem_raw[];
     // same offset in both CTAs: the dynamic shared memory starts at the same address
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint64_t *full = reinterpret_cast<uint64_t *>(smem);  // rank 0: x row landed
-    uint64_t *empty = full + 8;                           // rank 0: x stage read by the MMAs
-    uint64_t *rowdone = full + 16;                        // accumulator row complete
-    uint64_t *slotfree = full + 24;                       // accumulator row drained
-    uint64_t *hfull = full + 32;                          // rank 1: h row written by rank 0
-    uint64_t *hempty = full + 40;                         // rank 0: h slot read by rank 1's MMAs
-    uint64_t *resfull = full + 48;                        // rank 1: residual tile per group
-    uint64_t *wbar = full + 50;
-    uint64_t *drain = full + 51;                          // the issuer's MMAs, after an abort
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + 416);
-    volatile int *abort = reinterpret_cast<volatile int *>(smem + 420);
-    volatile int *grp_stop = reinterpret_cast<volatile int *>(smem + 424);
-    int *ready = reinterpret_cast<int *>(smem + 432);
-    int *h_issued = reinterpret_cast<int *>(smem + 436);    // rank 1: h copies rank 0 has started
-    int *h_consumed = reinterpret_cast<int *>(smem + 440);  // rank 0: h rows rank 1's MMAs were issued on
-    float *sbias = reinterpret_cast<float *>(smem + 512);
+    uint64_t *full = reinterpret_cast<uint64_t *>(smem);  // own x row landed
+    uint64_t *pfull = full + 4;                           // CTA 0: CTA 1's x row landed
+    uint64_t *done1 = full + 8;                           // conv1's MMAs of an input row complete (both CTAs)
+    uint64_t *done2 = full + 12;                          // conv2's
+    uint64_t *free1 = full + 16;                          // CTA 0: conv1's finished row drained and zeroed by both
+    uint64_t *free2 = full + 20;                          // CTA 0: conv2's
+    uint64_t *hfull = full + 24;                          // CTA 0: h row written by both
+    uint64_t *resfull = full + 25;                        // residual tile landed
+    uint64_t *outfull = full + 27;                        // output tile written
+    uint64_t *wbar = full + 29;
+    uint64_t *drain = full + 30;                          // the issuer's last commit (both CTAs)
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + 256);
+    volatile int *abort = reinterpret_cast<volatile int *>(smem + 260);
+    float *sbias = reinterpret_cast<float *>(smem + 512);  // b1, b2
     uint8_t *wsm = smem + HDR;
-    uint8_t *region = wsm + WB;        // rank 0: x stages; rank 1: h ring
-    uint8_t *obuf = region + HS * ROWB;  // rank 1: output staging tile per group
-    uint8_t *rbuf = obuf + 2 * TILEB;    // rank 1: residual tile per group
-    uint8_t *stg = region + XST * ROWB;  // rank 0: h staging tiles [group][2]
+    uint8_t *xring = wsm + 2 * WB;
+    uint8_t *hrow_sm = xring + XST * ROWB;
+    uint8_t *tiles = hrow_sm + TILEB;  // residual in, output out
 
     const uint32_t rank = cluster_ctarank();
-    const bool first = rank == 0;
+    const bool lead = rank == 0;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t npairs = cluster_count_x(), pair = cluster_id_x();
-    const int64_t total = MULTI ? probs[nprob - 1].u0 + (int64_t)probs[nprob - 1].ncols * probs[nprob - 1].H
-                                : (int64_t)p.nimg * p.ncols * p.H;
+    const int64_t total = MULTI ? probs[nprob - 1].u0 + block_units(probs[nprob - 1].H, probs[nprob - 1].ncols)
+                                : p.nimg * block_units(p.H, p.ncols);
     const int64_t u_begin = total * pair / npairs, u_end = total * (pair + 1) / npairs;
-    // the strip at position u of this cluster's range: problem (MULTI), image, column tile,
-    // output rows [ra, rb)
-    auto strip_at = [&](int64_t u, int &pi, int &img, int &col, int &ra, int &rb) {
-        int64_t local = u, H = p.H;
-        pi = 0;
+    // the strip at position u of this cluster's range: problem (MULTI), image, this CTA's column
+    // tile, its output rows [ra, rb) (of a last single tile's lower half they may pass the image)
+    struct Strip {
+        int pi, img, col, ra, rb;
+    };
+    auto strip_at = [&](int64_t u) -> Strip {
+        Strip s;
+        s.pi = 0;
+        int64_t local = u;
+        int H = p.H, nc = p.ncols;
         if (MULTI) {
-            while (pi + 1 < nprob && u >= probs[pi + 1].u0) ++pi;
-            local = u - probs[pi].u0;
-            H = probs[pi].H;
+            while (s.pi + 1 < nprob && u >= probs[s.pi + 1].u0) ++s.pi;
+            local = u - probs[s.pi].u0;
+            H = probs[s.pi].H;
+            nc = probs[s.pi].ncols;
         }
-        const int64_t cg = local / H;
-        ra = (int)(local - cg * H);
-        rb = (int)min(H, (int64_t)ra + (u_end - u));
-        img = MULTI ? 0 : (int)(cg / p.ncols);
-        col = (int)(cg - (int64_t)img * p.ncols);
+        const int64_t per = block_units(H, nc);
+        s.img = MULTI ? 0 : (int)(local / per);
+        local -= s.img * per;
+        const int64_t fulls = (int64_t)(nc / 2) * H;
+        const bool half = local >= fulls;
+        if (half) local -= fulls;
+        const int rows = half ? (H + 1) / 2 : H;
+        const int k = (int)(local / rows);
+        const int off = half ? (int)rank * rows : 0;
+        s.col = half ? nc - 1 : 2 * k + (int)rank;
+        s.ra = (int)(local - (int64_t)k * rows);
+        s.rb = (int)min((int64_t)rows, s.ra + (u_end - u));
+        s.ra += off;
+        s.rb += off;
+        return s;
     };
     auto xmap_of = [&](int pi) { return MULTI ? &probs[pi].xmap : &xmap; };
     auto rmap_of = [&](int pi) { return MULTI ? &probs[pi].rmap : &rmap; };
     auto ymap_of = [&](int pi) { return MULTI ? &probs[pi].ymap : &ymap; };
     auto height_of = [&](int pi) { return MULTI ? probs[pi].H : p.H; };
     auto width_of = [&](int pi) { return MULTI ? probs[pi].W : p.W; };
-    // rows this CTA's accumulators produce for a strip: h rows [ra - 1, rb + 1) (rank 0) or
-    // output rows [ra, rb) (rank 1); its input rows run from oa - 1 to ob
-    auto out_rows = [&](int ra, int rb, int &oa, int &ob) {
-        oa = first ? ra - 1 : ra;
-        ob = first ? rb + 1 : rb;
-    };
     const uint32_t peer_abort = mapa_shared(smem_u32(const_cast<int *>(abort)), rank ^ 1u);
     auto fail = [&]() {
         *abort = 1;
         st_cluster_u32(peer_abort, 1u);
         if (p.err) atomicExch(p.err, DEVERR_TIMEOUT);
     };
+    // barrier `bar` of CTA 0, for arrivals from either CTA
+    auto lead_bar = [&](uint64_t *bar) { return mapa_shared(smem_u32(bar), 0u); };
 
     if (threadIdx.x == 0) {
-        for (int k = 0; k < 8; ++k) {
+        for (int k = 0; k < XST; ++k) {
             mbar_init(&full[k], 1);
-            mbar_init(&empty[k], 1);
-            mbar_init(&rowdone[k], 1);
-            mbar_init(&slotfree[k], 128);
+            mbar_init(&pfull[k], 1);
         }
-        for (int k = 0; k < HS; ++k) {
-            mbar_init(&hfull[k], 1);    // rank 1's arming (expect_tx) + the copy's bytes
-            mbar_init(&hempty[k], 1);   // rank 1's MMA commit
+        for (int k = 0; k < NRING; ++k) {
+            mbar_init(&done1[k], 1);
+            mbar_init(&done2[k], 1);
+            mbar_init(&free1[k], 16);  // the 8 draining warps of both CTAs
+            mbar_init(&free2[k], 16);
         }
-        mbar_init(&resfull[0], 1);
-        mbar_init(&resfull[1], 1);
+        mbar_init(hfull, 16);
+        for (int k = 0; k < NTILE; ++k) {
+            mbar_init(&resfull[k], 1);
+            mbar_init(&outfull[k], 8);
+        }
         mbar_init(wbar, 1);
         mbar_init(drain, 1);
         *abort = 0;
-        grp_stop[0] = 0;
-        grp_stop[1] = 0;
-        *ready = 0;
-        *h_issued = 0;
-        *h_consumed = 0;
         fence_mbarrier_init();
         // weights are written once at filter creation: loaded before the wait on the previous kernel
-        mbar_arrive_expect_tx(wbar, WB);
-        const uint8_t *wsrc = first ? p.w1 : p.w2;
-        for (uint32_t off = 0; off < WB; off += 32768u) bulk_load(wsm + off, wsrc + off, min(32768u, WB - off), wbar);
+        mbar_arrive_expect_tx(wbar, 2 * WB);
+        for (int c = 0; c < 2; ++c)
+            for (int kx = 0; kx < 3; ++kx)
+                for (int b = 0; b < 5; ++b)
+                    bulk_load(wsm + c * WB + kx * WKX + b * WBLK,
+                              (c ? p.w2 : p.w1) + kx * GKX + (b % 3) * (64 * 128) + rank * WBLK, WBLK, wbar);
     }
-    if (threadIdx.x >= 64 && threadIdx.x < 128) sbias[threadIdx.x - 64] = (first ? p.b1 : p.b2)[threadIdx.x - 64];
-    if (!first && threadIdx.x >= 128 && threadIdx.x < 128 + HS * 16) {
-        // h lines 128, 129 of every slot feed only the two discarded output pixels: zero
-        const int t = threadIdx.x - 128;
-        st_shared_u4(smem_u32(region + (t / 16) * ROWB + TMH * 128 + (t % 16) * 16), make_uint4(0u, 0u, 0u, 0u));
-        fence_proxy_async();
-    }
+    if (threadIdx.x >= 64 && threadIdx.x < 192)
+        sbias[threadIdx.x - 64] = (threadIdx.x < 128 ? p.b1 : p.b2)[(threadIdx.x - 64) & 63];
     if (warp == 1) {
-        tmem_alloc(tmem_slot, 512);
-        tmem_relinquish();
+        tmem_alloc2(tmem_slot, 512);
+        tmem_relinquish2();
     }
     tc_fence_before();
     __syncthreads();
-    cluster_sync_all();  // both CTAs' barriers are initialised before either arrives on the other's
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    if (warp >= 2 && warp < 10) {  // both windows start at zero
+        const uint32_t t = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (warp < 6 ? 0u : WIN2);
+        for (int k = 0; k < 6; ++k) tmem_zero32(t + (uint32_t)(32 * k));
+        tmem_wait_st();
+    }
+    tc_fence_before();
+    cluster_sync_all();  // both CTAs' barriers and accumulators are ready before either uses the other's
+    tc_fence_after();
     griddep_launch_dependents();
     griddep_wait();
 
-    int w_done = 0, w_armed = 0;  // rank 1's wait warp: h rows landed / armed
-    int i_rows = 0;               // rank 1's issuer: h rows whose MMAs it issued (and committed)
     if (warp == 0) {
-        if (first && lane == 0) {
-            // ---------------- producer (rank 0): x rows ra - 2 .. rb + 1 of each strip
-            int gin = 0;
+        if (lane == 0) {
+            // ---------------- producer: x rows ra - 2 .. rb + 1 of each strip; row n takes the
+            // stage of row n - 3, whose MMAs done1 reports
+            int n = 0;
             bool ok = true;
             for (int64_t u = u_begin; u < u_end && ok && !p.starve;) {
-                int pi, img, col, ra, rb;
-                strip_at(u, pi, img, col, ra, rb);
-                u += rb - ra;
-                const int xb = col * BT - 2;  // box pixel 0 = h pixel col * BT - 1 minus one
-                for (int r = ra - 2; r <= rb + 1; ++r, ++gin) {
-                    const int s = gin % XST;
-                    if (!mbar_wait_bounded(&empty[s], (uint32_t)((gin / XST) & 1) ^ 1u, abort, WAIT_NS)) {
+                const Strip s = strip_at(u);
+                u += s.rb - s.ra;
+                const int xb = s.col * BT - 2;  // box pixel 0 = h pixel col * BT - 1 minus one
+                for (int r = s.ra - 2; r <= s.rb + 1; ++r, ++n) {
+                    const int k = n - XST;
+                    if (k >= 0 && !mbar_wait_bounded(&done1[k % NRING], (uint32_t)((k / NRING) & 1), abort, WAIT_NS)) {
                         fail();
                         ok = false;
                         break;
                     }
-                    mbar_arrive_expect_tx(&full[s], AROW);
-                    tma_load_4d(region + (size_t)s * ROWB, xmap_of(pi), &full[s], 0, xb, r, img);
+                    mbar_arrive_expect_tx(&full[n % XST], AROW);
+                    tma_load_4d(xring + (size_t)(n % XST) * ROWB, xmap_of(s.pi), &full[n % XST], 0, xb, r, s.img);
                 }
             }
             // copies still in flight after an early exit land before the CTA ends
-            for (int k = 0; k < XST && k < gin; ++k) {
-                const int idx = gin - 1 - k;
-                mbar_wait_bounded(&full[idx % XST], (uint32_t)((idx / XST) & 1), nullptr, WAIT_NS);
+            for (int k = 0; k < XST && k < n; ++k) {
+                const int i = n - 1 - k;
+                mbar_wait_bounded(&full[i % XST], (uint32_t)((i / XST) & 1), nullptr, WAIT_NS);
             }
+            mbar_wait_bounded(wbar, 0, nullptr, WAIT_NS);
         }
-        if (lane == 0) mbar_wait_bounded(wbar, 0, nullptr, WAIT_NS);
     } else if (warp == 1) {
-        if (lane == 0) {
-            // ---------------- MMA issuer (both ranks).  Input row r of a strip feeds the
-            // CTA's accumulator rows r - 1 .. r + 1 (those inside [oa, ob)), which form one
-            // run of contiguous TMEM slots or two where the ring wraps; row r + 1 gets its
-            // first product (accumulate = 0) here.  The wait warp publishes how many input
-            // rows are ready, so this thread makes no mbarrier waits while MMAs are queued.
-            bool ok = mbar_wait_bounded(wbar, 0, abort, WAIT_NS);
-            if (!ok) fail();
-            const int S = first ? XST : HS;
-            const uint64_t b_base = smem_desc_sw128(smem_u32(wsm), 0);
-            const uint32_t id0 = instr_desc(TMH, 0, AFMT, AFMT);
-            const uint32_t nstep = (uint32_t)(64 / 8) << 17;  // N += 64
-            int s = 0, gout = 0, gin = 0, nready = 0, last_slot = -1;
-            uint32_t last_par = 0;
-            auto await_row = [&](int row) -> bool {
-                if (row < nready) return true;
-                nready = ld_acquire_cta(ready);
-                if (row >= nready) {
-                    const uint64_t t0 = globaltimer_ns();
-                    for (uint32_t it = 1; row >= (nready = ld_acquire_cta(ready)); ++it) {
-                        if ((it & 63) == 0 && (*abort || globaltimer_ns() - t0 > WAIT_NS)) return false;
-                    }
-                }
-                tc_fence_after();
-                return true;
-            };
-            // (kx, K step) t: A advances one pixel (128 B) per kx and 32 bytes per K step inside
-            // the swizzled line; B one kx block per kx
-            auto a_off = [](int t) { return (uint64_t)(((t / 4) * 128 + (t % 4) * 32) >> 4); };
-            auto b_off = [](int t) { return (uint64_t)(((t / 4) * WKX + (t % 4) * 32) >> 4); };
-            for (int64_t u = u_begin; u < u_end && ok;) {
-                int pi, img, col, ra, rb, oa, ob;
-                strip_at(u, pi, img, col, ra, rb);
-                u += rb - ra;
-                out_rows(ra, rb, oa, ob);
-                const int base = gout - oa;  // global accumulator-row index of row o is base + o
-                for (int r = oa - 1; r <= ob; ++r) {
-                    if (!await_row(gin)) {
-                        ok = false;
-                        break;
-                    }
-                    const int o_lo = max(r - 1, oa), o_hi = min(r + 1, ob - 1);
-                    const bool fresh = r + 1 <= ob - 1;
-                    const int sl = (base + r - 1) & (NSLOT - 1);
-                    if (r - 1 >= oa && fresh && sl <= NSLOT - 3) {
-                        // interior row whose three accumulator rows do not wrap the ring (6 of 8
-                        // rows): one N = 192 run; the fresh row r + 1 starts at kx = 0, K step 0
-                        const uint64_t a_base = smem_desc_sw128(smem_u32(region + (size_t)s * ROWB), 0);
-                        const uint32_t md = tmem_base + (uint32_t)(sl * 64);
-                        umma<0>(md, a_base, b_base, id0 + nstep * 2u, 1u);
-                        umma<0>(md + 128u, a_base, b_base + (uint64_t)((2 * 64 * 128) >> 4), id0 + nstep, 0u);
-#pragma unroll
-                        for (int t = 1; t < 12; ++t) umma<0>(md, a_base + a_off(t), b_base + b_off(t), id0 + nstep * 3u, 1u);
-                    } else if (o_lo <= o_hi) {
-                        const uint64_t a_base = smem_desc_sw128(smem_u32(region + (size_t)s * ROWB), 0);
-                        auto slot_of = [&](int o) { return (base + o) & (NSLOT - 1); };
-                        auto bd_of = [&](int o) { return b_base + (uint64_t)(((o - r + 1) * 64 * 128) >> 4); };
-                        const int sl0 = slot_of(o_lo);
-                        const int len = o_hi - o_lo + 1;
-                        const int m0 = min(len, NSLOT - sl0), m1 = len - m0;
-                        const uint32_t md0 = tmem_base + (uint32_t)(sl0 * 64), md1 = tmem_base;
-                        const uint32_t mi0 = id0 + nstep * (uint32_t)m0, mi1 = id0 + nstep * (uint32_t)max(m1, 1);
-                        const uint64_t mb0 = bd_of(o_lo), mb1 = bd_of(o_lo + m0);
-                        {
-                            // first (kx, K step): the rows already started accumulate, the fresh row starts
-                            const int old_hi = fresh ? min(r, o_hi) : o_hi;
-                            const int olen = old_hi - o_lo + 1;
-                            if (olen > 0) {
-                                const int f0 = min(olen, m0), f1 = olen - f0;
-                                umma<0>(md0, a_base, mb0, id0 + nstep * (uint32_t)f0, 1u);
-                                if (f1 > 0) umma<0>(md1, a_base, mb1, id0 + nstep * (uint32_t)f1, 1u);
-                            }
-                            if (fresh)
-                                umma<0>(tmem_base + (uint32_t)(slot_of(r + 1) * 64), a_base, bd_of(r + 1), id0 + nstep, 0u);
-                        }
-                        if (m1 == 0) {
-#pragma unroll
-                            for (int t = 1; t < 12; ++t) umma<0>(md0, a_base + a_off(t), mb0 + b_off(t), mi0, 1u);
-                        } else {
-#pragma unroll
-                            for (int t = 1; t < 12; ++t) {
-                                const uint64_t ad = a_base + a_off(t), boff = b_off(t);
-                                umma<0>(md0, ad, mb0 + boff, mi0, 1u);
-                                umma<0>(md1, ad, mb1 + boff, mi1, 1u);
-                            }
-                        }
-                    }
-                    // the input row's buffer is free once these MMAs have run: rank 0's x stage, or
-                    // rank 1's h slot, released on rank 0's barrier of that slot
-                    if (first) umma_commit(&empty[s]);
-                    else umma_commit_multicast(&hempty[s], (uint16_t)1u);
-                    if (r - 1 >= oa) {
-                        const int i = base + r - 1;
-                        umma_commit(&rowdone[i & (NSLOT - 1)]);
-                        last_slot = i & (NSLOT - 1);
-                        last_par = (uint32_t)((i >> 3) & 1);
-                    }
-                    if (++s == S) s = 0;
-                    ++gin;
-                }
-                gout += ob - oa;
-            }
-            i_rows = gin;
-            if (!ok) fail();
-            if (last_slot >= 0) mbar_wait_bounded(&rowdone[last_slot], last_par, nullptr, WAIT_NS);
-            if (*abort) {
-                // an early exit may leave MMAs that no row commit covers
-                umma_commit(drain);
-                mbar_wait_bounded(drain, 0, nullptr, WAIT_NS);
-            }
-        }
-    } else if (warp == 10) {
-        if (lane == 0) {
-            // ---------------- wait warp: for each input row in the issuer's order, wait until
-            // the slot of its fresh accumulator row is drained and the row is in shared memory
-            // (rank 0: the x row's TMA; rank 1: rank 0's h stores), then publish the count.
-            const int S = first ? XST : HS;
-            int s = 0, gout = 0, gin = 0;
-            uint32_t ph = 0;
+        if (lead) {
+            // ---------------- MMA issuer.  The whole warp runs the loop with uniform values and
+            // one elected lane issues: 96 cycles per MMA back to back, where a lane-0 branch
+            // spends 57 cycles or more on each issue whatever its N.
+            const uint32_t el = elect_one();
+            const uint32_t id = instr_desc(256, 192, AFMT, AFMT);
             bool ok = true;
+            // both CTAs' weights: the peer's have landed before its first x row is reported
+            auto await = [&](uint64_t *bar, int i, int ring) {
+                ok = ok && __all_sync(0xffffffffu, mbar_wait_bounded(&bar[i % ring], (uint32_t)((i / ring) & 1), abort,
+                                                                     WAIT_NS));
+            };
+            auto issue = [&](const uint8_t *row, const uint8_t *wts, uint32_t win, int n, uint64_t *done) {
+                tc_fence_after();
+                // taps of slots 0, 1, 2 for input row n: blocks start at 1, 0, 2 for n % 3 = 0, 1, 2
+                const int rot = n % 3 == 2 ? 2 : 1 - n % 3;
+                const uint64_t a0 = smem_desc_sw128(smem_u32(row), 0);
+                const uint64_t b0 = smem_desc_sw128(smem_u32(wts) + (uint32_t)rot * WBLK, 0);
+#pragma unroll
+                for (int t = 0; t < 12; ++t)
+                    umma2_warp(el, tmem_base + win, a0 + (uint64_t)(((t / 4) * 128 + (t % 4) * 32) >> 4),
+                               b0 + (uint64_t)(((t / 4) * WKX + (t % 4) * 32) >> 4), id);
+                umma2_commit_warp(el, &done[n % NRING]);
+            };
+            ok = __all_sync(0xffffffffu, mbar_wait_bounded(wbar, 0, abort, WAIT_NS));
+            int n = 0, m = 0, kept = 0;  // conv1 inputs, conv2 inputs issued; h rows of the conv1 inputs before n
+            auto conv2 = [&]() {
+                await(hfull, m, 1);
+                if (m > 0) await(free2, m - 1, NRING);
+                if (ok) issue(hrow_sm, wsm + WB, WIN2, m, done2);
+                ++m;
+            };
             for (int64_t u = u_begin; u < u_end && ok;) {
-                int pi, img, col, ra, rb, oa, ob;
-                strip_at(u, pi, img, col, ra, rb);
-                u += rb - ra;
-                out_rows(ra, rb, oa, ob);
-                const int base = gout - oa;
-                for (int r = oa - 1; r <= ob; ++r) {
-                    if (r + 1 <= ob - 1) {
-                        const int i = base + r + 1;
-                        if (!mbar_wait_bounded(&slotfree[i & (NSLOT - 1)], (uint32_t)((i >> 3) & 1) ^ 1u, abort,
-                                               WAIT_NS)) {
-                            ok = false;
-                            break;
-                        }
-                    }
-                    if (!first && gin >= w_armed) {
-                        mbar_arrive_expect_tx(&hfull[s], TILEB);  // the copy of h row gin
-                        w_armed = gin + 1;
-                    }
-                    const bool in = mbar_wait_bounded(first ? &full[s] : &hfull[s], ph, abort, WAIT_NS);
-                    if (!in) {
-                        ok = false;
-                        break;
-                    }
-                    st_release_cta(ready, ++gin);
-                    w_done = gin;
-                    if (++s == S) {
-                        s = 0;
-                        ph ^= 1u;
-                    }
+                const Strip s = strip_at(u);
+                u += s.rb - s.ra;
+                const int rows = s.rb - s.ra + 4;
+                for (int t = 0; t < rows && ok; ++t, ++n) {
+                    await(full, n, XST);
+                    await(pfull, n, XST);
+                    if (n > 0) await(free1, n - 1, NRING);
+                    if (ok) issue(xring + (size_t)(n % XST) * ROWB, wsm, 0u, n, done1);
+                    if (ok && m < kept) conv2();
+                    if (t >= 2) ++kept;  // the strip's first two completed rows are dropped
                 }
-                gout += ob - oa;
+            }
+            while (ok && m < kept) conv2();
+            if (!ok && lane == 0) fail();
+            umma2_commit_warp(el, drain);  // after everything issued, also by an early exit
+        }
+    } else if (warp == 19) {
+        if (!lead && lane == 0) {
+            // ---------------- CTA 1: reports its weights and landed x rows to the issuer
+            bool ok = mbar_wait_bounded(wbar, 0, abort, WAIT_NS);
+            int n = 0;
+            for (int64_t u = u_begin; u < u_end && ok;) {
+                const Strip s = strip_at(u);
+                u += s.rb - s.ra;
+                for (int t = 0; t < s.rb - s.ra + 4 && ok; ++t, ++n) {
+                    ok = mbar_wait_bounded(&full[n % XST], (uint32_t)((n / XST) & 1), abort, WAIT_NS);
+                    if (ok) mbar_arrive_cluster(lead_bar(&pfull[n % XST]));
+                }
             }
             if (!ok) fail();
         }
-    } else if (first) {
-        // ---------------- rank 0 epilogue: two groups of 4 warps (2-5, 6-9) on alternate h
-        // rows; warp w reads TMEM lane quadrant w % 4 (pixel m), all 64 columns, stages the
-        // pixel's 128-byte line, and the group leader copies the row into rank 1's h slot
-        const int q = warp & 3;
-        const int g = (warp - 2) >> 2;
-        const int m = q * 32 + lane;
-        const bool leader = warp == 2 + 4 * g && lane == 0;
-        const int bar_id = 1 + g;
-        const uint32_t h_remote = mapa_shared(smem_u32(region), 1u);
-        const uint32_t hfull_remote = mapa_shared(smem_u32(hfull), 1u);
-        const uint32_t issued_remote = mapa_shared(smem_u32(h_issued), 1u);
-        // h row j has been read by rank 1's MMAs (its commit onto hempty)
-        auto consumed = [&](int j) {
-            return j < 0 || mbar_wait_bounded(&hempty[j % HS], (uint32_t)((j / HS) & 1), abort, WAIT_NS);
-        };
-        int gout = 0;
-        bool ok = true;
-        for (int64_t u = u_begin; u < u_end && ok;) {
-            int pi, img, col, ra, rb;
-            strip_at(u, pi, img, col, ra, rb);
-            u += rb - ra;
-            const int oa = ra - 1, ob = rb + 1;
-            const int px = col * BT - 1 + m;
-            const bool colok = px >= 0 && px < width_of(pi);
-            const int Hs = height_of(pi);
-            int o = oa + ((g - (gout & 1)) & 1);
-            for (; o < ob; o += 2) {
-                const int i = gout + (o - oa);
-                const int slot = i & (NSLOT - 1), hs = i % HS;
-                uint8_t *tile = stg + (size_t)(g * 2 + ((i >> 1) & 1)) * TILEB;
-                bool w = mbar_wait_bounded(&rowdone[slot], (uint32_t)((i >> 3) & 1), abort, WAIT_NS);
-                w = __all_sync(0xffffffffu, w);
-                float v[64];
-                if (w) {
-                    tc_fence_after();
-                    uint32_t rr[4][16];
-                    const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(slot * 64);
-#pragma unroll
-                    for (int jj = 0; jj < 4; ++jj) tmem_ld16_nowait(taddr + (uint32_t)(jj * 16), rr[jj]);
-                    tmem_wait_ld();
-#pragma unroll
-                    for (int jj = 0; jj < 4; ++jj)
-#pragma unroll
-                        for (int e = 0; e < 16; ++e) v[jj * 16 + e] = __uint_as_float(rr[jj][e]);
-                    tc_fence_before();
-                    mbar_arrive(&slotfree[slot]);
-                } else {
-#pragma unroll
-                    for (int e = 0; e < 64; ++e) v[e] = 0.f;
-                    if (lane == 0) {
+    } else if (warp == 18) {
+        if (lane == 0) {
+            // ---------------- residual tiles in, output tiles out: kept row k uses tile k % 2, whose
+            // residual is loaded once the store of row k - 2 has read it
+            int64_t ru = u_begin;
+            Strip rs = {0, 0, 0, 0, 0};
+            int ro = 0, loads = 0;
+            auto load_res = [&]() {
+                if (ro >= rs.rb) {
+                    if (ru >= u_end) return;
+                    rs = strip_at(ru);
+                    ru += rs.rb - rs.ra;
+                    ro = rs.ra;
+                }
+                const int k = loads % NTILE;
+                mbar_arrive_expect_tx(&resfull[k], TILEB);
+                tma_load_4d(tiles + (size_t)k * TILEB, rmap_of(rs.pi), &resfull[k], 0, rs.col * BT, ro, rs.img);
+                ++ro;
+                ++loads;
+            };
+            for (int k = 0; k < NTILE; ++k) load_res();
+            bool ok = true;
+            int yrow = 0;
+            for (int64_t u = u_begin; u < u_end && ok;) {
+                const Strip s = strip_at(u);
+                u += s.rb - s.ra;
+                const int Hs = height_of(s.pi);
+                for (int o = s.ra; o < s.rb; ++o, ++yrow) {
+                    const int k = yrow % NTILE;
+                    if (!mbar_wait_bounded(&outfull[k], (uint32_t)((yrow / NTILE) & 1), abort, WAIT_NS)) {
                         fail();
-                        grp_stop[g] = 1;
+                        ok = false;
+                        break;
                     }
-                }
-                // bias and LeakyReLU(0.1) in packed f32x2 arithmetic (the single-layer kernel's)
-#pragma unroll
-                for (int e = 0; e < 64; e += 4) {
-                    const float4 b = *reinterpret_cast<const float4 *>(sbias + e);
-                    add_f32x2(v[e], v[e + 1], b.x, b.y);
-                    add_f32x2(v[e + 2], v[e + 3], b.z, b.w);
-                }
-#pragma unroll
-                for (int e = 0; e < 64; e += 2) {
-                    float t0 = v[e], t1 = v[e + 1];
-                    mul_f32x2(t0, t1, 0.1f, 0.1f);
-                    v[e] = fmaxf(v[e], t0);
-                    v[e + 1] = fmaxf(v[e + 1], t1);
-                }
-                const bool keep = colok && o >= 0 && o < Hs;  // else conv2's zero padding
-                // the h slot's previous row (i - HS) and the staging tile's (i - 4) have been read
-                bool wf = consumed(i - HS) && consumed(i - 4);
-                wf = __all_sync(0xffffffffu, wf);
-                if (!wf && lane == 0) {
-                    fail();
-                    grp_stop[g] = 1;
-                }
-                if (w && wf) {
-                    uint8_t *line = tile + m * 128;
-#pragma unroll
-                    for (int uu = 0; uu < 8; ++uu) {
-                        const int unit = uu ^ (m & 7);
-                        uint4 ov = make_uint4(0u, 0u, 0u, 0u);
-                        if (keep) {
-                            ov.x = pack2<TO>(v[uu * 8 + 0], v[uu * 8 + 1]);
-                            ov.y = pack2<TO>(v[uu * 8 + 2], v[uu * 8 + 3]);
-                            ov.z = pack2<TO>(v[uu * 8 + 4], v[uu * 8 + 5]);
-                            ov.w = pack2<TO>(v[uu * 8 + 6], v[uu * 8 + 7]);
-                        }
-                        *reinterpret_cast<uint4 *>(line + unit * 16) = ov;
+                    if (o < Hs) {
+                        tma_store_4d(ymap_of(s.pi), tiles + (size_t)k * TILEB, 0, s.col * BT, o, s.img);
+                        bulk_commit_group();
+                        bulk_wait_group_read<0>();  // the store has read the tile
                     }
-                    fence_proxy_async();  // the staged row, before the copy reads it
-                }
-                if (leader && *abort) grp_stop[g] = 1;
-                named_barrier(bar_id, 128);
-                if (grp_stop[g]) {
-                    ok = false;
-                    break;
-                }
-                if (leader) {
-                    bulk_copy_to_cluster(h_remote + (uint32_t)hs * ROWB, tile, TILEB, hfull_remote + (uint32_t)hs * 8u);
-                    red_add_cluster(issued_remote, 1u);
+                    load_res();
                 }
             }
-            gout += ob - oa;
+            bulk_wait_group<0>();
+            // residual loads still in flight after an early exit land before the CTA ends
+            for (int k = max(0, loads - NTILE); k < loads; ++k)
+                mbar_wait_bounded(&resfull[k % NTILE], (uint32_t)((k / NTILE) & 1), nullptr, WAIT_NS);
         }
     } else {
-        // ---------------- rank 1 epilogue: bias + residual, staged 128-byte swizzled and
-        // written by one TMA store per row (126 pixels); the residual arrives by TMA, issued
-        // two rows ahead
+        // ---------------- epilogues: warp w reads TMEM lane quadrant w % 4 (pixel m) and one half of
+        // the channels; group 0 (warps 2-9) drains conv1's rows into the h row, group 1 (warps
+        // 10-17) conv2's into the output tiles.  (Four warps per group, each with all 64 columns,
+        // took 4700 cycles per row step: 1600 to drain and zero, 1400 to compute, 1300 to hand over.)
+        const int g = warp < 10 ? 0 : 1;
+        const int half = ((warp - 2) >> 2) & 1;
         const int q = warp & 3;
-        const int g = (warp - 2) >> 2;
         const int m = q * 32 + lane;
-        const bool leader = warp == 2 + 4 * g && lane == 0;
-        const int bar_id = 1 + g;
-        uint8_t *ot = obuf + g * TILEB + m * 128;
-        const uint8_t *rt = rbuf + g * TILEB + m * 128;
-        int gout = 0;
-        int res_loads = 0, last_res = -1;
-        bool ok = true;
-        for (int64_t u = u_begin; u < u_end && ok;) {
-            int pi, img, col, ra, rb;
-            strip_at(u, pi, img, col, ra, rb);
-            u += rb - ra;
-            const int x0 = col * BT;
-            int o = ra + ((g - (gout & 1)) & 1);
-            if (leader && o < rb) {
-                mbar_arrive_expect_tx(&resfull[g], TILEB);
-                tma_load_4d(rbuf + g * TILEB, rmap_of(pi), &resfull[g], 0, x0, o, img);
-                last_res = res_loads++;
+        const uint32_t lanes = tmem_base + ((uint32_t)(q * 32) << 16) + (g ? WIN2 : 0u) + 96u * (uint32_t)half;
+        uint64_t *done = g ? done2 : done1;
+        const uint32_t freed = lead_bar(g ? free2 : free1);
+        const float *sb = sbias + 64 * g + 32 * half;
+        bool w = true;
+        float v[32];
+        auto await = [&](uint64_t *bar, uint32_t parity) {
+            w = __all_sync(0xffffffffu, mbar_wait_bounded(bar, parity, abort, WAIT_NS));
+            if (!w && lane == 0) fail();
+            return w;
+        };
+        // waits for input row i's MMAs, takes the accumulator row they completed (slot (i - 1) % 3)
+        // into v, zeroes it and adds the bias, in packed f32x2 arithmetic (the single-layer kernel's)
+        auto drain_row = [&](int i, bool keep) {
+            if (!await(&done[i % NRING], (uint32_t)((i / NRING) & 1))) return false;
+            tc_fence_after();
+            const uint32_t t = lanes + 32u * (uint32_t)((i + 2) % 3);
+            if (keep) {
+                uint32_t r[32];
+                tmem_ld32_nowait(t, r);
+                tmem_wait_ld();
+#pragma unroll
+                for (int e = 0; e < 32; ++e) v[e] = __uint_as_float(r[e]);
             }
-            for (; o < rb; o += 2) {
-                const int i = gout + (o - ra);
-                const int slot = i & (NSLOT - 1);
-                const int k = i >> 1;  // this group's row count: the phase of its residual barrier
-                if (leader) bulk_wait_group_read<0>();  // the group's previous store has read its tile
-                named_barrier(bar_id, 128);
-                bool w = mbar_wait_bounded(&rowdone[slot], (uint32_t)((i >> 3) & 1), abort, WAIT_NS);
-                w = __all_sync(0xffffffffu, w);
-                float v[64];
-                if (w) {
-                    tc_fence_after();
-                    uint32_t rr[4][16];
-                    const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(slot * 64);
+            tmem_zero32(t);
+            tmem_wait_st();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(freed + (uint32_t)(i % NRING) * 8u);
+            if (keep) {
 #pragma unroll
-                    for (int jj = 0; jj < 4; ++jj) tmem_ld16_nowait(taddr + (uint32_t)(jj * 16), rr[jj]);
-                    tmem_wait_ld();
-#pragma unroll
-                    for (int jj = 0; jj < 4; ++jj)
-#pragma unroll
-                        for (int e = 0; e < 16; ++e) v[jj * 16 + e] = __uint_as_float(rr[jj][e]);
-                    tc_fence_before();
-                    mbar_arrive(&slotfree[slot]);
-                } else {
-#pragma unroll
-                    for (int e = 0; e < 64; ++e) v[e] = 0.f;
-                    if (lane == 0) {
-                        fail();
-                        grp_stop[g] = 1;
-                    }
-                }
-#pragma unroll
-                for (int e = 0; e < 64; e += 4) {
-                    const float4 b = *reinterpret_cast<const float4 *>(sbias + e);
+                for (int e = 0; e < 32; e += 4) {
+                    const float4 b = *reinterpret_cast<const float4 *>(sb + e);
                     add_f32x2(v[e], v[e + 1], b.x, b.y);
                     add_f32x2(v[e + 2], v[e + 3], b.z, b.w);
                 }
-                bool rw = mbar_wait_bounded(&resfull[g], (uint32_t)(k & 1), abort, WAIT_NS);
-                rw = __all_sync(0xffffffffu, rw);
-                if (!rw && lane == 0) {
-                    fail();
-                    grp_stop[g] = 1;
-                }
+            }
+            return true;
+        };
+        // 16-byte unit uu of this half's 64 bytes of a 128-byte-swizzled line
+        auto unit_at = [&](uint8_t *row, int uu) {
+            return reinterpret_cast<uint4 *>(row + m * 128 + (((half * 4 + uu) ^ (m & 7)) * 16));
+        };
+        auto pack_unit = [&](int uu) {
+            uint4 ov;
+            ov.x = pack2<TO>(v[uu * 8 + 0], v[uu * 8 + 1]);
+            ov.y = pack2<TO>(v[uu * 8 + 2], v[uu * 8 + 3]);
+            ov.z = pack2<TO>(v[uu * 8 + 4], v[uu * 8 + 5]);
+            ov.w = pack2<TO>(v[uu * 8 + 6], v[uu * 8 + 7]);
+            return ov;
+        };
+        int i = 0;  // input rows of this group's conv
+        if (g == 0) {
+            const uint32_t hfull_lead = lead_bar(hfull);
+            int hrow = 0;  // h rows written
+            for (int64_t u = u_begin; u < u_end && w;) {
+                const Strip s = strip_at(u);
+                u += s.rb - s.ra;
+                const int px = s.col * BT - 1 + m;
+                const bool colok = px >= 0 && px < width_of(s.pi);
+                const int Hs = height_of(s.pi);
+                for (int t = 0; t < s.rb - s.ra + 4; ++t, ++i) {
+                    const bool keep = t >= 2;
+                    if (!drain_row(i, keep)) break;
+                    if (!keep) continue;
 #pragma unroll
-                for (int uu = 0; uu < 8; ++uu) {
-                    const int unit = uu ^ (m & 7);
-                    const uint4 raw = *reinterpret_cast<const uint4 *>(rt + unit * 16);
-                    const uint32_t wd[4] = {raw.x, raw.y, raw.z, raw.w};
-#pragma unroll
-                    for (int h = 0; h < 4; ++h) {
-                        float r0, r1;
-                        unpack2<TO>(wd[h], r0, r1);
-                        add_f32x2(v[uu * 8 + 2 * h], v[uu * 8 + 2 * h + 1], r0, r1);
+                    for (int e = 0; e < 32; e += 2) {
+                        float t0 = v[e], t1 = v[e + 1];
+                        mul_f32x2(t0, t1, 0.1f, 0.1f);
+                        v[e] = fmaxf(v[e], t0);
+                        v[e + 1] = fmaxf(v[e + 1], t1);
                     }
-                }
+                    const int o = s.ra - 1 + t - 2;
+                    const bool inside = colok && o >= 0 && o < Hs;  // else conv2's zero padding
+                    uint4 ov[4];
 #pragma unroll
-                for (int uu = 0; uu < 8; ++uu) {
-                    const int unit = uu ^ (m & 7);
-                    uint4 ov;
-                    ov.x = pack2<TO>(v[uu * 8 + 0], v[uu * 8 + 1]);
-                    ov.y = pack2<TO>(v[uu * 8 + 2], v[uu * 8 + 3]);
-                    ov.z = pack2<TO>(v[uu * 8 + 4], v[uu * 8 + 5]);
-                    ov.w = pack2<TO>(v[uu * 8 + 6], v[uu * 8 + 7]);
-                    *reinterpret_cast<uint4 *>(ot + unit * 16) = ov;
-                }
-                fence_proxy_async();  // staging writes (and residual reads) before the async proxy
-                if (leader && *abort) grp_stop[g] = 1;
-                named_barrier(bar_id, 128);
-                if (grp_stop[g]) {
-                    ok = false;
-                    break;
-                }
-                if (leader) {
-                    tma_store_4d(ymap_of(pi), obuf + g * TILEB, 0, x0, o, img);
-                    bulk_commit_group();
-                    if (o + 2 < rb) {  // this group's next row; the tile's readers are done
-                        mbar_arrive_expect_tx(&resfull[g], TILEB);
-                        tma_load_4d(rbuf + g * TILEB, rmap_of(pi), &resfull[g], 0, x0, o + 2, img);
-                        last_res = res_loads++;
+                    for (int uu = 0; uu < 4; ++uu) {
+                        ov[uu] = pack_unit(uu);
+                        if (!inside) ov[uu] = make_uint4(0u, 0u, 0u, 0u);
                     }
+                    // the previous h row has been read by conv2's MMAs
+                    const int k = hrow - 1;
+                    if (k >= 0 && !await(&done2[k % NRING], (uint32_t)((k / NRING) & 1))) break;
+#pragma unroll
+                    for (int uu = 0; uu < 4; ++uu) *unit_at(hrow_sm, uu) = ov[uu];
+                    fence_proxy_async();  // the row, before the MMAs read it
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive_cluster(hfull_lead);
+                    ++hrow;
                 }
             }
-            gout += rb - ra;
-        }
-        if (leader) {
-            bulk_wait_group<0>();
-            // a residual load still in flight after an early exit lands before the CTA ends
-            if (last_res >= 0) mbar_wait_bounded(&resfull[g], (uint32_t)(last_res & 1), nullptr, WAIT_NS);
+        } else {
+            int yrow = 0;  // y rows finished
+            for (int64_t u = u_begin; u < u_end && w;) {
+                const Strip s = strip_at(u);
+                u += s.rb - s.ra;
+                for (int t = 0; t < s.rb - s.ra + 2; ++t, ++i) {
+                    const bool keep = t >= 2;
+                    if (!drain_row(i, keep)) break;
+                    if (!keep) continue;
+                    const int k = yrow % NTILE;
+                    if (!await(&resfull[k], (uint32_t)((yrow / NTILE) & 1))) break;
+                    uint8_t *tile = tiles + (size_t)k * TILEB;
+#pragma unroll
+                    for (int uu = 0; uu < 4; ++uu) {
+                        uint4 *at = unit_at(tile, uu);
+                        const uint4 raw = *at;
+                        const uint32_t wd[4] = {raw.x, raw.y, raw.z, raw.w};
+#pragma unroll
+                        for (int h = 0; h < 4; ++h) {
+                            float r0, r1;
+                            unpack2<TO>(wd[h], r0, r1);
+                            add_f32x2(v[uu * 8 + 2 * h], v[uu * 8 + 2 * h + 1], r0, r1);
+                        }
+                        *at = pack_unit(uu);
+                    }
+                    fence_proxy_async();  // the tile's writes before the async proxy
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&outfull[k]);
+                    ++yrow;
+                }
+            }
         }
     }
-    if (!first && warp == 1 && lane == 0) st_cluster_u32(mapa_shared(smem_u32(h_consumed), 0u), (uint32_t)i_rows);
     __syncthreads();
-    cluster_sync_all();  // every copy and MMA commit towards either CTA has been issued; the counts are final
-    if (!first && warp == 10 && lane == 0) {
-        // h copies rank 0 started that this CTA has not waited for (after an early exit) land first
-        const int issued = *h_issued;
-        for (int j = w_done; j < issued; ++j) {
-            const int s = j % HS;
-            if (j >= w_armed) mbar_arrive_expect_tx(&hfull[s], TILEB);
-            mbar_wait_bounded(&hfull[s], (uint32_t)((j / HS) & 1), nullptr, WAIT_NS);
-        }
-    }
-    if (first && warp == 2 && lane == 0) {
-        // rank 1's MMA commits onto this CTA's barriers have landed (the last one of each slot)
-        const int n = *h_consumed;
-        for (int j = max(0, n - HS); j < n; ++j)
-            mbar_wait_bounded(&hempty[j % HS], (uint32_t)((j / HS) & 1), nullptr, WAIT_NS);
-    }
+    cluster_sync_all();  // every arrival and MMA commit towards either CTA has been issued
+    if (warp == 1 && lane == 0) mbar_wait_bounded(drain, 0, nullptr, WAIT_NS);
+    __syncthreads();
     cluster_sync_all();  // neither CTA leaves while the other may still write into its shared memory
     if (warp == 1) {
         __syncwarp();
         tc_fence_after();
-        tmem_dealloc(tmem_base, 512);
+        tmem_dealloc2(tmem_base, 512);
     }
 }
 
@@ -655,7 +544,7 @@ int max_pairs() {
     return n;
 }
 
-// units: output rows x column tiles of the launch (each cluster gets an equal range)
+// units: the launch's pair rows (each cluster gets an equal range)
 template <int DT, bool MULTI>
 cudaError_t run_block(const CUtensorMap &xmap, const CUtensorMap &rmap, const CUtensorMap &ymap,
                       const BlockParams &p, const BlockProblem *probs, int nprob, int64_t units, cudaStream_t st) {
@@ -663,8 +552,9 @@ cudaError_t run_block(const CUtensorMap &xmap, const CUtensorMap &rmap, const CU
     if (e != cudaSuccess) return e;
     int npairs = max_pairs<DT, MULTI>();
     if (npairs < 1) return cudaErrorInvalidConfiguration;
-    // at least ~16 output rows per cluster: each strip costs conv1 two extra rows
-    npairs = (int)std::max<int64_t>(1, std::min<int64_t>(npairs, units / 16));
+    // a strip costs its cluster about five more row steps, but while clusters are idle a shorter
+    // strip still ends sooner
+    npairs = (int)std::max<int64_t>(1, std::min<int64_t>(npairs, units / 4));
     cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = 2;
@@ -739,7 +629,7 @@ cudaError_t launch_res_block(const ConvArgs &c1, const ConvArgs &c2, cudaStream_
     cudaError_t e = encode_block_maps(c1, c2, &xmap, &rmap, &ymap);
     if (e != cudaSuccess) return e;
     const BlockParams p = block_params(c1, c2);
-    const int64_t units = (int64_t)p.nimg * p.ncols * p.H;
+    const int64_t units = p.nimg * block_units(p.H, p.ncols);
     return c1.in_dt == DT_BF16 ? run_block<DT_BF16, false>(xmap, rmap, ymap, p, nullptr, 0, units, st)
                                : run_block<DT_F16, false>(xmap, rmap, ymap, p, nullptr, 0, units, st);
 }
@@ -764,7 +654,7 @@ cudaError_t launch_res_block_multi(const ConvArgs *c1, const ConvArgs *c2, int n
         q.ncols = (c1[i].W + BT - 1) / BT;
         q.pad_ = 0;
         q.u0 = units;
-        units += (int64_t)q.ncols * q.H;
+        units += block_units(q.H, q.ncols);
     }
     if (copy_table) {
         cudaError_t e = cudaMemcpyAsync(dev_tab, host_tab, sizeof(BlockProblem) * n, cudaMemcpyHostToDevice, st);
