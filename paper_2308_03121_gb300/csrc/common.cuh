@@ -9,6 +9,7 @@
 #include <cuda_fp8.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <string>
 #include <utility>
 
@@ -232,6 +233,24 @@ void prepare_weights_rows_ps4(const float *w_oihw, int dt, void *dst_host);
 // [kx][16-byte chunk][2 - ky][64 out][16 channels], no swizzle.
 size_t tc_rows_f8_weight_bytes();
 void prepare_weights_rows_f8(const float *w_oihw, float scale, void *dst_host);
+
+// Weights given as OIHW float32 on the device, laid out by one launch (csrc/weights.cu): the image
+// of the SIMT kernel, of the generic tensor-core kernel (slices of ns outputs; 16-byte K chunks,
+// or 64-channel 128-byte-swizzled ones) or of the row-streaming 64 -> 64 3x3 kernel, as the
+// host-side layouts above give them, and the bias padded with zeros to nbias values.
+enum WeightLayout : int { WL_SIMT = 0, WL_TC16 = 1, WL_TC128 = 2, WL_ROWS = 3 };
+struct WeightArgs {
+    const float *w, *bias;   // bias may be null (zero)
+    int cout, cin, k, cin_pad, cout_pad;
+    int layout, dt, ns;
+    float scale;             // multiplies every weight (FP8 quantisation), 1 otherwise
+    void *dst;
+    float *dst_bias;
+    int nbias;
+};
+cudaError_t launch_weights(const WeightArgs &a, cudaStream_t st);
+// max |v| of n device values, as float bits, by atomicMax into *out.
+cudaError_t launch_absmax(const float *v, int64_t n, unsigned *out, cudaStream_t st);
 
 // DCN: x blocked (activation dtype); offsets and mask in one blocked float32
 // tensor [om_cpad/4][H][W][4].  Channel order: torchvision's ([0, 18G) = (dy, dx)

@@ -44,58 +44,6 @@ struct AreaRec {
 std::mutex g_area_mu;
 std::vector<AreaRec> g_area;
 
-// SIMT image [cin_pad][k*k][cout_pad] float32, written whole (padding = 0).
-__global__ void simt_weights_kernel(const float *__restrict__ w, int cout, int cin, int kk, int cin_pad,
-                                    int cout_pad, float *__restrict__ dst) {
-    const int64_t n = (int64_t)cin_pad * kk * cout_pad;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int o = (int)(i % cout_pad);
-        const int64_t ct = i / cout_pad;
-        const int t = (int)(ct % kk), c = (int)(ct / kk);
-        dst[i] = (o < cout && c < cin) ? w[((int64_t)o * cin + c) * kk + t] : 0.f;
-    }
-}
-
-template <typename T>
-__device__ __forceinline__ T to_elem(float v);
-template <>
-__device__ __forceinline__ __nv_bfloat16 to_elem<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
-template <>
-__device__ __forceinline__ __half to_elem<__half>(float v) { return __float2half_rn(v); }
-
-// Tensor-core image per output slice of ns channels: [slice][tap][K chunk][n][chunk bytes],
-// with the 16-byte units of row n rotated by n & 7 in the 128-byte-swizzled form.
-// One thread per weight element; the destination was zeroed beforehand.
-template <typename T>
-__global__ void tc_weights_kernel(const float *__restrict__ w, int cout, int cin, int kk, int cin_pad, int ns,
-                                  int cpc, int sw128, uint8_t *__restrict__ dst) {
-    constexpr int esz = (int)sizeof(T);
-    const int cb = cpc * esz, chunks = cin_pad / cpc;
-    const int64_t n_el = (int64_t)cout * cin * kk;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_el;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int t = (int)(i % kk);
-        const int c = (int)((i / kk) % cin);
-        const int o = (int)(i / ((int64_t)kk * cin));
-        const int sl = o / ns, n = o % ns, kc = c / cpc, e = c % cpc;
-        int64_t off = (int64_t)sl * kk * chunks * ns * cb + (((int64_t)t * chunks + kc) * ns + n) * cb;
-        off += sw128 ? (int64_t)((((e * esz) >> 4) ^ (n & 7)) << 4) + (e * esz) % 16 : (int64_t)e * esz;
-        *reinterpret_cast<T *>(dst + off) = to_elem<T>(w[i]);
-    }
-}
-
-// Row-streaming 64 -> 64 image [kx][2 - ky][64 out][128 B swizzled 64 in]; one
-// thread per weight element, every destination byte written.
-template <typename T>
-__global__ void rows_weights_kernel(const float *__restrict__ w, uint8_t *__restrict__ dst) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= 64 * 64 * 9) return;
-    const int kx = i % 3, ky = (i / 3) % 3, c = (i / 9) % 64, n = i / 576;
-    const int64_t row = (int64_t)(2 - ky) * 64 + n;
-    const int64_t off = (int64_t)kx * 3 * 64 * 128 + row * 128 + (((c >> 3) ^ (n & 7)) << 4) + (c & 7) * 2;
-    *reinterpret_cast<T *>(dst + off) = to_elem<T>(w[i]);
-}
-
 // Bump allocator over the fixed area: 256-byte aligned slices, sizes checked
 // in 64-bit arithmetic before any device work.
 struct Carve {
@@ -157,11 +105,6 @@ nvisr_status area_for_current_device(uint8_t **out) {
     return NVISR_OK;
 }
 
-int grid_for(int64_t n, int threads) {
-    const int64_t blocks = (n + threads - 1) / threads;
-    return (int)std::min<int64_t>(std::max<int64_t>(blocks, 1), (int64_t)device_sm_count() * 16);
-}
-
 }  // namespace
 }  // namespace nvisr
 
@@ -191,6 +134,7 @@ extern "C" nvisr_status nvisr_conv2d_static(int32_t precision, const float *x, i
     Carve cv;
     const uint64_t o_err = cv.take(sizeof(int));
     const uint64_t o_bias = cv.take((uint64_t)cout_pad * 4);
+    // (the row kernel's image alone is written for its layers; room for both keeps the documented need)
     const uint64_t o_w = cv.take(wbytes);
     const uint64_t o_rows = rows ? cv.take(tc_rows_weight_bytes()) : 0;
     const uint64_t o_x = cv.take((uint64_t)cin_pad * px * esz);
@@ -206,41 +150,17 @@ extern "C" nvisr_status nvisr_conv2d_static(int32_t precision, const float *x, i
     cudaStream_t st = (cudaStream_t)stream;
     int *err = reinterpret_cast<int *>(area + o_err);
     float *db = reinterpret_cast<float *>(area + o_bias);
-    uint8_t *dw = area + o_w, *dwr = rows ? area + o_rows : nullptr;
     void *dx = area + o_x, *dy = area + o_y, *dr = res ? (void *)(area + o_r) : nullptr;
-
-    // what must start at zero: the error word, the bias padding, the weight image padding
     CS_TRY(cudaMemsetAsync(err, 0, sizeof(int), st));
-    CS_TRY(cudaMemsetAsync(db, 0, (size_t)cout_pad * 4, st));
-    if (bias) CS_TRY(cudaMemcpyAsync(db, bias, (size_t)cout * 4, cudaMemcpyDeviceToDevice, st));
-    const int kk = k * k;
-    if (tc) {
-        CS_TRY(cudaMemsetAsync(dw, 0, wbytes, st));
-        const int ns = cout_pad / tc_nslice(cin_pad, cout_pad, k, dt);
-        const int sw128 = layout_cpc(dt, cin_pad) == 64;
-        const int cpc = sw128 ? 64 : 16 / esz;
-        const int64_t n_el = (int64_t)cout * cin * kk;
-        if (dt == DT_BF16)
-            tc_weights_kernel<__nv_bfloat16><<<grid_for(n_el, 256), 256, 0, st>>>(weight, cout, cin, kk, cin_pad, ns,
-                                                                                  cpc, sw128, dw);
-        else
-            tc_weights_kernel<__half><<<grid_for(n_el, 256), 256, 0, st>>>(weight, cout, cin, kk, cin_pad, ns, cpc,
-                                                                           sw128, dw);
-        CS_TRY(cudaGetLastError());
-        if (rows) {
-            CS_TRY(cudaMemsetAsync(dwr, 0, tc_rows_weight_bytes(), st));
-            if (dt == DT_BF16) rows_weights_kernel<__nv_bfloat16><<<(64 * 64 * 9 + 255) / 256, 256, 0, st>>>(weight, dwr);
-            else rows_weights_kernel<__half><<<(64 * 64 * 9 + 255) / 256, 256, 0, st>>>(weight, dwr);
-            CS_TRY(cudaGetLastError());
-        }
-    } else {
-        const int64_t n = (int64_t)cin_pad * kk * cout_pad;
-        simt_weights_kernel<<<grid_for(n, 256), 256, 0, st>>>(weight, cout, cin, kk, cin_pad, cout_pad,
-                                                             reinterpret_cast<float *>(dw));
-        CS_TRY(cudaGetLastError());
-    }
-
     const int in_cpc = layout_cpc(dt, cin_pad), out_cpc = layout_cpc(dt, cout_pad);
+    WeightArgs wa{};
+    wa.w = weight; wa.bias = bias; wa.cout = cout; wa.cin = cin; wa.k = k; wa.cin_pad = cin_pad; wa.cout_pad = cout_pad;
+    wa.layout = rows ? WL_ROWS : (!tc ? WL_SIMT : (in_cpc == 64 ? WL_TC128 : WL_TC16));
+    wa.dt = dt;
+    wa.ns = tc ? cout_pad / tc_nslice(cin_pad, cout_pad, k, dt) : 0;
+    wa.scale = 1.f;
+    wa.dst = area + (rows ? o_rows : o_w); wa.dst_bias = db; wa.nbias = cout_pad;
+    CS_TRY(launch_weights(wa, st));
     PackArgs pa{};
     pa.src[0] = x;
     pa.nsrc = 1;
@@ -265,7 +185,9 @@ extern "C" nvisr_status nvisr_conv2d_static(int32_t precision, const float *x, i
         CS_TRY(launch_pack(pr, st));
     }
     ConvArgs a{};
-    a.x = dx; a.cin_pad = cin_pad; a.H = h; a.W = w; a.nimg = 1; a.w = dw; a.w_rows = dwr; a.bias = db;
+    a.x = dx; a.cin_pad = cin_pad; a.H = h; a.W = w; a.nimg = 1; a.bias = db;
+    a.w = rows ? nullptr : wa.dst;
+    a.w_rows = rows ? wa.dst : nullptr;
     a.cout = cout; a.cout_pad = cout_pad; a.k = k; a.act = act; a.res = dr; a.y = dy;
     a.in_dt = dt; a.out_dt = dt; a.acc_scale = 1.f; a.out_scale = 1.f; a.y2_scale = 1.f; a.err = err;
     a.in_cpc = in_cpc; a.out_cpc = out_cpc;

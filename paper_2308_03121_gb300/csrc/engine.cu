@@ -20,6 +20,7 @@
 
 #include "common.cuh"
 #include "netdesc.h"
+#include "scratch.h"
 
 namespace nvisr {
 
@@ -115,6 +116,11 @@ nvisr_status dalloc(nvisr_engine *e, size_t bytes, std::vector<DevBuf> &owned, v
                                            std::to_string(e->budget - e->used) + " left");
     void *p = nullptr;
     cudaError_t ce = cudaMalloc(&p, bytes);
+    if (ce == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        scratch_trim();  // the per-call entry points' kept working memory
+        ce = cudaMalloc(&p, bytes);
+    }
     if (ce != cudaSuccess) {
         cudaGetLastError();
         return fail(NVISR_OUT_OF_MEMORY, std::string("cudaMalloc: ") + cudaGetErrorString(ce));
@@ -2802,48 +2808,6 @@ nvisr_status nvisr_fig1_layout(int32_t n, int32_t b, int32_t *cell_frame, int32_
 
 namespace {
 
-struct Scratch {
-    std::vector<void *> ptrs;
-    ~Scratch() {
-        for (void *p : ptrs) cudaFree(p);
-    }
-    cudaError_t alloc(size_t bytes, void **out) {
-        cudaError_t e = cudaMalloc(out, std::max<size_t>(bytes, 256));
-        if (e == cudaSuccess) ptrs.push_back(*out);
-        return e;
-    }
-};
-
-// Quantisation scale (amax / 448) of a planar tensor, measured on the device.
-nvisr_status fp8_scale(const float *x, int C, int H, int W, Scratch &sc, cudaStream_t st, float *scale) {
-    void *tmp, *am;
-    const int cpad = round_up(C, 8);
-    NVISR_TRY_CUDA(sc.alloc((size_t)cpad * H * W * 2, &tmp));
-    NVISR_TRY_CUDA(sc.alloc(sizeof(unsigned), &am));
-    NVISR_TRY_CUDA(cudaMemsetAsync(am, 0, sizeof(unsigned), st));
-    PackArgs pa{};
-    pa.src[0] = x;
-    pa.nsrc = 1;
-    pa.ch_per_src = C;
-    pa.src_pitch = W;
-    pa.src_plane = (int64_t)W * H;
-    pa.H = H;
-    pa.W = W;
-    pa.dst = tmp;
-    pa.cpad = cpad;
-    pa.dt = DT_BF16;
-    pa.scale = 1.f;
-    pa.amax = (unsigned *)am;
-    NVISR_TRY_CUDA(launch_pack(pa, st));
-    unsigned h;
-    NVISR_TRY_CUDA(cudaMemcpyAsync(&h, am, 4, cudaMemcpyDeviceToHost, st));
-    NVISR_TRY_CUDA(cudaStreamSynchronize(st));
-    float a;
-    memcpy(&a, &h, 4);
-    *scale = a > 0.f ? a / 448.f : 1.f;
-    return NVISR_OK;
-}
-
 nvisr_status pack_planar(const float *x, int C, int cpad, int H, int W, int dt, float scale, void *dst,
                          cudaStream_t st, int cpc = 0) {
     PackArgs pa{};
@@ -2879,71 +2843,56 @@ nvisr_status nvisr_conv2d(int32_t precision, const float *x, int32_t cin, int32_
     const int idt = precision == NVISR_PREC_FP8 ? DT_E4M3 : adt;
     if (precision == NVISR_PREC_FP8 && (cin % 64 || cout != 64 || k != 3))
         return fail(NVISR_UNSUPPORTED_FORMAT, "conv2d: FP8 supports 64->64 3x3 layers");
-    const int cin_pad = tc ? round_up(cin, idt == DT_E4M3 ? 16 : 16) : round_up(cin, 8);
-    const int cout_pad = round_up(cout, 16);
-    Scratch sc;
-    // weights (host copy -> layout -> device)
-    std::vector<float> hw((size_t)cout * cin * k * k), hb(cout_pad, 0.f);
-    NVISR_TRY_CUDA(cudaMemcpyAsync(hw.data(), weight, hw.size() * 4, cudaMemcpyDeviceToHost, st));
-    if (bias) NVISR_TRY_CUDA(cudaMemcpyAsync(hb.data(), bias, (size_t)cout * 4, cudaMemcpyDeviceToHost, st));
-    NVISR_TRY_CUDA(cudaStreamSynchronize(st));
+    const int cin_pad = round_up(cin, tc ? 16 : 8), cout_pad = round_up(cout, 16);
+    const bool rows = tc && idt != DT_E4M3 && k == 3 && cin == 64 && cout == 64;
+    const size_t px = (size_t)h * w;
+    const int in_cpc = layout_cpc(idt, cin_pad), out_cpc = layout_cpc(adt, cout_pad);
+    Scratch sc(st);
+    const size_t o_w = sc.plan(rows ? tc_rows_weight_bytes()
+                                    : (tc ? tc_weight_bytes(cin_pad, cout_pad, k, idt) : simt_weight_bytes(cin_pad, cout_pad, k)));
+    const size_t o_b = sc.plan((size_t)cout_pad * 4);
+    const size_t o_x = sc.plan((size_t)cin_pad * px * dtype_size(idt));
+    const size_t o_y = sc.plan((size_t)cout_pad * px * dtype_size(adt));
+    const size_t o_r = res ? sc.plan((size_t)cout_pad * px * dtype_size(adt)) : 0;
+    const size_t o_m = sc.plan(2 * sizeof(unsigned));
+    NVISR_TRY_CUDA(sc.open());
     float sx = 1.f, sw = 1.f;
     if (idt == DT_E4M3) {
-        nvisr_status s = fp8_scale(x, cin, h, w, sc, st, &sx);
-        if (s != NVISR_OK) return s;
-        float amax = 0.f;
-        for (float v : hw) amax = std::max(amax, std::fabs(v));
-        sw = amax > 0.f ? amax / 448.f : 1.f;
+        // per-tensor scales (amax / 448) of x and the weights, measured on the device
+        unsigned *am = sc.at<unsigned>(o_m);
+        NVISR_TRY_CUDA(cudaMemsetAsync(am, 0, 2 * sizeof(unsigned), st));
+        NVISR_TRY_CUDA(launch_absmax(x, (int64_t)cin * (int64_t)px, am, st));
+        NVISR_TRY_CUDA(launch_absmax(weight, (int64_t)cout * cin * k * k, am + 1, st));
+        float a[2];
+        NVISR_TRY_CUDA(cudaMemcpyAsync(a, am, sizeof(a), cudaMemcpyDeviceToHost, st));
+        NVISR_TRY_CUDA(cudaStreamSynchronize(st));
+        sx = a[0] > 0.f ? a[0] / 448.f : 1.f;
+        sw = a[1] > 0.f ? a[1] / 448.f : 1.f;
     }
-    void *dw, *db, *dx, *dy, *dr = nullptr;
-    size_t wbytes;
-    std::vector<uint8_t> hwl;
-    if (tc) {
-        wbytes = tc_weight_bytes(cin_pad, cout_pad, k, idt);
-        hwl.resize(wbytes);
-        prepare_weights_tc(hw.data(), cout, cin, k, cin_pad, cout_pad, idt, 1.f / sw, hwl.data(),
-                           layout_cpc(idt, cin_pad) == 64);
-    } else {
-        wbytes = simt_weight_bytes(cin_pad, cout_pad, k);
-        hwl.resize(wbytes);
-        prepare_weights_simt(hw.data(), cout, cin, k, cin_pad, cout_pad, (float *)hwl.data());
-    }
-    NVISR_TRY_CUDA(sc.alloc(wbytes, &dw));
-    NVISR_TRY_CUDA(cudaMemcpyAsync(dw, hwl.data(), wbytes, cudaMemcpyHostToDevice, st));
-    void *dwr = nullptr;
-    std::vector<uint8_t> hrows;
-    if (tc && idt != DT_E4M3 && k == 3 && cin == 64 && cout == 64) {
-        hrows.resize(tc_rows_weight_bytes());
-        prepare_weights_rows(hw.data(), idt, hrows.data());
-        NVISR_TRY_CUDA(sc.alloc(hrows.size(), &dwr));
-        NVISR_TRY_CUDA(cudaMemcpyAsync(dwr, hrows.data(), hrows.size(), cudaMemcpyHostToDevice, st));
-    }
-    NVISR_TRY_CUDA(sc.alloc(cout_pad * 4, &db));
-    NVISR_TRY_CUDA(cudaMemcpyAsync(db, hb.data(), cout_pad * 4, cudaMemcpyHostToDevice, st));
-    NVISR_TRY_CUDA(sc.alloc((size_t)cin_pad * h * w * dtype_size(idt), &dx));
-    NVISR_TRY_CUDA(sc.alloc((size_t)cout_pad * h * w * dtype_size(adt), &dy));
-    const int in_cpc = layout_cpc(idt, cin_pad), out_cpc = layout_cpc(adt, cout_pad);
+    void *dx = sc.at<void>(o_x), *dy = sc.at<void>(o_y), *dr = res ? sc.at<void>(o_r) : nullptr;
+    WeightArgs wa{};
+    wa.w = weight; wa.bias = bias; wa.cout = cout; wa.cin = cin; wa.k = k; wa.cin_pad = cin_pad; wa.cout_pad = cout_pad;
+    wa.layout = rows ? WL_ROWS : (!tc ? WL_SIMT : (in_cpc == 64 ? WL_TC128 : WL_TC16));
+    wa.dt = idt;
+    wa.ns = tc ? cout_pad / tc_nslice(cin_pad, cout_pad, k, idt) : 0;
+    wa.scale = 1.f / sw;
+    wa.dst = sc.at<void>(o_w); wa.dst_bias = sc.at<float>(o_b); wa.nbias = cout_pad;
+    NVISR_TRY_CUDA(launch_weights(wa, st));
     nvisr_status s = pack_planar(x, cin, cin_pad, h, w, idt, 1.f / sx, dx, st, in_cpc);
     if (s != NVISR_OK) return s;
-    if (res) {
-        NVISR_TRY_CUDA(sc.alloc((size_t)cout_pad * h * w * dtype_size(adt), &dr));
-        if ((s = pack_planar(res, cout, cout_pad, h, w, adt, 1.f, dr, st, out_cpc)) != NVISR_OK) return s;
-    }
-    int *err;
-    NVISR_TRY_CUDA(sc.alloc(sizeof(int), (void **)&err));
-    NVISR_TRY_CUDA(cudaMemsetAsync(err, 0, sizeof(int), st));
+    if (res && (s = pack_planar(res, cout, cout_pad, h, w, adt, 1.f, dr, st, out_cpc)) != NVISR_OK) return s;
     ConvArgs a{};
-    a.x = dx; a.cin_pad = cin_pad; a.H = h; a.W = w; a.nimg = 1; a.w = dw; a.w_rows = dwr; a.bias = (const float *)db;
+    a.x = dx; a.cin_pad = cin_pad; a.H = h; a.W = w; a.nimg = 1; a.bias = wa.dst_bias;
+    a.w = rows ? nullptr : wa.dst;
+    a.w_rows = rows ? wa.dst : nullptr;
     a.cout = cout; a.cout_pad = cout_pad; a.k = k; a.act = act; a.res = dr; a.y = dy;
-    a.in_dt = idt; a.out_dt = adt; a.acc_scale = sx * sw; a.out_scale = 1.f; a.y2_scale = 1.f; a.err = err;
+    a.in_dt = idt; a.out_dt = adt; a.acc_scale = sx * sw; a.out_scale = 1.f; a.y2_scale = 1.f; a.err = sc.err();
     a.in_cpc = in_cpc; a.out_cpc = out_cpc;
     cudaError_t e = tc ? launch_conv_tc(a, st) : launch_conv_simt(a, st);
     if (e != cudaSuccess) return cuda_status(e, "conv2d");
     NVISR_TRY_CUDA(launch_unpack(dy, adt, cout_pad, out_cpc, cout, h, w, 1.f, y, w, st));
-    int herr = 0;
-    NVISR_TRY_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, st));
-    NVISR_TRY_CUDA(cudaStreamSynchronize(st));
-    if (herr) return fail(NVISR_DEVICE_TIMEOUT, "conv2d: a device-side wait exceeded its bound");
+    NVISR_TRY_CUDA(sc.finish());
+    if (sc.host_err()) return fail(NVISR_DEVICE_TIMEOUT, "conv2d: a device-side wait exceeded its bound");
     return NVISR_OK;
 }
 
@@ -2957,40 +2906,32 @@ nvisr_status nvisr_resblock2d(int32_t precision, const float *x, int32_t h, int3
     if (y < x + plane && x < y + plane) return fail(NVISR_INVALID_ARG, "resblock2d: y overlaps x");
     const int dt = precision == NVISR_PREC_FP16 ? DT_F16 : DT_BF16;
     cudaStream_t st = (cudaStream_t)stream;
-    Scratch sc;
-    std::vector<float> hw1((size_t)64 * 64 * 9), hw2(hw1.size()), hb1(64, 0.f), hb2(64, 0.f);
-    NVISR_TRY_CUDA(cudaMemcpyAsync(hw1.data(), w1, hw1.size() * 4, cudaMemcpyDeviceToHost, st));
-    NVISR_TRY_CUDA(cudaMemcpyAsync(hw2.data(), w2, hw2.size() * 4, cudaMemcpyDeviceToHost, st));
-    if (b1) NVISR_TRY_CUDA(cudaMemcpyAsync(hb1.data(), b1, 64 * 4, cudaMemcpyDeviceToHost, st));
-    if (b2) NVISR_TRY_CUDA(cudaMemcpyAsync(hb2.data(), b2, 64 * 4, cudaMemcpyDeviceToHost, st));
-    NVISR_TRY_CUDA(cudaStreamSynchronize(st));
-    std::vector<uint8_t> r1(tc_rows_weight_bytes()), r2(tc_rows_weight_bytes());
-    prepare_weights_rows(hw1.data(), dt, r1.data());
-    prepare_weights_rows(hw2.data(), dt, r2.data());
-    void *dr1, *dr2, *db1, *db2, *dx, *dh, *dy;
+    Scratch sc(st);
     const size_t abytes = plane * 2;
-    NVISR_TRY_CUDA(sc.alloc(r1.size(), &dr1));
-    NVISR_TRY_CUDA(sc.alloc(r2.size(), &dr2));
-    NVISR_TRY_CUDA(sc.alloc(64 * 4, &db1));
-    NVISR_TRY_CUDA(sc.alloc(64 * 4, &db2));
-    NVISR_TRY_CUDA(sc.alloc(abytes, &dx));
-    NVISR_TRY_CUDA(sc.alloc(abytes, &dh));
-    NVISR_TRY_CUDA(sc.alloc(abytes, &dy));
-    NVISR_TRY_CUDA(cudaMemcpyAsync(dr1, r1.data(), r1.size(), cudaMemcpyHostToDevice, st));
-    NVISR_TRY_CUDA(cudaMemcpyAsync(dr2, r2.data(), r2.size(), cudaMemcpyHostToDevice, st));
-    NVISR_TRY_CUDA(cudaMemcpyAsync(db1, hb1.data(), 64 * 4, cudaMemcpyHostToDevice, st));
-    NVISR_TRY_CUDA(cudaMemcpyAsync(db2, hb2.data(), 64 * 4, cudaMemcpyHostToDevice, st));
+    const size_t o_w1 = sc.plan(tc_rows_weight_bytes()), o_w2 = sc.plan(tc_rows_weight_bytes());
+    const size_t o_b1 = sc.plan(64 * 4), o_b2 = sc.plan(64 * 4);
+    const size_t o_x = sc.plan(abytes), o_y = sc.plan(abytes);
+    // the middle tensor's room: the fused form never writes it, but plans with its address
+    const size_t o_h = sc.plan(fused ? 256 : abytes);
+    NVISR_TRY_CUDA(sc.open());
+    void *dx = sc.at<void>(o_x), *dy = sc.at<void>(o_y), *dh = sc.at<void>(o_h);
+    for (int c = 0; c < 2; ++c) {
+        WeightArgs wa{};
+        wa.w = c ? w2 : w1; wa.bias = c ? b2 : b1;
+        wa.cout = wa.cin = wa.cin_pad = wa.cout_pad = wa.nbias = 64;
+        wa.k = 3; wa.layout = WL_ROWS; wa.dt = dt; wa.scale = 1.f;
+        wa.dst = sc.at<void>(c ? o_w2 : o_w1); wa.dst_bias = sc.at<float>(c ? o_b2 : o_b1);
+        NVISR_TRY_CUDA(launch_weights(wa, st));
+    }
     nvisr_status s = pack_planar(x, 64, 64, h, w, dt, 1.f, dx, st, 64);
     if (s != NVISR_OK) return s;
-    int *err;
-    NVISR_TRY_CUDA(sc.alloc(sizeof(int), (void **)&err));
-    NVISR_TRY_CUDA(cudaMemsetAsync(err, 0, sizeof(int), st));
     ConvArgs a1{};
     a1.x = dx; a1.cin_pad = 64; a1.in_cpc = 64; a1.out_cpc = 64; a1.H = h; a1.W = w; a1.nimg = 1;
-    a1.w_rows = dr1; a1.bias = (const float *)db1; a1.cout = 64; a1.cout_pad = 64; a1.k = 3; a1.act = 1;
-    a1.y = dh; a1.in_dt = dt; a1.out_dt = dt; a1.acc_scale = 1.f; a1.out_scale = 1.f; a1.y2_scale = 1.f; a1.err = err;
+    a1.w_rows = sc.at<void>(o_w1); a1.bias = sc.at<float>(o_b1); a1.cout = 64; a1.cout_pad = 64; a1.k = 3; a1.act = 1;
+    a1.y = dh; a1.in_dt = dt; a1.out_dt = dt; a1.acc_scale = 1.f; a1.out_scale = 1.f; a1.y2_scale = 1.f;
+    a1.err = sc.err();
     ConvArgs a2 = a1;
-    a2.x = dh; a2.w_rows = dr2; a2.bias = (const float *)db2; a2.act = 0; a2.res = dx; a2.y = dy;
+    a2.x = dh; a2.w_rows = sc.at<void>(o_w2); a2.bias = sc.at<float>(o_b2); a2.act = 0; a2.res = dx; a2.y = dy;
     cudaError_t e;
     if (fused) {
         if (!res_block_fits(a1, a2)) return fail(NVISR_UNSUPPORTED_FORMAT, "resblock2d: no fused form for these buffers");
@@ -3001,10 +2942,8 @@ nvisr_status nvisr_resblock2d(int32_t precision, const float *x, int32_t h, int3
     }
     if (e != cudaSuccess) return cuda_status(e, "resblock2d");
     NVISR_TRY_CUDA(launch_unpack(dy, dt, 64, 64, 64, h, w, 1.f, y, w, st));
-    int herr = 0;
-    NVISR_TRY_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, st));
-    NVISR_TRY_CUDA(cudaStreamSynchronize(st));
-    if (herr) return fail(NVISR_DEVICE_TIMEOUT, "resblock2d: a device-side wait exceeded its bound");
+    NVISR_TRY_CUDA(sc.finish());
+    if (sc.host_err()) return fail(NVISR_DEVICE_TIMEOUT, "resblock2d: a device-side wait exceeded its bound");
     return NVISR_OK;
 }
 
@@ -3024,74 +2963,51 @@ nvisr_status nvisr_dcn2d(int32_t precision, const float *x, int32_t cin, int32_t
         return fail(NVISR_UNSUPPORTED_FORMAT, "dcn2d: FP32 DCN needs cin % 8 == 0 and 4k channels per group");
     cudaStream_t st = (cudaStream_t)stream;
     const int cin_pad = cin, cout_pad = round_up(cout, 16);
-    Scratch sc;
-    std::vector<float> hw((size_t)cout * cin * 9), hb(cout_pad, 0.f);
-    NVISR_TRY_CUDA(cudaMemcpyAsync(hw.data(), weight, hw.size() * 4, cudaMemcpyDeviceToHost, st));
-    if (bias) NVISR_TRY_CUDA(cudaMemcpyAsync(hb.data(), bias, (size_t)cout * 4, cudaMemcpyDeviceToHost, st));
-    NVISR_TRY_CUDA(cudaStreamSynchronize(st));
-    std::vector<uint8_t> hwl;
-    if (tc) {
-        hwl.resize(tc_weight_bytes(cin_pad, cout_pad, 3, adt));
-        prepare_weights_tc(hw.data(), cout, cin, 3, cin_pad, cout_pad, adt, 1.f, hwl.data(), false);
-    } else {
-        hwl.resize(simt_weight_bytes(cin_pad, cout_pad, 3));
-        prepare_weights_simt(hw.data(), cout, cin, 3, cin_pad, cout_pad, (float *)hwl.data());
-    }
-    void *dw, *db, *dx, *dy, *dom;
-    NVISR_TRY_CUDA(sc.alloc(hwl.size(), &dw));
-    NVISR_TRY_CUDA(cudaMemcpyAsync(dw, hwl.data(), hwl.size(), cudaMemcpyHostToDevice, st));
-    NVISR_TRY_CUDA(sc.alloc(cout_pad * 4, &db));
-    NVISR_TRY_CUDA(cudaMemcpyAsync(db, hb.data(), cout_pad * 4, cudaMemcpyHostToDevice, st));
-    NVISR_TRY_CUDA(sc.alloc((size_t)cin_pad * h * w * dtype_size(adt), &dx));
-    NVISR_TRY_CUDA(sc.alloc((size_t)cout_pad * h * w * dtype_size(adt), &dy));
+    const size_t px = (size_t)h * w;
     // offsets then mask, as one blocked float32 operand [27G -> pad 4]
     const int om_c = 27 * groups, om_cpad = round_up(om_c, 4);
-    NVISR_TRY_CUDA(sc.alloc((size_t)om_cpad * h * w * 4, &dom));
+    Scratch sc(st);
+    const size_t o_w = sc.plan(tc ? tc_weight_bytes(cin_pad, cout_pad, 3, adt) : simt_weight_bytes(cin_pad, cout_pad, 3));
+    const size_t o_b = sc.plan((size_t)cout_pad * 4);
+    const size_t o_x = sc.plan((size_t)cin_pad * px * dtype_size(adt));
+    const size_t o_y = sc.plan((size_t)cout_pad * px * dtype_size(adt));
+    const size_t o_om = sc.plan((size_t)om_cpad * px * 4), o_j = sc.plan((size_t)om_c * px * 4);
+    NVISR_TRY_CUDA(sc.open());
+    void *dx = sc.at<void>(o_x), *dy = sc.at<void>(o_y);
+    float *dom = sc.at<float>(o_om);
+    WeightArgs wa{};
+    wa.w = weight; wa.bias = bias; wa.cout = cout; wa.cin = cin; wa.k = 3; wa.cin_pad = cin_pad; wa.cout_pad = cout_pad;
+    wa.layout = tc ? WL_TC16 : WL_SIMT;
+    wa.dt = adt;
+    wa.ns = tc ? cout_pad / tc_nslice(cin_pad, cout_pad, 3, adt) : 0;
+    wa.scale = 1.f;
+    wa.dst = sc.at<void>(o_w); wa.dst_bias = sc.at<float>(o_b); wa.nbias = cout_pad;
+    NVISR_TRY_CUDA(launch_weights(wa, st));
     {
-        PackArgs pa{};
-        pa.src[0] = offsets;
-        pa.src[1] = mask;
-        pa.nsrc = 1;
-        pa.ch_per_src = 18 * groups;
-        pa.src_pitch = w;
-        pa.src_plane = (int64_t)w * h;
-        pa.H = h;
-        pa.W = w;
-        pa.dst = dom;
-        pa.cpad = om_cpad;
-        pa.dt = DT_F32;
-        pa.scale = 1.f;
         // offsets (18G channels) then mask (9G channels): two packs into one tensor
         // would split a 4-channel chunk when 18G % 4 != 0, so pack from a joined copy
-        void *joined;
-        NVISR_TRY_CUDA(sc.alloc((size_t)om_c * h * w * 4, &joined));
-        NVISR_TRY_CUDA(cudaMemcpyAsync(joined, offsets, (size_t)18 * groups * h * w * 4, cudaMemcpyDeviceToDevice, st));
-        NVISR_TRY_CUDA(cudaMemcpyAsync((float *)joined + (size_t)18 * groups * h * w, mask, (size_t)9 * groups * h * w * 4,
+        float *joined = sc.at<float>(o_j);
+        NVISR_TRY_CUDA(cudaMemcpyAsync(joined, offsets, (size_t)18 * groups * px * 4, cudaMemcpyDeviceToDevice, st));
+        NVISR_TRY_CUDA(cudaMemcpyAsync(joined + (size_t)18 * groups * px, mask, (size_t)9 * groups * px * 4,
                                        cudaMemcpyDeviceToDevice, st));
-        pa.src[0] = (const float *)joined;
-        pa.ch_per_src = om_c;
-        NVISR_TRY_CUDA(launch_pack(pa, st));
+        const nvisr_status s = pack_planar(joined, om_c, om_cpad, h, w, DT_F32, 1.f, dom, st);
+        if (s != NVISR_OK) return s;
     }
     // the tensor-core gather reads x in 8-channel planes
     const int x_cpc = tc ? 8 : layout_cpc(adt, cin_pad), y_cpc = layout_cpc(adt, cout_pad);
     nvisr_status s = pack_planar(x, cin, cin_pad, h, w, adt, 1.f, dx, st, x_cpc);
     if (s != NVISR_OK) return s;
-    int *err;
-    NVISR_TRY_CUDA(sc.alloc(sizeof(int), (void **)&err));
-    NVISR_TRY_CUDA(cudaMemsetAsync(err, 0, sizeof(int), st));
     DcnArgs d{};
     d.x = dx; d.cin_pad = cin_pad; d.H = h; d.W = w; d.groups = groups;
-    d.om = (const float *)dom; d.om_cpad = om_cpad; d.mask_logits = 0;
-    d.w = dw; d.bias = (const float *)db; d.cout = cout; d.cout_pad = cout_pad; d.y = dy;
-    d.in_dt = adt; d.out_dt = adt; d.acc_scale = 1.f; d.out_scale = 1.f; d.err = err;
+    d.om = dom; d.om_cpad = om_cpad; d.mask_logits = 0;
+    d.w = wa.dst; d.bias = wa.dst_bias; d.cout = cout; d.cout_pad = cout_pad; d.y = dy;
+    d.in_dt = adt; d.out_dt = adt; d.acc_scale = 1.f; d.out_scale = 1.f; d.err = sc.err();
     d.x_cpc = x_cpc; d.y_cpc = y_cpc;
     cudaError_t e = tc ? launch_dcn_tc(d, st) : launch_dcn_simt(d, st);
     if (e != cudaSuccess) return cuda_status(e, "dcn2d");
     NVISR_TRY_CUDA(launch_unpack(dy, adt, cout_pad, y_cpc, cout, h, w, 1.f, y, w, st));
-    int herr = 0;
-    NVISR_TRY_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, st));
-    NVISR_TRY_CUDA(cudaStreamSynchronize(st));
-    if (herr) return fail(NVISR_DEVICE_TIMEOUT, "dcn2d: a device-side wait exceeded its bound");
+    NVISR_TRY_CUDA(sc.finish());
+    if (sc.host_err()) return fail(NVISR_DEVICE_TIMEOUT, "dcn2d: a device-side wait exceeded its bound");
     return NVISR_OK;
 }
 
