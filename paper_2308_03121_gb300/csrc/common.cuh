@@ -110,11 +110,8 @@ cudaError_t launch_requant(const nvisr_format &fmt, const float *in, int64_t in_
                            int64_t py, void *u, int64_t pu, void *v, int64_t pv, cudaStream_t st,
                            const SkipArgs *skip = nullptr, int yuv = 0);
 
-// Up to 8 planar float32 frames of 3 channels each (tuple, frame-major
-// channels) or one planar tensor of C channels -> blocked tensor of dtype dt
-// with cpad channels (zero filled past the real channels).  scale multiplies
-// every value before conversion (FP8 quantisation), and amax (optional)
-// receives max |value| (before scaling) via atomicMax on its float bits.
+// Up to 8 planar float32 frames of 3 channels each (frame-major channels) -> blocked tensor of
+// dtype dt with cpad channels (zero filled past the real channels).
 struct PackArgs {
     const float *src[8];
     int nsrc;            // number of source tensors
@@ -126,8 +123,6 @@ struct PackArgs {
     int cpad;
     int dt;
     int cpc;             // channels per chunk of dst (0 = one 16-byte unit)
-    float scale;
-    unsigned *amax;
 };
 cudaError_t launch_pack(const PackArgs &a, cudaStream_t st);
 // Batched pack: n packs whose arguments (cpc set explicitly, same dtype) are in
@@ -135,10 +130,12 @@ cudaError_t launch_pack(const PackArgs &a, cudaStream_t st);
 bool pack_rows_fits(const PackArgs &a);
 cudaError_t launch_pack_table(const PackArgs *host_tab, const PackArgs *dev_tab, int n, cudaStream_t st);
 
-// blocked tensor (cpc channels per chunk) -> planar float32 [C][H][W]
-// (first C channels; value*scale).
-cudaError_t launch_unpack(const void *src, int dt, int cpad, int cpc, int C, int H, int W, float scale,
-                          float *dst, int64_t dst_pitch, cudaStream_t st);
+// Planar float32 [C][H][W] <-> blocked tensor of dtype dt (cpad channels, cpc per chunk: one
+// 16-byte unit (0), or 64 16-bit channels); values are multiplied by scale.
+cudaError_t launch_pack_planar(const float *src, int C, int cpad, int H, int W, int dt, float scale, void *dst, int cpc,
+                               cudaStream_t st);
+cudaError_t launch_unpack_planar(const void *src, int dt, int cpad, int cpc, int C, int H, int W, float scale,
+                                 float *dst, cudaStream_t st);
 
 // Convolution layer (3x3 or 1x1, stride 1, zero padding) on blocked tensors.
 struct ConvArgs {

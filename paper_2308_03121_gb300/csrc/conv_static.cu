@@ -161,29 +161,8 @@ extern "C" nvisr_status nvisr_conv2d_static(int32_t precision, const float *x, i
     wa.scale = 1.f;
     wa.dst = area + (rows ? o_rows : o_w); wa.dst_bias = db; wa.nbias = cout_pad;
     CS_TRY(launch_weights(wa, st));
-    PackArgs pa{};
-    pa.src[0] = x;
-    pa.nsrc = 1;
-    pa.ch_per_src = cin;
-    pa.src_pitch = w;
-    pa.src_plane = (int64_t)w * h;
-    pa.H = h;
-    pa.W = w;
-    pa.dst = dx;
-    pa.cpad = cin_pad;
-    pa.dt = dt;
-    pa.cpc = in_cpc;
-    pa.scale = 1.f;
-    CS_TRY(launch_pack(pa, st));
-    if (res) {
-        PackArgs pr = pa;
-        pr.src[0] = res;
-        pr.ch_per_src = cout;
-        pr.dst = dr;
-        pr.cpad = cout_pad;
-        pr.cpc = out_cpc;
-        CS_TRY(launch_pack(pr, st));
-    }
+    CS_TRY(launch_pack_planar(x, cin, cin_pad, h, w, dt, 1.f, dx, in_cpc, st));
+    if (res) CS_TRY(launch_pack_planar(res, cout, cout_pad, h, w, dt, 1.f, dr, out_cpc, st));
     ConvArgs a{};
     a.x = dx; a.cin_pad = cin_pad; a.H = h; a.W = w; a.nimg = 1; a.bias = db;
     a.w = rows ? nullptr : wa.dst;
@@ -192,7 +171,7 @@ extern "C" nvisr_status nvisr_conv2d_static(int32_t precision, const float *x, i
     a.in_dt = dt; a.out_dt = dt; a.acc_scale = 1.f; a.out_scale = 1.f; a.y2_scale = 1.f; a.err = err;
     a.in_cpc = in_cpc; a.out_cpc = out_cpc;
     CS_TRY(tc ? launch_conv_tc(a, st) : launch_conv_simt(a, st));
-    CS_TRY(launch_unpack(dy, dt, cout_pad, out_cpc, cout, h, w, 1.f, y, w, st));
+    CS_TRY(launch_unpack_planar(dy, dt, cout_pad, out_cpc, cout, h, w, 1.f, y, st));
     int herr = 0;
     CS_TRY(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, st));
     CS_TRY(cudaStreamSynchronize(st));

@@ -1606,7 +1606,6 @@ nvisr_status forward_tuple(nvisr_filter *f, const std::vector<int64_t> &idx, boo
     pa.cpad = pk.cpad;
     pa.dt = pk.dt;
     pa.cpc = pk.cpc;
-    pa.scale = 1.f;
     cudaError_t e;
     {
         ProfScope ps(f, NVISR_K_PACK);
@@ -1697,8 +1696,7 @@ nvisr_status forward_group(nvisr_filter *f, const std::vector<int64_t> &idx) {
             pa.cpad = t.cpad;
             pa.dt = t.dt;
             pa.cpc = t.cpc;
-            pa.scale = 1.f;
-            cudaError_t e;
+                    cudaError_t e;
             {
                 ProfScope ps(f, NVISR_K_PACK);
                 e = launch_pack(pa, f->eng->stream);
@@ -2612,8 +2610,7 @@ nvisr_status nvisr_batch_step(nvisr_batch *b, int32_t *produced) {
             pa.cpad = pk.cpad;
             pa.dt = pk.dt;
             pa.cpc = pk.cpc ? pk.cpc : chunk_channels(pk.dt);
-            pa.scale = 1.f;
-            if (!pack_rows_fits(pa)) return fail(NVISR_INTERNAL, "batch_step: tuple pack layout not supported");
+                    if (!pack_rows_fits(pa)) return fail(NVISR_INTERNAL, "batch_step: tuple pack layout not supported");
             for (const Step &s : f->steps)
                 if (s.op == OP_CONV && s.out_t < 0) set_final_skip(f, s, pf.frames[i].data());
         }
@@ -2806,29 +2803,6 @@ nvisr_status nvisr_fig1_layout(int32_t n, int32_t b, int32_t *cell_frame, int32_
 
 // ---------------------------------------------------------------- per-call layer entry points
 
-namespace {
-
-nvisr_status pack_planar(const float *x, int C, int cpad, int H, int W, int dt, float scale, void *dst,
-                         cudaStream_t st, int cpc = 0) {
-    PackArgs pa{};
-    pa.src[0] = x;
-    pa.nsrc = 1;
-    pa.ch_per_src = C;
-    pa.src_pitch = W;
-    pa.src_plane = (int64_t)W * H;
-    pa.H = H;
-    pa.W = W;
-    pa.dst = dst;
-    pa.cpad = cpad;
-    pa.dt = dt;
-    pa.cpc = cpc;
-    pa.scale = scale;
-    NVISR_TRY_CUDA(launch_pack(pa, st));
-    return NVISR_OK;
-}
-
-}  // namespace
-
 extern "C" {
 
 nvisr_status nvisr_conv2d(int32_t precision, const float *x, int32_t cin, int32_t h, int32_t w, const float *weight,
@@ -2878,9 +2852,8 @@ nvisr_status nvisr_conv2d(int32_t precision, const float *x, int32_t cin, int32_
     wa.scale = 1.f / sw;
     wa.dst = sc.at<void>(o_w); wa.dst_bias = sc.at<float>(o_b); wa.nbias = cout_pad;
     NVISR_TRY_CUDA(launch_weights(wa, st));
-    nvisr_status s = pack_planar(x, cin, cin_pad, h, w, idt, 1.f / sx, dx, st, in_cpc);
-    if (s != NVISR_OK) return s;
-    if (res && (s = pack_planar(res, cout, cout_pad, h, w, adt, 1.f, dr, st, out_cpc)) != NVISR_OK) return s;
+    NVISR_TRY_CUDA(launch_pack_planar(x, cin, cin_pad, h, w, idt, 1.f / sx, dx, in_cpc, st));
+    if (res) NVISR_TRY_CUDA(launch_pack_planar(res, cout, cout_pad, h, w, adt, 1.f, dr, out_cpc, st));
     ConvArgs a{};
     a.x = dx; a.cin_pad = cin_pad; a.H = h; a.W = w; a.nimg = 1; a.bias = wa.dst_bias;
     a.w = rows ? nullptr : wa.dst;
@@ -2890,7 +2863,7 @@ nvisr_status nvisr_conv2d(int32_t precision, const float *x, int32_t cin, int32_
     a.in_cpc = in_cpc; a.out_cpc = out_cpc;
     cudaError_t e = tc ? launch_conv_tc(a, st) : launch_conv_simt(a, st);
     if (e != cudaSuccess) return cuda_status(e, "conv2d");
-    NVISR_TRY_CUDA(launch_unpack(dy, adt, cout_pad, out_cpc, cout, h, w, 1.f, y, w, st));
+    NVISR_TRY_CUDA(launch_unpack_planar(dy, adt, cout_pad, out_cpc, cout, h, w, 1.f, y, st));
     NVISR_TRY_CUDA(sc.finish());
     if (sc.host_err()) return fail(NVISR_DEVICE_TIMEOUT, "conv2d: a device-side wait exceeded its bound");
     return NVISR_OK;
@@ -2923,8 +2896,7 @@ nvisr_status nvisr_resblock2d(int32_t precision, const float *x, int32_t h, int3
         wa.dst = sc.at<void>(c ? o_w2 : o_w1); wa.dst_bias = sc.at<float>(c ? o_b2 : o_b1);
         NVISR_TRY_CUDA(launch_weights(wa, st));
     }
-    nvisr_status s = pack_planar(x, 64, 64, h, w, dt, 1.f, dx, st, 64);
-    if (s != NVISR_OK) return s;
+    NVISR_TRY_CUDA(launch_pack_planar(x, 64, 64, h, w, dt, 1.f, dx, 64, st));
     ConvArgs a1{};
     a1.x = dx; a1.cin_pad = 64; a1.in_cpc = 64; a1.out_cpc = 64; a1.H = h; a1.W = w; a1.nimg = 1;
     a1.w_rows = sc.at<void>(o_w1); a1.bias = sc.at<float>(o_b1); a1.cout = 64; a1.cout_pad = 64; a1.k = 3; a1.act = 1;
@@ -2941,7 +2913,7 @@ nvisr_status nvisr_resblock2d(int32_t precision, const float *x, int32_t h, int3
         if (e == cudaSuccess) e = launch_conv_tc(a2, st);
     }
     if (e != cudaSuccess) return cuda_status(e, "resblock2d");
-    NVISR_TRY_CUDA(launch_unpack(dy, dt, 64, 64, 64, h, w, 1.f, y, w, st));
+    NVISR_TRY_CUDA(launch_unpack_planar(dy, dt, 64, 64, 64, h, w, 1.f, y, st));
     NVISR_TRY_CUDA(sc.finish());
     if (sc.host_err()) return fail(NVISR_DEVICE_TIMEOUT, "resblock2d: a device-side wait exceeded its bound");
     return NVISR_OK;
@@ -2990,13 +2962,11 @@ nvisr_status nvisr_dcn2d(int32_t precision, const float *x, int32_t cin, int32_t
         NVISR_TRY_CUDA(cudaMemcpyAsync(joined, offsets, (size_t)18 * groups * px * 4, cudaMemcpyDeviceToDevice, st));
         NVISR_TRY_CUDA(cudaMemcpyAsync(joined + (size_t)18 * groups * px, mask, (size_t)9 * groups * px * 4,
                                        cudaMemcpyDeviceToDevice, st));
-        const nvisr_status s = pack_planar(joined, om_c, om_cpad, h, w, DT_F32, 1.f, dom, st);
-        if (s != NVISR_OK) return s;
+        NVISR_TRY_CUDA(launch_pack_planar(joined, om_c, om_cpad, h, w, DT_F32, 1.f, dom, 0, st));
     }
     // the tensor-core gather reads x in 8-channel planes
     const int x_cpc = tc ? 8 : layout_cpc(adt, cin_pad), y_cpc = layout_cpc(adt, cout_pad);
-    nvisr_status s = pack_planar(x, cin, cin_pad, h, w, adt, 1.f, dx, st, x_cpc);
-    if (s != NVISR_OK) return s;
+    NVISR_TRY_CUDA(launch_pack_planar(x, cin, cin_pad, h, w, adt, 1.f, dx, x_cpc, st));
     DcnArgs d{};
     d.x = dx; d.cin_pad = cin_pad; d.H = h; d.W = w; d.groups = groups;
     d.om = dom; d.om_cpad = om_cpad; d.mask_logits = 0;
@@ -3005,7 +2975,7 @@ nvisr_status nvisr_dcn2d(int32_t precision, const float *x, int32_t cin, int32_t
     d.x_cpc = x_cpc; d.y_cpc = y_cpc;
     cudaError_t e = tc ? launch_dcn_tc(d, st) : launch_dcn_simt(d, st);
     if (e != cudaSuccess) return cuda_status(e, "dcn2d");
-    NVISR_TRY_CUDA(launch_unpack(dy, adt, cout_pad, y_cpc, cout, h, w, 1.f, y, w, st));
+    NVISR_TRY_CUDA(launch_unpack_planar(dy, adt, cout_pad, y_cpc, cout, h, w, 1.f, y, st));
     NVISR_TRY_CUDA(sc.finish());
     if (sc.host_err()) return fail(NVISR_DEVICE_TIMEOUT, "dcn2d: a device-side wait exceeded its bound");
     return NVISR_OK;

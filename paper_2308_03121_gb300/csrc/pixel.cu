@@ -629,55 +629,11 @@ __global__ void __launch_bounds__(128) requant420_kernel(const float *__restrict
 }
 
 template <typename T>
-__device__ __forceinline__ T cvt_out(float v);
-template <>
-__device__ __forceinline__ float cvt_out<float>(float v) { return v; }
-template <>
-__device__ __forceinline__ __nv_bfloat16 cvt_out<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
-template <>
-__device__ __forceinline__ __half cvt_out<__half>(float v) { return __float2half_rn(v); }
-template <>
-__device__ __forceinline__ __nv_fp8_e4m3 cvt_out<__nv_fp8_e4m3>(float v) { return __nv_fp8_e4m3(v); }
-
-template <typename T>
 __device__ __forceinline__ float cvt_in(T v) { return (float)v; }
 template <>
 __device__ __forceinline__ float cvt_in<__nv_bfloat16>(__nv_bfloat16 v) { return __bfloat162float(v); }
 template <>
 __device__ __forceinline__ float cvt_in<__half>(__half v) { return __half2float(v); }
-
-// One thread per 16-byte unit of the destination, in memory order: unit idx
-// is (chunk c, pixel p, unit v of the chunk) with idx = (c*HW + p)*upch + v.
-template <typename T>
-__global__ void __launch_bounds__(256) pack_kernel(PackArgs a) {
-    constexpr int UPC = 16 / sizeof(T);  // channels per unit
-    const int64_t HW = (int64_t)a.H * a.W;
-    const int upch = a.cpc / UPC;         // units per chunk
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= HW * (a.cpad / UPC)) return;
-    const int64_t cp = idx / upch;
-    const int v = (int)(idx - cp * upch);
-    const int c = (int)(cp / HW);
-    const int64_t p = cp - (int64_t)c * HW;
-    const int y = (int)(p / a.W), x = (int)(p - (int64_t)y * a.W);
-    const int creal = a.nsrc * a.ch_per_src;
-    alignas(16) T vals[UPC];
-    float amax = 0.f;
-#pragma unroll
-    for (int e = 0; e < UPC; ++e) {
-        const int ch = c * a.cpc + v * UPC + e;
-        float val = 0.f;
-        if (ch < creal) {
-            const int s = ch / a.ch_per_src, cc = ch - s * a.ch_per_src;
-            val = a.src[s][cc * a.src_plane + (int64_t)y * a.src_pitch + x];
-        }
-        amax = fmaxf(amax, fabsf(val));
-        vals[e] = cvt_out<T>(val * a.scale);
-    }
-    *reinterpret_cast<uint4 *>(reinterpret_cast<uint8_t *>(a.dst) + idx * 16) =
-        *reinterpret_cast<const uint4 *>(vals);
-    if (a.amax) atomicMax(a.amax, __float_as_uint(amax));
-}
 
 // 16 bytes of UPC consecutive channels, converted from float.
 template <typename T>
@@ -724,8 +680,7 @@ __device__ __forceinline__ uint4 pack_unit<__nv_fp8_e4m3>(const float *v) {
 // destination unit of the 4 pixels is one 16-byte store, contiguous across the
 // 4 pixels (and across the warp) for every unit index.  Needs 16-byte aligned
 // source rows whose pitch covers W rounded up to 4 (the last group of a row
-// reads into that padding and stores only pixels < W); otherwise the per-unit
-// kernel above runs.
+// reads into that padding and stores only pixels < W), as the frame ring has.
 template <typename T>
 __device__ __forceinline__ void pack_rows(const PackArgs &a) {
     constexpr int UPC = 16 / sizeof(T);
@@ -736,7 +691,6 @@ __device__ __forceinline__ void pack_rows(const PackArgs &a) {
     const int upch = a.cpc / UPC;
     const int creal = a.nsrc * a.ch_per_src;
     const int64_t p0 = (int64_t)y * a.W + x0;
-    float amax = 0.f;
     for (int u = 0; u < a.cpad / UPC; ++u) {  // unit index over all channels
         float v[4][UPC];
 #pragma unroll
@@ -747,21 +701,16 @@ __device__ __forceinline__ void pack_rows(const PackArgs &a) {
                 const int s = ch / a.ch_per_src, cc = ch - s * a.ch_per_src;
                 f = __ldg(reinterpret_cast<const float4 *>(a.src[s] + cc * a.src_plane + (int64_t)y * a.src_pitch + x0));
             }
-            amax = fmaxf(amax, fmaxf(fmaxf(fabsf(f.x), fabsf(f.y)), fmaxf(fabsf(f.z), fabsf(f.w))));
-            v[0][e] = f.x * a.scale;
-            v[1][e] = f.y * a.scale;
-            v[2][e] = f.z * a.scale;
-            v[3][e] = f.w * a.scale;
+            v[0][e] = f.x;
+            v[1][e] = f.y;
+            v[2][e] = f.z;
+            v[3][e] = f.w;
         }
         const int c = u / upch, vv = u - c * upch;
         uint8_t *d = reinterpret_cast<uint8_t *>(a.dst) + (((int64_t)c * HW + p0) * upch + vv) * 16;
 #pragma unroll
         for (int k = 0; k < 4; ++k)
             if (x0 + k < a.W) *reinterpret_cast<uint4 *>(d + (int64_t)k * upch * 16) = pack_unit<T>(v[k]);
-    }
-    if (a.amax) {
-        const unsigned m = __reduce_max_sync(__activemask(), __float_as_uint(amax));
-        if ((threadIdx.x & 31) == (__ffs(__activemask()) - 1)) atomicMax(a.amax, m);
     }
 }
 
@@ -777,25 +726,122 @@ __global__ void __launch_bounds__(128) pack_rows_table_kernel(const PackArgs *__
     pack_rows<T>(tab[blockIdx.z]);
 }
 
-template <typename T>
-__global__ void __launch_bounds__(256) unpack_kernel(const uint8_t *__restrict__ src, int cpad, int cpc, int C,
-                                                     int H, int W, float scale, float *dst, int64_t pitch) {
-    constexpr int UPC = 16 / sizeof(T);
-    const int64_t HW = (int64_t)H * W;
-    const int upch = cpc / UPC;
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= HW * (cpad / UPC)) return;
-    const int64_t cp = idx / upch;
-    const int v = (int)(idx - cp * upch);
-    const int c = (int)(cp / HW);
-    const int64_t p = cp - (int64_t)c * HW;
-    const int y = (int)(p / W), x = (int)(p - (int64_t)y * W);
-    alignas(16) T vals[UPC];
-    *reinterpret_cast<uint4 *>(vals) = *reinterpret_cast<const uint4 *>(src + idx * 16);
+// Layout change between a layer's planar float32 tensor [C][HW] and its blocked form, for whole
+// frames without row padding.  Both directions move each byte once (HBM-bound); what costs time
+// is touching memory in pieces below its 32-byte sectors, so a warp covers full lines on both
+// sides.
+//
+// Blocks of 64 16-bit channels (a 128-byte line per pixel): a warp takes 32 pixels x 4 units of 8
+// channels; lane = (unit lane / 8, pixels lane % 8).  VEC (pixel planes 16-byte aligned): a lane
+// owns 4 adjacent pixels, so a channel is one 16-byte access per lane (128 contiguous bytes per
+// unit) and a pixel's units are 64 contiguous bytes of its line.  Otherwise (odd sizes) a lane owns
+// pixels l, l + 8, ..., and a channel is four 4-byte accesses (32 contiguous bytes).
+// A BF16 residual block at 1920 x 1080 with both around it: 965 -> 461 us a call (pack 314, unpack
+// 429 us before, with a thread per 4 pixels and all channels, and one per unit in memory order).
+constexpr int LINE_PX = 32 * 4;  // pixels per block of 256 threads: 8 warps = 4 pixel groups x 2 channel halves
+template <bool VEC>
+__device__ __forceinline__ int64_t line_px(int j) {
+    const int lane = threadIdx.x & 31, g = threadIdx.x >> 6;
+    const int64_t p0 = (int64_t)blockIdx.x * LINE_PX + g * 32;
+    return p0 + (VEC ? (lane & 7) * 4 + j : (lane & 7) + 8 * j);
+}
+
+template <typename T, bool VEC>
+__global__ void __launch_bounds__(256) pack_lines_kernel(const float *__restrict__ src, int64_t HW, int C, int nblk,
+                                                         float scale, uint8_t *__restrict__ dst) {
+    const int unit = ((threadIdx.x >> 5) & 1) * 4 + ((threadIdx.x & 31) >> 3);
+    for (int blk = blockIdx.y; blk < nblk; blk += gridDim.y) {
+        const int c0 = blk * 64 + unit * 8;
+        float v[4][8];
 #pragma unroll
-    for (int e = 0; e < UPC; ++e) {
-        const int ch = c * cpc + v * UPC + e;
-        if (ch < C) dst[(int64_t)ch * pitch * H + (int64_t)y * pitch + x] = cvt_in<T>(vals[e]) * scale;
+        for (int e = 0; e < 8; ++e) {
+            const float *row = src + (int64_t)(c0 + e) * HW;
+            const bool real = c0 + e < C;
+            if (VEC) {
+                const int64_t p = line_px<true>(0);
+                const float4 f = real && p < HW ? __ldg(reinterpret_cast<const float4 *>(row + p)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                v[0][e] = f.x; v[1][e] = f.y; v[2][e] = f.z; v[3][e] = f.w;
+            } else {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) v[j][e] = real && line_px<false>(j) < HW ? __ldg(row + line_px<false>(j)) : 0.f;
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int64_t p = line_px<VEC>(j);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) v[j][e] *= scale;
+            if (p < HW)
+                *reinterpret_cast<uint4 *>(dst + ((int64_t)blk * HW + p) * 128 + unit * 16) = pack_unit<T>(v[j]);
+        }
+    }
+}
+
+template <typename T, bool VEC>
+__global__ void __launch_bounds__(256) unpack_lines_kernel(const uint8_t *__restrict__ src, int64_t HW, int C,
+                                                           int nblk, float scale, float *__restrict__ dst) {
+    const int unit = ((threadIdx.x >> 5) & 1) * 4 + ((threadIdx.x & 31) >> 3);
+    for (int blk = blockIdx.y; blk < nblk; blk += gridDim.y) {
+        const int c0 = blk * 64 + unit * 8;
+        float v[4][8];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int64_t p = line_px<VEC>(j);
+            alignas(16) T t[8];
+            *reinterpret_cast<uint4 *>(t) =
+                p < HW ? __ldg(reinterpret_cast<const uint4 *>(src + ((int64_t)blk * HW + p) * 128 + unit * 16))
+                       : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) v[j][e] = cvt_in<T>(t[e]) * scale;
+        }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            if (c0 + e >= C) break;
+            float *row = dst + (int64_t)(c0 + e) * HW;
+            if (VEC) {
+                const int64_t p = line_px<true>(0);
+                if (p < HW) *reinterpret_cast<float4 *>(row + p) = make_float4(v[0][e], v[1][e], v[2][e], v[3][e]);
+            } else {
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (line_px<false>(j) < HW) row[line_px<false>(j)] = v[j][e];
+            }
+        }
+    }
+}
+
+// Blocks of one 16-byte unit (8 16-bit, 16 FP8 or 4 float32 channels): a lane takes one pixel of
+// unit blockIdx.y, so each channel and the unit itself are contiguous across the warp whatever
+// the alignment.
+template <typename T>
+__global__ void __launch_bounds__(256) pack_units_kernel(const float *__restrict__ src, int64_t HW, int C, int nunits,
+                                                         float scale, uint8_t *__restrict__ dst) {
+    constexpr int UPC = 16 / sizeof(T);
+    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= HW) return;
+    for (int u = blockIdx.y; u < nunits; u += gridDim.y) {
+        float v[UPC];
+#pragma unroll
+        for (int e = 0; e < UPC; ++e) {
+            const int c = u * UPC + e;
+            v[e] = c < C ? __ldg(src + (int64_t)c * HW + p) * scale : 0.f;
+        }
+        *reinterpret_cast<uint4 *>(dst + ((int64_t)u * HW + p) * 16) = pack_unit<T>(v);
+    }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256) unpack_units_kernel(const uint8_t *__restrict__ src, int64_t HW, int C,
+                                                           int nunits, float scale, float *__restrict__ dst) {
+    constexpr int UPC = 16 / sizeof(T);
+    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= HW) return;
+    for (int u = blockIdx.y; u < nunits; u += gridDim.y) {
+        alignas(16) T t[UPC];
+        *reinterpret_cast<uint4 *>(t) = __ldg(reinterpret_cast<const uint4 *>(src + ((int64_t)u * HW + p) * 16));
+#pragma unroll
+        for (int e = 0; e < UPC; ++e)
+            if (u * UPC + e < C) dst[(int64_t)(u * UPC + e) * HW + p] = cvt_in<T>(t[e]) * scale;
     }
 }
 
@@ -911,25 +957,45 @@ cudaError_t launch_pack(const PackArgs &a0, cudaStream_t st) {
     PackArgs a = a0;
     const int upc = chunk_channels(a.dt);
     if (a.cpc == 0) a.cpc = upc;
-    if (a.cpc % upc || a.cpad % a.cpc) return cudaErrorInvalidValue;
-    if (pack_rows_fits(a)) {
-        dim3 blk(128), grd((a.W / 4 + 127) / 128, a.H);
-        switch (a.dt) {
-            case DT_F32: pack_rows_kernel<float><<<grd, blk, 0, st>>>(a); break;
-            case DT_BF16: pack_rows_kernel<__nv_bfloat16><<<grd, blk, 0, st>>>(a); break;
-            case DT_F16: pack_rows_kernel<__half><<<grd, blk, 0, st>>>(a); break;
-            default: pack_rows_kernel<__nv_fp8_e4m3><<<grd, blk, 0, st>>>(a); break;
+    if (!pack_rows_fits(a)) return cudaErrorInvalidValue;
+    dim3 blk(128), grd((a.W / 4 + 127) / 128, a.H);
+    switch (a.dt) {
+        case DT_F32: pack_rows_kernel<float><<<grd, blk, 0, st>>>(a); break;
+        case DT_BF16: pack_rows_kernel<__nv_bfloat16><<<grd, blk, 0, st>>>(a); break;
+        case DT_F16: pack_rows_kernel<__half><<<grd, blk, 0, st>>>(a); break;
+        default: pack_rows_kernel<__nv_fp8_e4m3><<<grd, blk, 0, st>>>(a); break;
+    }
+    return cudaGetLastError();
+}
+
+cudaError_t launch_pack_planar(const float *src, int C, int cpad, int H, int W, int dt, float scale, void *dst, int cpc,
+                               cudaStream_t st) {
+    const int upc = chunk_channels(dt);
+    if (cpc == 0) cpc = upc;
+    const int64_t HW = (int64_t)H * W;
+    uint8_t *d = static_cast<uint8_t *>(dst);
+    if (cpc == 64 && upc == 8) {
+        if (cpad % 64) return cudaErrorInvalidValue;
+        const int n = cpad / 64;
+        const dim3 grd((unsigned)((HW + LINE_PX - 1) / LINE_PX), (unsigned)std::min(n, 65535));
+        const bool vec = HW % 4 == 0 && (reinterpret_cast<uintptr_t>(src) & 15) == 0;
+        if (dt == DT_BF16) {
+            if (vec) pack_lines_kernel<__nv_bfloat16, true><<<grd, 256, 0, st>>>(src, HW, C, n, scale, d);
+            else pack_lines_kernel<__nv_bfloat16, false><<<grd, 256, 0, st>>>(src, HW, C, n, scale, d);
+        } else {
+            if (vec) pack_lines_kernel<__half, true><<<grd, 256, 0, st>>>(src, HW, C, n, scale, d);
+            else pack_lines_kernel<__half, false><<<grd, 256, 0, st>>>(src, HW, C, n, scale, d);
         }
         return cudaGetLastError();
     }
-    const int64_t n = (int64_t)a.H * a.W * (a.cpad / upc);
-    const int block = 256;
-    const int64_t grid = (n + block - 1) / block;
-    switch (a.dt) {
-        case DT_F32: pack_kernel<float><<<(unsigned)grid, block, 0, st>>>(a); break;
-        case DT_BF16: pack_kernel<__nv_bfloat16><<<(unsigned)grid, block, 0, st>>>(a); break;
-        case DT_F16: pack_kernel<__half><<<(unsigned)grid, block, 0, st>>>(a); break;
-        default: pack_kernel<__nv_fp8_e4m3><<<(unsigned)grid, block, 0, st>>>(a); break;
+    if (cpc != upc || cpad % upc) return cudaErrorInvalidValue;
+    const int n = cpad / upc;
+    const dim3 grd((unsigned)((HW + 255) / 256), (unsigned)std::min(n, 65535));
+    switch (dt) {
+        case DT_F32: pack_units_kernel<float><<<grd, 256, 0, st>>>(src, HW, C, n, scale, d); break;
+        case DT_BF16: pack_units_kernel<__nv_bfloat16><<<grd, 256, 0, st>>>(src, HW, C, n, scale, d); break;
+        case DT_F16: pack_units_kernel<__half><<<grd, 256, 0, st>>>(src, HW, C, n, scale, d); break;
+        default: pack_units_kernel<__nv_fp8_e4m3><<<grd, 256, 0, st>>>(src, HW, C, n, scale, d); break;
     }
     return cudaGetLastError();
 }
@@ -962,20 +1028,34 @@ cudaError_t launch_pack_table(const PackArgs *host_tab, const PackArgs *dev_tab,
     return cudaGetLastError();
 }
 
-cudaError_t launch_unpack(const void *src, int dt, int cpad, int cpc, int C, int H, int W, float scale, float *dst,
-                          int64_t dst_pitch, cudaStream_t st) {
+cudaError_t launch_unpack_planar(const void *src, int dt, int cpad, int cpc, int C, int H, int W, float scale,
+                                 float *dst, cudaStream_t st) {
     const int upc = chunk_channels(dt);
     if (cpc == 0) cpc = upc;
-    if (cpc % upc || cpad % cpc) return cudaErrorInvalidValue;
-    const int64_t n = (int64_t)H * W * (cpad / upc);
-    const int block = 256;
-    const unsigned grid = (unsigned)((n + block - 1) / block);
-    const uint8_t *s = (const uint8_t *)src;
+    const int64_t HW = (int64_t)H * W;
+    const uint8_t *s = static_cast<const uint8_t *>(src);
+    if (cpc == 64 && upc == 8) {
+        if (cpad % 64) return cudaErrorInvalidValue;
+        const int n = cpad / 64;
+        const dim3 grd((unsigned)((HW + LINE_PX - 1) / LINE_PX), (unsigned)std::min(n, 65535));
+        const bool vec = HW % 4 == 0 && (reinterpret_cast<uintptr_t>(dst) & 15) == 0;
+        if (dt == DT_BF16) {
+            if (vec) unpack_lines_kernel<__nv_bfloat16, true><<<grd, 256, 0, st>>>(s, HW, C, n, scale, dst);
+            else unpack_lines_kernel<__nv_bfloat16, false><<<grd, 256, 0, st>>>(s, HW, C, n, scale, dst);
+        } else {
+            if (vec) unpack_lines_kernel<__half, true><<<grd, 256, 0, st>>>(s, HW, C, n, scale, dst);
+            else unpack_lines_kernel<__half, false><<<grd, 256, 0, st>>>(s, HW, C, n, scale, dst);
+        }
+        return cudaGetLastError();
+    }
+    if (cpc != upc || cpad % upc) return cudaErrorInvalidValue;
+    const int n = cpad / upc;
+    const dim3 grd((unsigned)((HW + 255) / 256), (unsigned)std::min(n, 65535));
     switch (dt) {
-        case DT_F32: unpack_kernel<float><<<grid, block, 0, st>>>(s, cpad, cpc, C, H, W, scale, dst, dst_pitch); break;
-        case DT_BF16: unpack_kernel<__nv_bfloat16><<<grid, block, 0, st>>>(s, cpad, cpc, C, H, W, scale, dst, dst_pitch); break;
-        case DT_F16: unpack_kernel<__half><<<grid, block, 0, st>>>(s, cpad, cpc, C, H, W, scale, dst, dst_pitch); break;
-        default: unpack_kernel<__nv_fp8_e4m3><<<grid, block, 0, st>>>(s, cpad, cpc, C, H, W, scale, dst, dst_pitch); break;
+        case DT_F32: unpack_units_kernel<float><<<grd, 256, 0, st>>>(s, HW, C, n, scale, dst); break;
+        case DT_BF16: unpack_units_kernel<__nv_bfloat16><<<grd, 256, 0, st>>>(s, HW, C, n, scale, dst); break;
+        case DT_F16: unpack_units_kernel<__half><<<grd, 256, 0, st>>>(s, HW, C, n, scale, dst); break;
+        default: unpack_units_kernel<__nv_fp8_e4m3><<<grd, 256, 0, st>>>(s, HW, C, n, scale, dst); break;
     }
     return cudaGetLastError();
 }
