@@ -249,8 +249,9 @@ cudaError_t launch_weights(const WeightArgs &a, cudaStream_t st);
 // max |v| of n device values, as float bits, by atomicMax into *out.
 cudaError_t launch_absmax(const float *v, int64_t n, unsigned *out, cudaStream_t st);
 
-// DCN: x blocked (activation dtype); offsets and mask in one blocked float32
-// tensor [om_cpad/4][H][W][4].  Channel order: torchvision's ([0, 18G) = (dy, dx)
+// DCN: x blocked (activation dtype; the tensor-core kernel takes it in pixel pairs, see below);
+// offsets and mask either planar float32 ([18G][H][W] and [9G][H][W] in torchvision's order) or
+// in one blocked float32 tensor [om_cpad/4][H][W][4].  Channel order of the latter: torchvision's ([0, 18G) = (dy, dx)
 // per (group, tap), [18G, 27G) = mask per (group, tap)), or tap-major (for tap
 // k a block of 3G channels: (dy, dx) of each group, then each group's mask),
 // which puts all of a tap's offsets and masks in 3G/4 adjacent 4-channel
@@ -262,10 +263,12 @@ __host__ __device__ inline int dcn_mask_channel(int g, int k, int G, bool tap_ma
     return tap_major ? 3 * G * k + 2 * G + g : 18 * G + g * 9 + k;
 }
 struct DcnArgs {
-    const void *x;
+    const void *x;           // SIMT: blocked; tensor cores: the pixel pairs of channels 0-31
+    const void *x_hi;        // tensor cores: the pixel pairs of channels 32-63
     int cin_pad, H, W, groups;
-    int x_cpc, y_cpc;        // channels per chunk of x and y (0 = 16-byte units)
-    const float *om;
+    int x_cpc, y_cpc;        // channels per chunk of x (SIMT) and y (0 = 16-byte units)
+    const float *om;         // blocked offsets and mask, or the planar offsets
+    const float *om_mask;    // the planar mask; null: om is blocked
     int om_cpad;
     int om_tap_major;        // channel order of om (tap-major needs an even G)
     int mask_logits;
@@ -280,9 +283,13 @@ struct DcnArgs {
 };
 cudaError_t launch_dcn_simt(const DcnArgs &a, cudaStream_t st);
 cudaError_t launch_dcn_tc(const DcnArgs &a, cudaStream_t st);
-// Copies a 16-bit activation from the blocked layout with x_cpc channels per
-// chunk into 8-channel planes [cpad/8][H][W][8] (the DCN gather's layout).
-cudaError_t launch_dcn_relayout8(const void *x, int cpad, int H, int W, int x_cpc, void *y, cudaStream_t st);
+// The DCN gather's input: for each 8-channel chunk a plane [H][W] of 32-byte entries, the 16-bit
+// channels of pixels x and x + 1 (zero past the row's end): one aligned load fetches a sample
+// row's two corners.  Chunks 0-3 go to lo, 4-7 to hi (DCN_PAIR_BYTES a pixel each).
+constexpr int DCN_PAIR_BYTES = 4 * 32;
+// From a blocked 64-channel tensor (8 or 64 channels per chunk), or from planar float32 [64][H][W].
+cudaError_t launch_dcn_pairs(const void *x, int H, int W, int x_cpc, void *lo, void *hi, cudaStream_t st);
+cudaError_t launch_dcn_pairs_planar(const float *x, int H, int W, int dt, void *lo, void *hi, cudaStream_t st);
 
 int device_sm_count();
 // The driver's tensor-map encoder (cuTensorMapEncodeTiled), or null when it is missing.

@@ -7,18 +7,21 @@
 //     y[o,p] = b[o] + sum_{c,k} w[o,c,k] * m[g,k](p) * bilinear(x_c, p + p_k + d[g,k](p))
 // with out-of-image bilinear corners contributing zero.
 //
-// Kernel: one CTA per SM walks 128-pixel row tiles.  For each tile and tap,
-// sixteen producer warps (a warp per 8-channel chunk and half tile, a lane pair
-// per pixel) read the tap's offsets and mask, issue the bilinear corner loads
-// of all their pixels before using any (so many gathers are in flight at
-// once), blend them in FP32 with the mask folded into the row weights, and store 8-byte halves of the
-// 16-byte rows of the canonical no-swizzle K-major A tile in shared memory (the
-// sampled im2col tile of that tap).  A single thread issues the tap's
-// tcgen05.mma's against the resident weights into a double-buffered TMEM
-// accumulator; four epilogue warps add the bias and store the blocked output.
-// Every wait is bounded in time.  x is best given in 8-channel planes
-// (launch_dcn_relayout8), where the two columns of a bilinear corner pair share
-// a cache line; any supported layout gives the same result.
+// Kernel: one CTA per SM walks 128-pixel row tiles.  For each tile and tap, sixteen producer
+// warps (a warp per 8-channel chunk and half tile, a lane per pixel) read the tap's offsets and
+// mask, issue the bilinear corner loads of all their pixels before using any (so many gathers
+// are in flight at once), blend them in FP32 with the mask folded into the row weights, and
+// store 16-byte rows of the canonical no-swizzle K-major A tile in shared memory (the sampled
+// im2col tile of that tap).  One warp issues the tap's tcgen05.mma's against the resident
+// weights into a double-buffered TMEM accumulator; four epilogue warps add the bias and store
+// the blocked output.  Every wait is bounded in time.
+//
+// What bounds it: the L1 data stage, one wavefront per distinct 128-byte line of a request, and
+// instruction issue.  x comes in pixel pairs (launch_dcn_pairs): a 32-byte entry holds the
+// 8 channels of pixels x and x + 1, so a lane fetches both corners of a sample row with one
+// aligned 32-byte load and blends all 8 channels itself.  (From 16-byte entries a lane pair
+// shared each pixel: 9 shuffles per 16 pixels for the records and the halves, and twice the
+// blend's overhead: 311 M warp instructions at 960 x 540 and 8 groups.)
 #include "common.cuh"
 #include "sm100_ptx.cuh"
 
@@ -27,11 +30,16 @@ namespace nvisr {
 namespace {
 
 constexpr int TM = 128;
-constexpr int NGATHER = 512;            // gather threads (a lane pair per pixel and chunk)
+constexpr int NGATHER = 512;            // gather threads (a lane per pixel and chunk, two passes)
 constexpr int MMA_WARP = NGATHER / 32;  // then 4 epilogue warps, the first also loads the weights and issues the MMAs
 constexpr int NT = NGATHER + 128;       // 20 warps: 5 per SM sub-partition leaves 96 registers a thread
 constexpr uint64_t WAIT_NS = 2000000000ull;
 constexpr int SMEM_LIMIT = 232448;
+// Stages of sampled taps.  Shared memory beyond 164 KB would shrink L1, which needs a line for every
+// corner load in flight: at 960 x 540 with independent offsets of sigma 2 px a whole nvisr_dcn2d
+// call takes 492 us with 5 stages (92 KB of L1) and 798 us with 8 (28 KB); the space-time filter's
+// layer with its input copy 340 against 400 us.
+constexpr int MAX_STAGES = 5;
 
 template <typename T>
 struct Cv;
@@ -80,8 +88,19 @@ __device__ __forceinline__ void ffma2(float2 &acc, float s, float2 v) {
     asm("mov.b64 {%0, %1}, %2;" : "=f"(acc.x), "=f"(acc.y) : "l"(d));
 }
 
-// T: 16-bit element type of x / y; NS: output channels (one slice); C: input channels.
-template <typename T, int NS, int C>
+__device__ __forceinline__ float2 fmul2(float s, float2 v) {
+    uint64_t d, x, w;
+    float2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(v.x), "f"(v.y));
+    asm("mov.b64 %0, {%1, %1};" : "=l"(w) : "f"(s));
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(w), "l"(x));
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(d));
+    return r;
+}
+
+// T: 16-bit element type of x / y; NS: output channels (one slice); C: input channels; PLANAR:
+// planar offsets and mask.
+template <typename T, int NS, int C, bool PLANAR>
 __global__ void __launch_bounds__(NT, 1) dcn_tc_kernel(const DcnArgs a, int stages) {
     constexpr int CPC = 8;                 // channels per 16-byte chunk
     constexpr int NCH = C / CPC;           // chunks per tap (= K / 8)
@@ -108,7 +127,7 @@ __global__ void __launch_bounds__(NT, 1) dcn_tc_kernel(const DcnArgs a, int stag
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int H = a.H, W = a.W;
     // blocked layouts [C/cpc][H][W][cpc]: byte address of the 8-channel unit starting at channel c
-    const int xcpc = a.x_cpc, ycpc = a.y_cpc;
+    const int ycpc = a.y_cpc;
     const int64_t HW = (int64_t)H * W;
     const int tiles_x = (W + TM - 1) / TM;
     const int ntiles = tiles_x * H;
@@ -126,6 +145,10 @@ __global__ void __launch_bounds__(NT, 1) dcn_tc_kernel(const DcnArgs a, int stag
         mbar_init(wbar, 1);
         *abort = 0;
         fence_mbarrier_init();
+        // the weights are not the previous kernel's: they load before the wait below
+        mbar_arrive_expect_tx(wbar, wbytes);
+        for (uint32_t off = 0; off < wbytes; off += 32768u)
+            bulk_load(wsm + off, static_cast<const uint8_t *>(a.w) + off, min(32768u, wbytes - off), wbar);
     }
     if (warp == MMA_WARP) {
         tmem_alloc(tmem_slot, NCOLS);
@@ -142,118 +165,103 @@ __global__ void __launch_bounds__(NT, 1) dcn_tc_kernel(const DcnArgs a, int stag
 
     if (warp < NGATHER / 32) {
         // ------------------------------------------------ gather producers
-        // A lane pair holds one sample row of one (pixel, 8-channel chunk): lane c
-        // loads column x0 + c.  With x in 8-channel planes both columns sit in one
-        // 128-byte line (unless x0 ends a line), so a warp's load of 16 pixels of
-        // one chunk touches about 18 lines instead of 32 (the L1 data stage takes
-        // a wavefront per line).  The pair then swaps halves: lane 0 blends
-        // channels 0-3 and lane 1 channels 4-7, each from all four corners.
         constexpr int NGW = NGATHER / 32;  // gather warps
         constexpr int WPC = NGW / NCH;     // warps per chunk
         constexpr int PPW = TM / WPC;      // pixels per warp
-        constexpr int NPASS = PPW / 16;    // 16 pixels (32 lanes) per pass
-        static_assert(NGW % NCH == 0 && PPW % 16 == 0, "gather mapping");
+        constexpr int NPASS = PPW / 32;    // 32 pixels per pass
+        static_assert(NGW % NCH == 0 && PPW % 32 == 0, "gather mapping");
         const int cc = warp % NCH;         // channel chunk of this warp
-        const int c = lane & 1;            // column x0 + c of the corner pair
-        const int pb = (warp / NCH) * PPW + (lane >> 1);
-        const uint8_t *x = static_cast<const uint8_t *>(a.x);
+        const int pb = (warp / NCH) * PPW + lane;
         const int G = a.groups;
         const int g = (cc * CPC) / (a.cin_pad / G);
         const bool tapm = a.om_tap_major != 0;
-        const uint8_t *plane = x + (int64_t)((cc * CPC) / xcpc) * HW * xcpc * 2 + ((cc * CPC) % xcpc) * 2;
-        const uint32_t pstride = (uint32_t)xcpc * 2;  // bytes per pixel in the plane (the plane is < 2 GiB)
-        const uint32_t rowb = (uint32_t)W * pstride;  // bytes per row of the plane
-        static_assert(NPASS % 2 == 0, "passes shared by a lane pair");
-        constexpr int NP2 = NPASS / 2;
+        // this chunk's plane of 32-byte pixel pairs (below 4 GiB)
+        const uint8_t *plane = static_cast<const uint8_t *>(cc < NCH / 2 ? a.x : a.x_hi) + (int64_t)(cc % (NCH / 2)) * HW * 32;
+        const uint32_t rowb = (uint32_t)W * 32u;
         int s = 0;
         uint32_t ph = 0;
         bool ok = true;
-        // Corner values.  A corner is loaded only when its weight is nonzero, which the
-        // bounds checks allow only inside the image.  A skipped corner keeps the value
-        // of an earlier load (or zero), which its weight of zero cancels (x is finite).
-        uint4 v[NPASS][2];
+        // Corner values [pass][row]: words 0-3 the entry's first pixel, 4-7 the second.  A row is
+        // loaded only when its weights are not all zero, which the bounds checks allow only
+        // inside the image.  A skipped row keeps the values of an earlier load (or zero), which
+        // its zero weights cancel (x is finite).
+        uint32_t v[NPASS][2][8];
 #pragma unroll
-        for (int j = 0; j < NPASS; ++j) v[j][0] = v[j][1] = make_uint4(0u, 0u, 0u, 0u);
-        // offsets and mask of this lane's passes h = 2i + c for tap k of tile t: loaded one
-        // tap ahead of their use, so that their DRAM latency overlaps the previous tap
-        auto load_om = [&](int t, int k, float2 (&d)[NP2], float (&lg)[NP2]) {
+        for (int h = 0; h < NPASS; ++h)
+#pragma unroll
+            for (int e = 0; e < 8; ++e) v[h][0][e] = v[h][1][e] = 0u;
+        // offsets and mask of this lane's pixels for tap k of tile t: loaded one tap ahead of
+        // their use, so that their DRAM latency overlaps the previous tap
+        auto load_om = [&](int t, int k, float2 (&d)[NPASS], float (&lg)[NPASS]) {
             const int y = t / tiles_x;
             const int xb = (t - y * tiles_x) * TM;
-            const int cd = dcn_off_channel(g, k, G, tapm), cm = dcn_mask_channel(g, k, G, tapm);
-            // float offsets in 32 bits (the tensor is < 2^31 floats)
-            const uint32_t od = (uint32_t)(cd >> 2) * (uint32_t)HW * 4u + (cd & 3);
-            const uint32_t oms = (uint32_t)(cm >> 2) * (uint32_t)HW * 4u + (cm & 3);
+            // float offsets in 32 bits (the tensors are < 2^31 floats)
+            uint32_t od, oms;
+            if (PLANAR) {
+                od = (uint32_t)dcn_off_channel(g, k, G, false) * (uint32_t)HW;
+                oms = (uint32_t)(g * 9 + k) * (uint32_t)HW;
+            } else {
+                const int cd = dcn_off_channel(g, k, G, tapm), cm = dcn_mask_channel(g, k, G, tapm);
+                od = (uint32_t)(cd >> 2) * (uint32_t)HW * 4u + (cd & 3);
+                oms = (uint32_t)(cm >> 2) * (uint32_t)HW * 4u + (cm & 3);
+            }
 #pragma unroll
-            for (int i = 0; i < NP2; ++i) {
-                const int px = xb + pb + (2 * i + c) * 16;
-                const uint32_t pix4 = (uint32_t)(y * W + min(px, W - 1)) * 4u;
-                d[i] = __ldg(reinterpret_cast<const float2 *>(a.om + od + pix4));
-                lg[i] = __ldg(a.om + oms + pix4);
+            for (int h = 0; h < NPASS; ++h) {
+                const uint32_t pix = (uint32_t)(y * W + min(xb + pb + 32 * h, W - 1));
+                if (PLANAR) {
+                    d[h] = make_float2(__ldg(a.om + od + pix), __ldg(a.om + od + (uint32_t)HW + pix));
+                    lg[h] = __ldg(a.om_mask + oms + pix);
+                } else {
+                    d[h] = __ldg(reinterpret_cast<const float2 *>(a.om + od + pix * 4u));
+                    lg[h] = __ldg(a.om + oms + pix * 4u);
+                }
             }
         };
-        float2 nd[NP2];
-        float nlg[NP2];
+        float2 nd[NPASS];
+        float nlg[NPASS];
         if (blockIdx.x < ntiles && !a.starve) load_om(blockIdx.x, 0, nd, nlg);
         for (int t = blockIdx.x; t < ntiles && ok && !a.starve; t += gridDim.x) {
             const int y = t / tiles_x;
             const int xb = (t - y * tiles_x) * TM;
             for (int k = 0; k < 9; ++k) {
-                // The lane pair shares its sample records: lane c computes those of the
-                // passes h = 2i + c (offsets, mask, corner weights, position), and both
-                // lanes then read each pass's record from the lane that computed it.
-                // Record: row weights wy0, wy1 (times the mask), column weights wx0, wx1
-                // (each zero outside the image), and y0 * W + x0.
-                float2 cd2[NP2];
-                float clg[NP2];
+                float2 cd[NPASS];
+                float clg[NPASS];
 #pragma unroll
-                for (int i = 0; i < NP2; ++i) {
-                    cd2[i] = nd[i];
-                    clg[i] = nlg[i];
+                for (int h = 0; h < NPASS; ++h) {
+                    cd[h] = nd[h];
+                    clg[h] = nlg[h];
                 }
                 if (k < 8) load_om(t, k + 1, nd, nlg);
                 else if (t + (int)gridDim.x < ntiles) load_om(t + gridDim.x, 0, nd, nlg);
-                float ewy0[NP2], ewy1[NP2], ewx0[NP2], ewx1[NP2];
-                uint32_t eb[NP2];
+                // row weights (times the mask) and column weights, each zero outside the image,
+                // then the corner loads (every load of the tap is issued before the first blend)
+                float wy[NPASS][2], wxa[NPASS], wxb[NPASS];
 #pragma unroll
-                for (int i = 0; i < NP2; ++i) {
-                    const int px = xb + pb + (2 * i + c) * 16;
-                    const float2 d = cd2[i];
-                    const float lg = clg[i];
+                for (int h = 0; h < NPASS; ++h) {
+                    const int px = xb + pb + 32 * h;
                     // mask = sigmoid(logit) with the fast exponential and division: a relative
                     // error near 1e-6, far below the 16-bit rounding of the sample it scales
                     // (0 and 1 at the extremes); the exact form cost 4 % of the launch
-                    const float m = a.mask_logits ? __fdividef(1.f, 1.f + __expf(-lg)) : lg;
-                    const float sy = (float)(y + k / 3 - 1) + d.x;
-                    const float sx = (float)(px + k % 3 - 1) + d.y;
+                    const float m = a.mask_logits ? __fdividef(1.f, 1.f + __expf(-clg[h])) : clg[h];
+                    const float sy = (float)(y + k / 3 - 1) + cd[h].x;
+                    const float sx = (float)(px + k % 3 - 1) + cd[h].y;
                     const float fy = floorf(sy), fx = floorf(sx);
                     const int y0 = (int)fy, x0 = (int)fx;
                     const float ly = sy - fy, lx = sx - fx;
                     const bool in = px < W;
-                    ewy0[i] = in && (unsigned)y0 < (unsigned)H ? (1.f - ly) * m : 0.f;
-                    ewy1[i] = in && (unsigned)(y0 + 1) < (unsigned)H ? ly * m : 0.f;
-                    ewx0[i] = (unsigned)x0 < (unsigned)W ? 1.f - lx : 0.f;
-                    ewx1[i] = (unsigned)(x0 + 1) < (unsigned)W ? lx : 0.f;
-                    eb[i] = (uint32_t)y0 * (uint32_t)W + (uint32_t)x0;
+                    wy[h][0] = in && (unsigned)y0 < (unsigned)H ? (1.f - ly) * m : 0.f;
+                    wy[h][1] = in && (unsigned)(y0 + 1) < (unsigned)H ? ly * m : 0.f;
+                    const float wx0 = (unsigned)x0 < (unsigned)W ? 1.f - lx : 0.f;
+                    const float wx1 = (unsigned)(x0 + 1) < (unsigned)W ? lx : 0.f;
+                    // left of the image (x0 = -1) column x0 + 1 is entry 0's first pixel
+                    wxa[h] = x0 < 0 ? wx1 : wx0;
+                    wxb[h] = x0 < 0 ? 0.f : wx1;
+                    const bool need = wxa[h] != 0.f || wxb[h] != 0.f;
+                    const uint32_t o0 = ((uint32_t)y0 * (uint32_t)W + (uint32_t)max(x0, 0)) * 32u;
+                    if (need && wy[h][0] != 0.f) ld_global_nc_v8(plane + o0, v[h][0]);
+                    if (need && wy[h][1] != 0.f) ld_global_nc_v8(plane + (o0 + rowb), v[h][1]);
                 }
-                // each pass's record from the lane that computed it, then its corner loads
-                // (every load of the tap is issued before the first blend)
-                float wy0[NPASS], wy1[NPASS], wxo[NPASS], wxp[NPASS];
-#pragma unroll
-                for (int h = 0; h < NPASS; ++h) {
-                    const int src = (lane & ~1) | (h & 1);
-                    wy0[h] = __shfl_sync(0xffffffffu, ewy0[h >> 1], src);
-                    wy1[h] = __shfl_sync(0xffffffffu, ewy1[h >> 1], src);
-                    const float x0w = __shfl_sync(0xffffffffu, ewx0[h >> 1], src);
-                    const float x1w = __shfl_sync(0xffffffffu, ewx1[h >> 1], src);
-                    const uint32_t bs = __shfl_sync(0xffffffffu, eb[h >> 1], src);
-                    wxo[h] = c ? x1w : x0w;  // weight of this lane's column x0 + c
-                    wxp[h] = c ? x0w : x1w;  // weight of the partner's column
-                    const uint32_t o0 = (bs + (uint32_t)c) * pstride;
-                    if (wy0[h] != 0.f && wxo[h] != 0.f) v[h][0] = __ldg(reinterpret_cast<const uint4 *>(plane + o0));
-                    if (wy1[h] != 0.f && wxo[h] != 0.f) v[h][1] = __ldg(reinterpret_cast<const uint4 *>(plane + (o0 + rowb)));
-                }
-                // the corner loads are in flight while the warp waits for a free stage; the
-                // shuffles below need the whole warp: it leaves together
+                // the corner loads are in flight while the warp waits for a free stage
                 const bool got = mbar_wait_bounded(&empty[s], ph ^ 1, abort, WAIT_NS);
                 if (!__all_sync(0xffffffffu, got)) {
                     *abort = 1;
@@ -261,27 +269,25 @@ __global__ void __launch_bounds__(NT, 1) dcn_tc_kernel(const DcnArgs a, int stag
                     ok = false;
                     break;
                 }
-                uint8_t *stg = stage0 + (size_t)s * STAGE + (size_t)cc * LBO + c * 8;
+                uint8_t *stg = stage0 + (size_t)s * STAGE + (size_t)cc * LBO;
 #pragma unroll
                 for (int h = 0; h < NPASS; ++h) {
-                    // lane 0 blends channels 0-3 and lane 1 channels 4-7: each keeps its half
-                    // of its own column x0 + c and takes the partner's half of column x0 + 1 - c
-                    float2 acc[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+                    // channels 0-3 add column x0 before x0 + 1, channels 4-7 the other way round
+                    float2 acc[4];
 #pragma unroll
                     for (int r = 0; r < 2; ++r) {
-                        const uint4 q = v[h][r];
-                        const uint32_t k0 = c ? q.z : q.x, k1 = c ? q.w : q.y;
-                        const uint32_t g0 = __shfl_xor_sync(0xffffffffu, c ? q.x : q.z, 1);
-                        const uint32_t g1 = __shfl_xor_sync(0xffffffffu, c ? q.y : q.w, 1);
-                        const float wr = r ? wy1[h] : wy0[h];
-                        const float wa = wr * wxo[h], wb = wr * wxp[h];
-                        ffma2(acc[0], wa, unpack_pair<T>(k0));
-                        ffma2(acc[1], wa, unpack_pair<T>(k1));
-                        ffma2(acc[0], wb, unpack_pair<T>(g0));
-                        ffma2(acc[1], wb, unpack_pair<T>(g1));
+                        const float fa = wy[h][r] * wxa[h], fb = wy[h][r] * wxb[h];
+#pragma unroll
+                        for (int w = 0; w < 4; ++w) {
+                            const float2 pa = unpack_pair<T>(v[h][r][w]), pbv = unpack_pair<T>(v[h][r][4 + w]);
+                            if (r == 0) acc[w] = fmul2(w < 2 ? fa : fb, w < 2 ? pa : pbv);
+                            else ffma2(acc[w], w < 2 ? fa : fb, w < 2 ? pa : pbv);
+                            ffma2(acc[w], w < 2 ? fb : fa, w < 2 ? pbv : pa);
+                        }
                     }
-                    *reinterpret_cast<uint2 *>(stg + (size_t)(pb + h * 16) * 16) =
-                        make_uint2(pack_pair<T>(acc[0].x, acc[0].y), pack_pair<T>(acc[1].x, acc[1].y));
+                    *reinterpret_cast<uint4 *>(stg + (size_t)(pb + h * 32) * 16) =
+                        make_uint4(pack_pair<T>(acc[0].x, acc[0].y), pack_pair<T>(acc[1].x, acc[1].y),
+                                   pack_pair<T>(acc[2].x, acc[2].y), pack_pair<T>(acc[3].x, acc[3].y));
                 }
                 fence_proxy_async();  // generic smem writes -> visible to the tensor core
                 mbar_arrive(&full[s]);
@@ -290,8 +296,8 @@ __global__ void __launch_bounds__(NT, 1) dcn_tc_kernel(const DcnArgs a, int stag
         }
     } else {
         // ------------------------------------------------ epilogue (the last 4 warps, one per lane quadrant);
-        // lane 0 of the first also loads the weights and issues every tile's MMAs, and
-        // that warp stores its quadrant of tile i - 1 after issuing tile i
+        // the first also issues every tile's MMAs (its elected lane), and stores its quadrant
+        // of tile i - 1 after issuing tile i
         const bool issuer = warp == MMA_WARP;
         const int q = warp & 3;
         const int m = q * 32 + lane;
@@ -301,73 +307,65 @@ __global__ void __launch_bounds__(NT, 1) dcn_tc_kernel(const DcnArgs a, int stag
         bool issue = true;   // the issuer still issues
         int s = 0, last_ab = -1;
         uint32_t ph = 0, last_par = 0;
-        if (issuer) {
+        uint32_t el = 0;
+        auto fail = [&]() {
             if (lane == 0) {
-                mbar_arrive_expect_tx(wbar, wbytes);
-                for (uint32_t off = 0; off < wbytes; off += 32768u)
-                    bulk_load(wsm + off, static_cast<const uint8_t *>(a.w) + off, min(32768u, wbytes - off), wbar);
-                issue = mbar_wait_bounded(wbar, 0, abort, WAIT_NS);
-                if (!issue) {
-                    *abort = 1;
-                    if (a.err) atomicExch(a.err, DEVERR_TIMEOUT);
-                }
+                *abort = 1;
+                if (a.err) atomicExch(a.err, DEVERR_TIMEOUT);
             }
-            issue = __shfl_sync(0xffffffffu, issue, 0);
+        };
+        auto await = [&](uint64_t *bar, uint32_t parity) {
+            return (bool)__all_sync(0xffffffffu, mbar_wait_bounded(bar, parity, abort, WAIT_NS));
+        };
+        if (issuer) {
+            el = elect_one();
+            issue = await(wbar, 0);
+            if (!issue) fail();
         }
         // issues the 9 taps of tile number it (buffer it & 1); false when a wait gave up
         auto issue_tile = [&](int it) -> bool {
-            bool good = true;
-            if (lane == 0) {
-                const int ab = it & 1;
-                const uint32_t u = (uint32_t)(it >> 1);
-                good = mbar_wait_bounded(&tempty[ab], (u & 1) ^ 1, abort, WAIT_NS);
-                if (good) {
+            const int ab = it & 1;
+            const uint32_t u = (uint32_t)(it >> 1);
+            bool good = await(&tempty[ab], (u & 1) ^ 1);
+            if (good) {
+                tc_fence_after();
+                const uint32_t d_tmem = tmem_base + (uint32_t)(ab * NS);
+                for (int k = 0; k < 9; ++k) {
+                    good = await(&full[s], ph);
+                    if (!good) {
+                        if (k > 0) {  // the final wait then covers the taps already issued
+                            umma_commit_warp(el, &tfull[ab]);
+                            last_ab = ab;
+                            last_par = u & 1;
+                        }
+                        break;
+                    }
                     tc_fence_after();
-                    const uint32_t d_tmem = tmem_base + (uint32_t)(ab * NS);
-                    for (int k = 0; k < 9 && good; ++k) {
-                        good = mbar_wait_bounded(&full[s], ph, abort, WAIT_NS);
-                        if (!good) {
-                            if (k > 0) {  // the final wait then covers the taps already issued
-                                umma_commit(&tfull[ab]);
-                                last_ab = ab;
-                                last_par = u & 1;
-                            }
-                            break;
-                        }
-                        tc_fence_after();
-                        const uint32_t sb = smem_u32(stage0 + (size_t)s * STAGE);
+                    const uint32_t sb = smem_u32(stage0 + (size_t)s * STAGE);
 #pragma unroll
-                        for (int j = 0; j < NCH / 2; ++j) {
-                            const uint64_t ad = smem_desc(sb + 2 * j * LBO, LBO, 128);
-                            const uint64_t bd = smem_desc(wbase + (uint32_t)((k * NCH + 2 * j) * NS * 16), NS * 16, 128);
-                            umma<0>(d_tmem, ad, bd, IDESC, (k | j) != 0 ? 1u : 0u);
-                        }
-                        umma_commit(&empty[s]);
-                        if (++s == S) { s = 0; ph ^= 1; }
+                    for (int j = 0; j < NCH / 2; ++j) {
+                        const uint64_t ad = smem_desc(sb + 2 * j * LBO, LBO, 128);
+                        const uint64_t bd = smem_desc(wbase + (uint32_t)((k * NCH + 2 * j) * NS * 16), NS * 16, 128);
+                        umma_warp<0>(el, d_tmem, ad, bd, IDESC, (k | j) != 0 ? 1u : 0u);
                     }
-                    if (good) {
-                        umma_commit(&tfull[ab]);
-                        last_ab = ab;
-                        last_par = u & 1;
-                    }
+                    umma_commit_warp(el, &empty[s]);
+                    if (++s == S) { s = 0; ph ^= 1; }
                 }
-                if (!good) {
-                    *abort = 1;
-                    if (a.err) atomicExch(a.err, DEVERR_TIMEOUT);
+                if (good) {
+                    umma_commit_warp(el, &tfull[ab]);
+                    last_ab = ab;
+                    last_par = u & 1;
                 }
             }
-            return __shfl_sync(0xffffffffu, good, 0);
+            if (!good) fail();
+            return good;
         };
         // stores this warp's quadrant of tile t (number it); false when the wait gave up
         auto store_tile = [&](int t, int it) -> bool {
             const int ab = it & 1;
             const uint32_t u = (uint32_t)(it >> 1);
-            const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&tfull[ab], u & 1, abort, WAIT_NS));
-            if (!ok) {
-                if (lane == 0) {
-                    *abort = 1;
-                    if (a.err) atomicExch(a.err, DEVERR_TIMEOUT);
-                }
+            if (!await(&tfull[ab], u & 1)) {
+                fail();
                 return false;
             }
             tc_fence_after();
@@ -423,18 +421,18 @@ __global__ void __launch_bounds__(NT, 1) dcn_tc_kernel(const DcnArgs a, int stag
     }
 }
 
-template <typename T, int NS, int C>
+template <typename T, int NS, int C, bool PLANAR>
 cudaError_t run(const DcnArgs &a, cudaStream_t st) {
     constexpr uint32_t STAGE = (C / 8) * TM * 16;
     constexpr uint32_t wbytes = 9 * (C / 8) * NS * 16;
     const uint32_t wround = (wbytes + 1023) & ~1023u;
     int stages = (SMEM_LIMIT - 2048 - (int)wround) / (int)STAGE;
-    if (stages > 8) stages = 8;
+    if (stages > MAX_STAGES) stages = MAX_STAGES;
     if (stages < 2) return cudaErrorInvalidConfiguration;
     int smem = 2048 + (int)wround + stages * (int)STAGE;
     if (smem < 118 * 1024) smem = 118 * 1024;
-    auto kern = dcn_tc_kernel<T, NS, C>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    auto kern = dcn_tc_kernel<T, NS, C, PLANAR>;
+    cudaError_t e = set_smem_limit<dcn_tc_kernel<T, NS, C, PLANAR>>(smem);
     if (e != cudaSuccess) return e;
     const int tiles = ((a.W + TM - 1) / TM) * a.H;
     int grid = device_sm_count();
@@ -442,43 +440,88 @@ cudaError_t run(const DcnArgs &a, cudaStream_t st) {
     return launch_dependent(kern, grid, NT, smem, st, a, stages);
 }
 
-// One thread per (pixel, 8-channel chunk), chunk fastest: a warp reads four
-// pixels' 128-byte channel lines and writes 64-byte runs of eight planes.
-__global__ void relayout8_kernel(const uint4 *__restrict__ x, int64_t HW, int nch, int xcpc, uint4 *__restrict__ y) {
+// One thread per (pixel, 8-channel chunk), chunk fastest: a warp reads four pixels' 128-byte
+// channel lines (and their right neighbours, which L1 holds) and writes four 32-byte entries of
+// eight planes, 128 contiguous bytes each.
+__global__ void __launch_bounds__(256) dcn_pairs_kernel(const uint4 *__restrict__ x, int64_t HW, int W, int per,
+                                                        uint4 *__restrict__ lo, uint4 *__restrict__ hi) {
     const int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (u >= HW * nch) return;
-    const int64_t p = u / nch;
-    const int cc = (int)(u - p * nch);
-    const int per = xcpc / 8;  // 16-byte chunks per pixel in the source layout
-    y[(int64_t)cc * HW + p] = __ldg(x + ((int64_t)(cc / per) * HW + p) * per + cc % per);
+    const int64_t p = u >> 3;
+    const int cc = (int)(u & 7);
+    if (p >= HW) return;
+    const uint4 *src = x + ((int64_t)(cc / per) * HW + p) * per + cc % per;  // per: chunks per pixel line
+    const bool last = (int)(p % W) == W - 1;
+    const uint4 v0 = __ldg(src);
+    const uint4 v1 = last ? make_uint4(0u, 0u, 0u, 0u) : __ldg(src + per);
+    uint4 *d = (cc < 4 ? lo : hi) + ((int64_t)(cc & 3) * HW + p) * 2;
+    d[0] = v0;
+    d[1] = v1;
+}
+
+// The same from planar float32: one lane per pixel, blockIdx.y the chunk; a lane's right
+// neighbour comes from lane + 1 (lane 31 reads it itself).
+template <typename T>
+__global__ void __launch_bounds__(256) dcn_pairs_planar_kernel(const float *__restrict__ x, int64_t HW, int W,
+                                                               uint4 *__restrict__ lo, uint4 *__restrict__ hi) {
+    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int cc = blockIdx.y;
+    const float *src = x + (int64_t)cc * 8 * HW;
+    auto load = [&](int64_t q) {
+        float f[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) f[e] = q < HW ? __ldg(src + (int64_t)e * HW + q) : 0.f;
+        return make_uint4(pack_pair<T>(f[0], f[1]), pack_pair<T>(f[2], f[3]), pack_pair<T>(f[4], f[5]),
+                          pack_pair<T>(f[6], f[7]));
+    };
+    const uint4 v0 = load(p);
+    uint4 v1;
+    v1.x = __shfl_down_sync(0xffffffffu, v0.x, 1);
+    v1.y = __shfl_down_sync(0xffffffffu, v0.y, 1);
+    v1.z = __shfl_down_sync(0xffffffffu, v0.z, 1);
+    v1.w = __shfl_down_sync(0xffffffffu, v0.w, 1);
+    if ((threadIdx.x & 31) == 31) v1 = load(p + 1);
+    if (p >= HW) return;
+    if ((int)(p % W) == W - 1) v1 = make_uint4(0u, 0u, 0u, 0u);
+    uint4 *d = (cc < 4 ? lo : hi) + ((int64_t)(cc & 3) * HW + p) * 2;
+    d[0] = v0;
+    d[1] = v1;
 }
 
 }  // namespace
 
-cudaError_t launch_dcn_relayout8(const void *x, int cpad, int H, int W, int x_cpc, void *y, cudaStream_t st) {
-    if (cpad % 8 || x_cpc % 8 || cpad % x_cpc) return cudaErrorInvalidValue;
-    const int64_t HW = (int64_t)H * W, units = HW * (cpad / 8);
-    if (units == 0) return cudaSuccess;
-    const int64_t blocks = (units + 255) / 256;
-    relayout8_kernel<<<(unsigned)blocks, 256, 0, st>>>(static_cast<const uint4 *>(x), HW, cpad / 8, x_cpc,
-                                                       static_cast<uint4 *>(y));
+cudaError_t launch_dcn_pairs(const void *x, int H, int W, int x_cpc, void *lo, void *hi, cudaStream_t st) {
+    if (x_cpc != 8 && x_cpc != 64) return cudaErrorInvalidValue;
+    const int64_t HW = (int64_t)H * W;
+    dcn_pairs_kernel<<<(unsigned)((HW * 8 + 255) / 256), 256, 0, st>>>(static_cast<const uint4 *>(x), HW, W, x_cpc / 8,
+                                                                       static_cast<uint4 *>(lo), static_cast<uint4 *>(hi));
+    return cudaGetLastError();
+}
+
+cudaError_t launch_dcn_pairs_planar(const float *x, int H, int W, int dt, void *lo, void *hi, cudaStream_t st) {
+    const int64_t HW = (int64_t)H * W;
+    const dim3 grd((unsigned)((HW + 255) / 256), 8);
+    uint4 *l = static_cast<uint4 *>(lo), *h = static_cast<uint4 *>(hi);
+    if (dt == DT_BF16) dcn_pairs_planar_kernel<__nv_bfloat16><<<grd, 256, 0, st>>>(x, HW, W, l, h);
+    else if (dt == DT_F16) dcn_pairs_planar_kernel<__half><<<grd, 256, 0, st>>>(x, HW, W, l, h);
+    else return cudaErrorInvalidValue;
     return cudaGetLastError();
 }
 
 cudaError_t launch_dcn_tc(const DcnArgs &a0, cudaStream_t st) {
     DcnArgs a = a0;
     a.starve = test_starve();
-    if (a.x_cpc == 0) a.x_cpc = 8;
     if (a.y_cpc == 0) a.y_cpc = 8;
     if (a.cin_pad != 64 || a.cout_pad != 64 || (a.cin_pad / a.groups) % 8) return cudaErrorNotSupported;
-    // x in 8-channel planes (launch_dcn_relayout8); y blocked by 8 or 64 channels
-    if (a.x_cpc != 8 || (a.y_cpc != 8 && a.y_cpc != 64)) return cudaErrorNotSupported;
+    if (!a.x_hi || (a.y_cpc != 8 && a.y_cpc != 64)) return cudaErrorNotSupported;
     if (a.om_tap_major && a.groups % 2) return cudaErrorNotSupported;
-    // 32-bit gather offsets into a plane of x and into om
-    if ((int64_t)a.H * a.W * a.x_cpc * 2 >= (int64_t(1) << 31) || (int64_t)a.H * a.W * a.om_cpad >= (int64_t(1) << 31))
+    // 32-bit gather offsets into a plane of x and into the offsets and mask
+    if ((int64_t)a.H * a.W * 32 >= (int64_t(1) << 32) || (int64_t)a.H * a.W * a.om_cpad >= (int64_t(1) << 31))
         return cudaErrorNotSupported;
-    if (a.in_dt == DT_BF16 && a.out_dt == DT_BF16) return run<__nv_bfloat16, 64, 64>(a, st);
-    if (a.in_dt == DT_F16 && a.out_dt == DT_F16) return run<__half, 64, 64>(a, st);
+    const bool planar = a.om_mask != nullptr;
+    if (a.in_dt == DT_BF16 && a.out_dt == DT_BF16)
+        return planar ? run<__nv_bfloat16, 64, 64, true>(a, st) : run<__nv_bfloat16, 64, 64, false>(a, st);
+    if (a.in_dt == DT_F16 && a.out_dt == DT_F16)
+        return planar ? run<__half, 64, 64, true>(a, st) : run<__half, 64, 64, false>(a, st);
     return cudaErrorNotSupported;
 }
 

@@ -256,7 +256,7 @@ struct nvisr_filter {
     std::vector<Weights> weights;  // per layer (shared layers point to the owner)
     std::vector<int> om_tap_g;     // per layer: G when its output rows are stored tap-major, else 0
     std::vector<Tensor> tensors;
-    void *dcn_x8 = nullptr;        // DCN input in 8-channel planes (tensor-core path)
+    void *dcn_lo = nullptr, *dcn_hi = nullptr;  // DCN input in pixel pairs (tensor-core path)
     std::vector<Step> steps;
     std::vector<char> blk;           // step i and i + 1 form a residual block run as one fused launch
     int pack_t = -1;               // tensor id of the packed tuple
@@ -1291,16 +1291,21 @@ nvisr_status build_plan_group(nvisr_filter *f, const float *blob) {
             f->wvar.push_back(Wv);
         }
     }
-    // the tensor-core DCN gathers from its input copied into 8-channel planes
-    size_t x8 = 0;
+    // the tensor-core DCN gathers from its input copied into pixel pairs.  Half of them may use
+    // the first output's float32 image where it is large enough: the run's last layers write it
+    // after every DCN, and an output of an earlier run has left it by then
+    size_t pairs = 0;
     for (const Step &st : f->steps)
-        if (st.op == OP_DCN && f->tc && f->tensors[st.in_t].cpc != 8) {
-            const Tensor &T = f->tensors[st.in_t];
-            x8 = std::max(x8, (size_t)T.cpad * T.H * T.W * dtype_size(T.dt));
-        }
-    if (x8) {
-        nvisr_status s = dalloc(f->eng, x8, f->owned, &f->dcn_x8, f->guard);
+        if (st.op == OP_DCN && f->tc)
+            pairs = std::max(pairs, (size_t)DCN_PAIR_BYTES * f->tensors[st.in_t].H * f->tensors[st.in_t].W);
+    if (pairs) {
+        nvisr_status s = dalloc(f->eng, pairs, f->owned, &f->dcn_lo, f->guard);
         if (s != NVISR_OK) return s;
+        if (sizeof(float) * 3 * f->opitch * H * net.scale_y >= pairs) {
+            f->dcn_hi = f->out_rgb[0];
+        } else if ((s = dalloc(f->eng, pairs, f->owned, &f->dcn_hi, f->guard)) != NVISR_OK) {
+            return s;
+        }
     }
     for (Tensor &T : f->tensors)
         if (T.parent >= 0) {
@@ -1534,11 +1539,12 @@ nvisr_status run_step(nvisr_filter *f, const Step &s, const float *const *frames
         d.y = o.ptr; d.in_dt = in.dt; d.out_dt = o.dt; d.acc_scale = 1.f; d.out_scale = 1.f;
         d.err = f->eng->err_word;
         ProfScope ps(f, NVISR_K_DCN);
-        if (f->tc && in.cpc != 8) {
-            cudaError_t e = launch_dcn_relayout8(in.ptr, in.cpad, in.H, in.W, in.cpc, f->dcn_x8, st);
+        if (f->tc) {
+            if (in.cpad != 64) return cuda_status(cudaErrorNotSupported, ("dcn layer " + L.name).c_str());
+            cudaError_t e = launch_dcn_pairs(in.ptr, in.H, in.W, in.cpc, f->dcn_lo, f->dcn_hi, st);
             if (e != cudaSuccess) return cuda_status(e, ("dcn layer " + L.name + " relayout").c_str());
-            d.x = f->dcn_x8;
-            d.x_cpc = 8;
+            d.x = f->dcn_lo;
+            d.x_hi = f->dcn_hi;
         }
         cudaError_t e = f->tc ? launch_dcn_tc(d, st) : launch_dcn_simt(d, st);
         if (e != cudaSuccess) return cuda_status(e, ("dcn layer " + L.name).c_str());
@@ -2936,17 +2942,14 @@ nvisr_status nvisr_dcn2d(int32_t precision, const float *x, int32_t cin, int32_t
     cudaStream_t st = (cudaStream_t)stream;
     const int cin_pad = cin, cout_pad = round_up(cout, 16);
     const size_t px = (size_t)h * w;
-    // offsets then mask, as one blocked float32 operand [27G -> pad 4]
-    const int om_c = 27 * groups, om_cpad = round_up(om_c, 4);
     Scratch sc(st);
     const size_t o_w = sc.plan(tc ? tc_weight_bytes(cin_pad, cout_pad, 3, adt) : simt_weight_bytes(cin_pad, cout_pad, 3));
     const size_t o_b = sc.plan((size_t)cout_pad * 4);
-    const size_t o_x = sc.plan((size_t)cin_pad * px * dtype_size(adt));
+    const size_t o_x = sc.plan(tc ? DCN_PAIR_BYTES * px : (size_t)cin_pad * px * 4);
+    const size_t o_xh = tc ? sc.plan(DCN_PAIR_BYTES * px) : 0;
     const size_t o_y = sc.plan((size_t)cout_pad * px * dtype_size(adt));
-    const size_t o_om = sc.plan((size_t)om_cpad * px * 4), o_j = sc.plan((size_t)om_c * px * 4);
     NVISR_TRY_CUDA(sc.open());
     void *dx = sc.at<void>(o_x), *dy = sc.at<void>(o_y);
-    float *dom = sc.at<float>(o_om);
     WeightArgs wa{};
     wa.w = weight; wa.bias = bias; wa.cout = cout; wa.cin = cin; wa.k = 3; wa.cin_pad = cin_pad; wa.cout_pad = cout_pad;
     wa.layout = tc ? WL_TC16 : WL_SIMT;
@@ -2955,24 +2958,16 @@ nvisr_status nvisr_dcn2d(int32_t precision, const float *x, int32_t cin, int32_t
     wa.scale = 1.f;
     wa.dst = sc.at<void>(o_w); wa.dst_bias = sc.at<float>(o_b); wa.nbias = cout_pad;
     NVISR_TRY_CUDA(launch_weights(wa, st));
-    {
-        // offsets (18G channels) then mask (9G channels): two packs into one tensor
-        // would split a 4-channel chunk when 18G % 4 != 0, so pack from a joined copy
-        float *joined = sc.at<float>(o_j);
-        NVISR_TRY_CUDA(cudaMemcpyAsync(joined, offsets, (size_t)18 * groups * px * 4, cudaMemcpyDeviceToDevice, st));
-        NVISR_TRY_CUDA(cudaMemcpyAsync(joined + (size_t)18 * groups * px, mask, (size_t)9 * groups * px * 4,
-                                       cudaMemcpyDeviceToDevice, st));
-        NVISR_TRY_CUDA(launch_pack_planar(joined, om_c, om_cpad, h, w, DT_F32, 1.f, dom, 0, st));
-    }
-    // the tensor-core gather reads x in 8-channel planes
-    const int x_cpc = tc ? 8 : layout_cpc(adt, cin_pad), y_cpc = layout_cpc(adt, cout_pad);
-    NVISR_TRY_CUDA(launch_pack_planar(x, cin, cin_pad, h, w, adt, 1.f, dx, x_cpc, st));
+    const int y_cpc = layout_cpc(adt, cout_pad);
+    if (tc) NVISR_TRY_CUDA(launch_dcn_pairs_planar(x, h, w, adt, dx, sc.at<void>(o_xh), st));
+    else NVISR_TRY_CUDA(launch_pack_planar(x, cin, cin_pad, h, w, adt, 1.f, dx, 0, st));
     DcnArgs d{};
     d.x = dx; d.cin_pad = cin_pad; d.H = h; d.W = w; d.groups = groups;
-    d.om = dom; d.om_cpad = om_cpad; d.mask_logits = 0;
+    d.om = offsets; d.om_mask = mask; d.om_cpad = round_up(27 * groups, 4); d.mask_logits = 0;
+    d.x_hi = tc ? sc.at<void>(o_xh) : nullptr;
     d.w = wa.dst; d.bias = wa.dst_bias; d.cout = cout; d.cout_pad = cout_pad; d.y = dy;
     d.in_dt = adt; d.out_dt = adt; d.acc_scale = 1.f; d.out_scale = 1.f; d.err = sc.err();
-    d.x_cpc = x_cpc; d.y_cpc = y_cpc;
+    d.y_cpc = y_cpc;
     cudaError_t e = tc ? launch_dcn_tc(d, st) : launch_dcn_simt(d, st);
     if (e != cudaSuccess) return cuda_status(e, "dcn2d");
     NVISR_TRY_CUDA(launch_unpack_planar(dy, adt, cout_pad, y_cpc, cout, h, w, 1.f, y, st));
