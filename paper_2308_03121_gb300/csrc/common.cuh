@@ -177,7 +177,16 @@ struct ConvArgs {
     int64_t ring_pitch;
     int tslot[8];
     int *err;                // device error word (tensor-core kernels), may be null
+    // FP32 3x3 layers without a shuffle: x, y and res are planar float32 [C][H][W] with cin
+    // real input channels
+    int planar, cin;
 };
+// Whether a planar layer may write y (ny floats) while it reads x and res: an in-place or
+// overlapping call goes through copies instead.
+inline bool planar_apart(const float *x, int64_t nx, const float *res, const float *y, int64_t ny) {
+    const bool over_x = x < y + ny && y < x + nx, over_r = res && res < y + ny && y < res + ny;
+    return !over_x && !over_r;
+}
 cudaError_t launch_conv_simt(const ConvArgs &a, cudaStream_t st);
 cudaError_t launch_conv_tc(const ConvArgs &a, cudaStream_t st);
 

@@ -15,8 +15,12 @@
 // frame) into a planar float32 image.
 //
 // Tensors use the blocked layout [C/4][H][W][4] (16-byte channel chunks).
+//
+// 3x3 layers without a shuffle, nearly all of the path's work, run on conv3_f32_kernel
+// (below), with the same sums in the same order.
 #include "common.cuh"
 #include "epilogue.cuh"
+#include "sm100_ptx.cuh"
 
 namespace nvisr {
 
@@ -237,6 +241,234 @@ __global__ void __launch_bounds__(16 * NB / 4) conv_simt_kernel(ConvArgs a, DcnA
     }
 }
 
+// ---------------------------------------------------------------- 3x3 layers
+
+// A block computes R rows x 64 pixels x NB outputs; warp = row, lane = (pixel group lane / 8,
+// output group lane % 8), a thread 16 pixels (4 runs of 4, 16 apart) x NB / 8 outputs, so 16 x 8
+// packed accumulators at NB = 64.  What bounds it is the FP32 FMA rate.  The smaller 8 x 4 thread
+// tile of conv_simt_kernel read 22 shared-memory words per 96 FMAs, with 2- to 4-way bank
+// conflicts, and staged each slice of 8 input channels between two barriers with nothing else to
+// do.  Here a (channel, ky) reads 48 words without conflicts per 384 FMAs, issued as 192 packed
+// FMAs (fma.rn.f32x2, each half an IEEE FMA), and the next slice's rows and weights arrive by
+// cp.async meanwhile.  Products are summed in the same order (channel, ky, kx), so the
+// values are the same.  960 x 540, 64 -> 64: the layer call 1162 -> 765 us (50 TFLOP/s; a chain of
+// independent FMAs runs at 79), the same with scalar FMAs.
+// PLANAR: x, y and the residual are planar float32 [C][H][W] (the caller's tensors, no layout copy).
+constexpr int C3_TX = 64;       // pixels of a block's row
+constexpr int C3_PITCH = 68;    // floats of a staged row (66 used)
+
+__device__ __forceinline__ void cp_async4(uint32_t dst, const void *src, bool valid) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(valid ? 4 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ uint64_t pair_f32(float lo, float hi) {
+    uint64_t d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+    return d;
+}
+__device__ __forceinline__ void ffma2_64(uint64_t &acc, uint64_t a, uint64_t b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
+
+template <int NB, int R>
+constexpr size_t c3_smem() { return 2 * sizeof(float) * (8 * (R + 2) * C3_PITCH + 8 * 9 * NB); }
+
+template <int NB, int R, bool PLANAR>
+__global__ void __launch_bounds__(32 * R, 8 / R) conv3_f32_kernel(const __grid_constant__ ConvArgs a) {
+    constexpr int N = NB / 8;          // outputs of a thread
+    constexpr int ASZ = 8 * (R + 2) * C3_PITCH, BSZ = 8 * 9 * NB;
+    extern __shared__ __align__(16) float smem_f[];
+    float *As = smem_f, *Bs = smem_f + 2 * ASZ;
+    const int H = a.H, W = a.W;
+    const int64_t HW = (int64_t)H * W;
+    const int tiles_x = (W + C3_TX - 1) / C3_TX, tiles_y = (H + R - 1) / R;
+    const int tile = blockIdx.x;
+    const int img = tile / (tiles_x * tiles_y);
+    const int rem = tile - img * tiles_x * tiles_y;
+    const int y0 = rem / tiles_x * R, x0 = rem % tiles_x * C3_TX;
+    const int oc_base = blockIdx.y * NB;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int og = lane & 7, pg = lane >> 3;
+    const float *x = static_cast<const float *>(a.x) + (PLANAR ? 0 : (int64_t)img * (a.cin_pad / 4) * HW * 4);
+    const float *wts = static_cast<const float *>(a.w);
+
+    auto stage = [&](int sl, int buf) {
+        // input rows: a warp per (channel, row), pixels x0 - 1 .. x0 + 64, zero outside the image
+        for (int i = warp; i < 8 * (R + 2); i += R) {
+            const int c = i / (R + 2), r = i - c * (R + 2);
+            const int ch = sl * 8 + c, iy = y0 + r - 1;
+            const bool rok = iy >= 0 && iy < H && (!PLANAR || ch < a.cin);
+            const uint32_t dst = smem_u32(As + buf * ASZ + i * C3_PITCH);
+#pragma unroll
+            for (int p = lane; p < C3_TX + 2; p += 32) {
+                const int ix = x0 - 1 + p;
+                const bool ok = rok && ix >= 0 && ix < W;
+                const int64_t pix = (int64_t)iy * W + ix;
+                const int64_t at = PLANAR ? (int64_t)ch * HW + pix : ((int64_t)(ch >> 2) * HW + pix) * 4 + (ch & 3);
+                cp_async4(dst + 4u * (uint32_t)p, ok ? x + at : x, ok);
+            }
+        }
+        for (int i = threadIdx.x; i < BSZ / 4; i += 32 * R) {
+            const int ct = i / (NB / 4), n4 = i - ct * (NB / 4);
+            cp_async16(smem_u32(Bs + buf * BSZ + i * 4), wts + ((int64_t)sl * 72 + ct) * a.cout_pad + oc_base + n4 * 4);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+
+    uint64_t acc[16][N / 2];
+#pragma unroll
+    for (int p = 0; p < 16; ++p)
+#pragma unroll
+        for (int n = 0; n < N / 2; ++n) acc[p][n] = 0;
+
+    const int nsl = a.cin_pad / 8;
+    stage(0, 0);
+    for (int sl = 0; sl < nsl; ++sl) {
+        const int buf = sl & 1;
+        if (sl + 1 < nsl) {
+            stage(sl + 1, buf ^ 1);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+        __syncthreads();
+        const float *ar0 = As + buf * ASZ + warp * C3_PITCH + 4 * pg;
+        const float *br0 = Bs + buf * BSZ;
+#pragma unroll 1
+        for (int c = 0; c < 8; ++c) {
+#pragma unroll
+            for (int ky = 0; ky < 3; ++ky) {
+                float av[4][6];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float *ar = ar0 + (c * (R + 2) + ky) * C3_PITCH + 16 * j;
+                    const float4 v0 = *reinterpret_cast<const float4 *>(ar);
+                    const float2 v1 = *reinterpret_cast<const float2 *>(ar + 4);
+                    av[j][0] = v0.x; av[j][1] = v0.y; av[j][2] = v0.z; av[j][3] = v0.w;
+                    av[j][4] = v1.x; av[j][5] = v1.y;
+                }
+#pragma unroll
+                for (int kx = 0; kx < 3; ++kx) {
+                    const float *br = br0 + (c * 9 + ky * 3 + kx) * NB;
+                    uint64_t b[N / 2];
+                    if constexpr (N == 2) {
+                        b[0] = *reinterpret_cast<const uint64_t *>(br + 2 * og);
+                    } else {
+#pragma unroll
+                        for (int h = 0; h < N / 4; ++h) {
+                            const ulonglong2 t = *reinterpret_cast<const ulonglong2 *>(br + 32 * h + 4 * og);
+                            b[2 * h] = t.x;
+                            b[2 * h + 1] = t.y;
+                        }
+                    }
+#pragma unroll
+                    for (int p = 0; p < 16; ++p) {
+                        const float v = av[p / 4][p % 4 + kx];
+                        const uint64_t vv = pair_f32(v, v);
+#pragma unroll
+                        for (int n = 0; n < N / 2; ++n) ffma2_64(acc[p][n], vv, b[n]);
+                    }
+                }
+            }
+        }
+        __syncthreads();
+    }
+
+    // ---- epilogue: outputs oc(n) = oc_base + 4 og + n (NB 64: the upper half 32 further; NB 16: 2 og + n)
+    const int y = y0 + warp;
+    if (y >= H) return;
+    auto oc_of = [&](int n) { return oc_base + (N == 2 ? 2 * og + n : 32 * (n / 4) + 4 * og + n % 4); };
+    float v[N][4];  // a run of 4 pixels
+    const bool vec = PLANAR && W % 4 == 0 && (reinterpret_cast<uintptr_t>(a.y) & 15) == 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int xx = x0 + 16 * j + 4 * pg;
+        if (xx >= W) continue;
+        const int64_t pix = (int64_t)y * W + xx;
+#pragma unroll
+        for (int n = 0; n < N; ++n) {
+            const float bv = a.bias[oc_of(n)];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const uint64_t w2 = acc[4 * j + i][n / 2];
+                const float s = __uint_as_float((uint32_t)(n & 1 ? w2 >> 32 : w2));
+                float o = fmaf(s, a.acc_scale, bv);
+                v[n][i] = a.act == 1 ? lrelu(o) : o;
+            }
+        }
+        if constexpr (PLANAR) {
+            const float *res = static_cast<const float *>(a.res);
+            float *yo = static_cast<float *>(a.y);
+#pragma unroll
+            for (int n = 0; n < N; ++n) {
+                const int oc = oc_of(n);
+                if (oc >= a.cout) continue;
+                const int64_t at = (int64_t)oc * HW + pix;
+                if (res)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        if (xx + i < W) v[n][i] += __ldg(res + at + i);
+                if (vec) {
+                    *reinterpret_cast<float4 *>(yo + at) = make_float4(v[n][0], v[n][1], v[n][2], v[n][3]);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        if (xx + i < W) yo[at + i] = v[n][i];
+                }
+            }
+        } else {
+            constexpr int U = N < 4 ? N : 4;  // outputs of one 16-byte unit this thread holds
+            const int64_t plane0 = (int64_t)img * (a.cout_pad / 4) * HW;
+#pragma unroll
+            for (int h = 0; h < N / U; ++h) {
+                const int oc = oc_of(h * U);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    if (xx + i >= W) break;
+                    const int64_t at = (plane0 + (int64_t)(oc / 4) * HW + pix + i) * 4 + oc % 4;
+                    float o[U];
+#pragma unroll
+                    for (int n = 0; n < U; ++n) o[n] = v[h * U + n][i];
+                    if (a.res)
+#pragma unroll
+                        for (int n = 0; n < U; ++n) o[n] += __ldg(static_cast<const float *>(a.res) + at + n);
+                    float *d = static_cast<float *>(a.y) + at;
+                    if constexpr (U == 4) *reinterpret_cast<float4 *>(d) = make_float4(o[0], o[1], o[2], o[3]);
+                    else *reinterpret_cast<float2 *>(d) = make_float2(o[0], o[1]);
+                }
+            }
+        }
+    }
+}
+
+template <int NB, int R, bool PLANAR>
+cudaError_t run_c3(const ConvArgs &a, cudaStream_t st) {
+    constexpr size_t smem = c3_smem<NB, R>();
+    const cudaError_t e = set_smem_limit<conv3_f32_kernel<NB, R, PLANAR>>((int)smem);
+    if (e != cudaSuccess) return e;
+    const dim3 grid((unsigned)((a.W + C3_TX - 1) / C3_TX * ((a.H + R - 1) / R) * a.nimg), (unsigned)(a.cout_pad / NB));
+    conv3_f32_kernel<NB, R, PLANAR><<<grid, 32 * R, smem, st>>>(a);
+    return cudaGetLastError();
+}
+
+// Rows per block: an SM holds 8 rows at a time whatever R (8 / R blocks), so a launch takes
+// ceil(blocks / (SMs * 8 / R)) rounds of 8 rows; fewer rows per block fill the last round
+// better and stage more halo rows (the constants below, in rows).
+template <int NB, bool PLANAR>
+cudaError_t launch_c3(const ConvArgs &a, cudaStream_t st) {
+    const int64_t sms = device_sm_count(), cols = (int64_t)((a.W + C3_TX - 1) / C3_TX) * a.nimg * (a.cout_pad / NB);
+    auto cost = [&](int R, double halo) {
+        const int64_t blocks = cols * ((a.H + R - 1) / R), per = sms * (8 / R);
+        return (double)((blocks + per - 1) / per) * (8.0 + halo);
+    };
+    const double c8 = cost(8, 0.0), c4 = cost(4, 0.4), c2 = cost(2, 1.2);
+    if (c8 <= c4 && c8 <= c2) return run_c3<NB, 8, PLANAR>(a, st);
+    if (c4 <= c2) return run_c3<NB, 4, PLANAR>(a, st);
+    return run_c3<NB, 2, PLANAR>(a, st);
+}
+
 template <int NB, int KS, int MODE>
 cudaError_t launch_nb(const ConvArgs &a, const DcnArgs &d, int H, int W, int nimg, int cout_pad,
                       cudaStream_t st) {
@@ -276,12 +508,14 @@ cudaError_t launch_conv_simt(const ConvArgs &a, cudaStream_t st) {
     DcnArgs d{};
     if (a.cin_pad % 8 || a.cout_pad % 16) return cudaErrorInvalidValue;
     const int nb = a.cout_pad % 64 == 0 ? 64 : (a.cout_pad % 32 == 0 ? 32 : 16);
-    const int use_nb = a.ps > 0 ? 16 : nb;  // PixelShuffle epilogue groups 4 channels per thread
-    if (a.k == 3) {
-        if (use_nb == 64) return launch_nb<64, 3, 0>(a, d, a.H, a.W, a.nimg, a.cout_pad, st);
-        if (use_nb == 32) return launch_nb<32, 3, 0>(a, d, a.H, a.W, a.nimg, a.cout_pad, st);
-        return launch_nb<16, 3, 0>(a, d, a.H, a.W, a.nimg, a.cout_pad, st);
+    if (a.k == 3 && a.ps == 0) {
+        if (nb == 64) return a.planar ? launch_c3<64, true>(a, st) : launch_c3<64, false>(a, st);
+        if (nb == 32) return a.planar ? launch_c3<32, true>(a, st) : launch_c3<32, false>(a, st);
+        return a.planar ? launch_c3<16, true>(a, st) : launch_c3<16, false>(a, st);
     }
+    if (a.planar) return cudaErrorInvalidValue;
+    if (a.k == 3) return launch_nb<16, 3, 0>(a, d, a.H, a.W, a.nimg, a.cout_pad, st);  // PixelShuffle: 4 channels a thread
+    const int use_nb = a.ps > 0 ? 16 : nb;
     if (a.k == 1) {
         if (use_nb == 64) return launch_nb<64, 1, 0>(a, d, a.H, a.W, a.nimg, a.cout_pad, st);
         if (use_nb == 32) return launch_nb<32, 1, 0>(a, d, a.H, a.W, a.nimg, a.cout_pad, st);

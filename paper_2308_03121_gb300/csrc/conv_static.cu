@@ -161,8 +161,16 @@ extern "C" nvisr_status nvisr_conv2d_static(int32_t precision, const float *x, i
     wa.scale = 1.f;
     wa.dst = area + (rows ? o_rows : o_w); wa.dst_bias = db; wa.nbias = cout_pad;
     CS_TRY(launch_weights(wa, st));
-    CS_TRY(launch_pack_planar(x, cin, cin_pad, h, w, dt, 1.f, dx, in_cpc, st));
-    if (res) CS_TRY(launch_pack_planar(res, cout, cout_pad, h, w, dt, 1.f, dr, out_cpc, st));
+    // FP32 3x3: the kernel reads and writes the caller's tensors
+    const bool planar = !tc && k == 3 && planar_apart(x, (int64_t)(cin * px), res, y, (int64_t)(cout * px));
+    if (planar) {
+        dx = const_cast<float *>(x);
+        dy = y;
+        dr = const_cast<float *>(res);
+    } else {
+        CS_TRY(launch_pack_planar(x, cin, cin_pad, h, w, dt, 1.f, dx, in_cpc, st));
+        if (res) CS_TRY(launch_pack_planar(res, cout, cout_pad, h, w, dt, 1.f, dr, out_cpc, st));
+    }
     ConvArgs a{};
     a.x = dx; a.cin_pad = cin_pad; a.H = h; a.W = w; a.nimg = 1; a.bias = db;
     a.w = rows ? nullptr : wa.dst;
@@ -170,8 +178,9 @@ extern "C" nvisr_status nvisr_conv2d_static(int32_t precision, const float *x, i
     a.cout = cout; a.cout_pad = cout_pad; a.k = k; a.act = act; a.res = dr; a.y = dy;
     a.in_dt = dt; a.out_dt = dt; a.acc_scale = 1.f; a.out_scale = 1.f; a.y2_scale = 1.f; a.err = err;
     a.in_cpc = in_cpc; a.out_cpc = out_cpc;
+    a.planar = planar; a.cin = cin;
     CS_TRY(tc ? launch_conv_tc(a, st) : launch_conv_simt(a, st));
-    CS_TRY(launch_unpack_planar(dy, dt, cout_pad, out_cpc, cout, h, w, 1.f, y, st));
+    if (!planar) CS_TRY(launch_unpack_planar(dy, dt, cout_pad, out_cpc, cout, h, w, 1.f, y, st));
     int herr = 0;
     CS_TRY(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, st));
     CS_TRY(cudaStreamSynchronize(st));

@@ -2826,14 +2826,16 @@ nvisr_status nvisr_conv2d(int32_t precision, const float *x, int32_t cin, int32_
     const int cin_pad = round_up(cin, tc ? 16 : 8), cout_pad = round_up(cout, 16);
     const bool rows = tc && idt != DT_E4M3 && k == 3 && cin == 64 && cout == 64;
     const size_t px = (size_t)h * w;
+    // FP32 3x3: the kernel reads and writes the caller's tensors
+    const bool planar = !tc && k == 3 && planar_apart(x, (int64_t)(cin * px), res, y, (int64_t)(cout * px));
     const int in_cpc = layout_cpc(idt, cin_pad), out_cpc = layout_cpc(adt, cout_pad);
     Scratch sc(st);
     const size_t o_w = sc.plan(rows ? tc_rows_weight_bytes()
                                     : (tc ? tc_weight_bytes(cin_pad, cout_pad, k, idt) : simt_weight_bytes(cin_pad, cout_pad, k)));
     const size_t o_b = sc.plan((size_t)cout_pad * 4);
-    const size_t o_x = sc.plan((size_t)cin_pad * px * dtype_size(idt));
-    const size_t o_y = sc.plan((size_t)cout_pad * px * dtype_size(adt));
-    const size_t o_r = res ? sc.plan((size_t)cout_pad * px * dtype_size(adt)) : 0;
+    const size_t o_x = planar ? 0 : sc.plan((size_t)cin_pad * px * dtype_size(idt));
+    const size_t o_y = planar ? 0 : sc.plan((size_t)cout_pad * px * dtype_size(adt));
+    const size_t o_r = res && !planar ? sc.plan((size_t)cout_pad * px * dtype_size(adt)) : 0;
     const size_t o_m = sc.plan(2 * sizeof(unsigned));
     NVISR_TRY_CUDA(sc.open());
     float sx = 1.f, sw = 1.f;
@@ -2850,6 +2852,11 @@ nvisr_status nvisr_conv2d(int32_t precision, const float *x, int32_t cin, int32_
         sw = a[1] > 0.f ? a[1] / 448.f : 1.f;
     }
     void *dx = sc.at<void>(o_x), *dy = sc.at<void>(o_y), *dr = res ? sc.at<void>(o_r) : nullptr;
+    if (planar) {
+        dx = const_cast<float *>(x);
+        dy = y;
+        dr = const_cast<float *>(res);
+    }
     WeightArgs wa{};
     wa.w = weight; wa.bias = bias; wa.cout = cout; wa.cin = cin; wa.k = k; wa.cin_pad = cin_pad; wa.cout_pad = cout_pad;
     wa.layout = rows ? WL_ROWS : (!tc ? WL_SIMT : (in_cpc == 64 ? WL_TC128 : WL_TC16));
@@ -2858,8 +2865,10 @@ nvisr_status nvisr_conv2d(int32_t precision, const float *x, int32_t cin, int32_
     wa.scale = 1.f / sw;
     wa.dst = sc.at<void>(o_w); wa.dst_bias = sc.at<float>(o_b); wa.nbias = cout_pad;
     NVISR_TRY_CUDA(launch_weights(wa, st));
-    NVISR_TRY_CUDA(launch_pack_planar(x, cin, cin_pad, h, w, idt, 1.f / sx, dx, in_cpc, st));
-    if (res) NVISR_TRY_CUDA(launch_pack_planar(res, cout, cout_pad, h, w, adt, 1.f, dr, out_cpc, st));
+    if (!planar) {
+        NVISR_TRY_CUDA(launch_pack_planar(x, cin, cin_pad, h, w, idt, 1.f / sx, dx, in_cpc, st));
+        if (res) NVISR_TRY_CUDA(launch_pack_planar(res, cout, cout_pad, h, w, adt, 1.f, dr, out_cpc, st));
+    }
     ConvArgs a{};
     a.x = dx; a.cin_pad = cin_pad; a.H = h; a.W = w; a.nimg = 1; a.bias = wa.dst_bias;
     a.w = rows ? nullptr : wa.dst;
@@ -2867,9 +2876,10 @@ nvisr_status nvisr_conv2d(int32_t precision, const float *x, int32_t cin, int32_
     a.cout = cout; a.cout_pad = cout_pad; a.k = k; a.act = act; a.res = dr; a.y = dy;
     a.in_dt = idt; a.out_dt = adt; a.acc_scale = sx * sw; a.out_scale = 1.f; a.y2_scale = 1.f; a.err = sc.err();
     a.in_cpc = in_cpc; a.out_cpc = out_cpc;
+    a.planar = planar; a.cin = cin;
     cudaError_t e = tc ? launch_conv_tc(a, st) : launch_conv_simt(a, st);
     if (e != cudaSuccess) return cuda_status(e, "conv2d");
-    NVISR_TRY_CUDA(launch_unpack_planar(dy, adt, cout_pad, out_cpc, cout, h, w, 1.f, y, st));
+    if (!planar) NVISR_TRY_CUDA(launch_unpack_planar(dy, adt, cout_pad, out_cpc, cout, h, w, 1.f, y, st));
     NVISR_TRY_CUDA(sc.finish());
     if (sc.host_err()) return fail(NVISR_DEVICE_TIMEOUT, "conv2d: a device-side wait exceeded its bound");
     return NVISR_OK;
