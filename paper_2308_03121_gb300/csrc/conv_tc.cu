@@ -199,6 +199,11 @@ __global__ void __launch_bounds__(NTHREADS, 1) conv_tc_kernel(const __grid_const
         mbar_init(drain, 1);
         *abort = 0;
         fence_mbarrier_init();
+        // the weights are not the previous kernel's: they load before the wait below
+        mbar_arrive_expect_tx(wbar, p.wbytes);
+        const uint8_t *wsrc = p.wts + (size_t)slice * p.wbytes;
+        for (uint32_t off = 0; off < p.wbytes; off += 32768u)
+            bulk_load(wsm + off, wsrc + off, min(32768u, p.wbytes - off), wbar);
     }
     if (warp == 1) {
         tmem_alloc(tmem_slot, NCOLS);
@@ -213,13 +218,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) conv_tc_kernel(const __grid_const
 
     if (warp == 0) {
         if (lane == 0) {
-            // ---------------- producer: weights once, then input halos
-            mbar_arrive_expect_tx(wbar, p.wbytes);
-            const uint8_t *wsrc = p.wts + (size_t)slice * p.wbytes;
-            for (uint32_t off = 0; off < p.wbytes; off += 32768u) {
-                const uint32_t n = min(32768u, p.wbytes - off);
-                bulk_load(wsm + off, wsrc + off, n, wbar);
-            }
+            // ---------------- producer: input halos
             int s = 0;
             uint32_t ph = 0;
             int issued = 0;
@@ -257,10 +256,15 @@ __global__ void __launch_bounds__(NTHREADS, 1) conv_tc_kernel(const __grid_const
             mbar_wait_bounded(wbar, 0, nullptr, WAIT_NS);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            // ---------------- MMA issuer
-            bool ok = mbar_wait_bounded(wbar, 0, abort, WAIT_NS);
-            if (!ok) raise_abort(abort, p.err);
+        {
+            // ---------------- MMA issuer: a converged warp, of which the elected lane issues
+            const uint32_t el = elect_one();
+            auto await = [&](uint64_t *bar, uint32_t parity) {
+                const bool w = __all_sync(0xffffffffu, mbar_wait_bounded(bar, parity, abort, WAIT_NS));
+                if (!w && lane == 0) raise_abort(abort, p.err);
+                return w;
+            };
+            bool ok = await(wbar, 0);
             const uint32_t wbase = smem_u32(wsm);
             int s = 0;
             uint32_t ph = 0;
@@ -269,18 +273,11 @@ __global__ void __launch_bounds__(NTHREADS, 1) conv_tc_kernel(const __grid_const
             for (int t = cta0; t < ntiles && ok; t += cta_stride, ++it) {
                 const int a = it & 1;
                 const uint32_t u = (uint32_t)(it >> 1);
-                if (!mbar_wait_bounded(&tempty[a], (u & 1) ^ 1, abort, WAIT_NS)) {
-                    raise_abort(abort, p.err);
-                    break;
-                }
+                if (!await(&tempty[a], (u & 1) ^ 1)) break;
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)(a * NS);
                 for (int g = 0; g < groups; ++g) {
-                    if (!mbar_wait_bounded(&full[s], ph, abort, WAIT_NS)) {
-                        raise_abort(abort, p.err);
-                        ok = false;
-                        break;
-                    }
+                    if (!(ok = await(&full[s], ph))) break;
                     tc_fence_after();
                     // descriptors of tap 0 / K-step 0; others add (byte offset >> 4) to the start field
                     if (CBI == 16) {
@@ -293,7 +290,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) conv_tc_kernel(const __grid_const
                             const uint64_t bt = b0 + (uint64_t)((uint32_t)(tap * p.cin_chunks) * (uint32_t)NS);
 #pragma unroll
                             for (int j = 0; j < NCH / 2; ++j) {
-                                umma<KIND>(d_tmem, at + (uint64_t)(2 * j * (LBO_A >> 4)),
+                                umma_warp<KIND>(el, d_tmem, at + (uint64_t)(2 * j * (LBO_A >> 4)),
                                            bt + (uint64_t)(2 * j * NS), IDESC, (g | tap | j) != 0 ? 1u : 0u);
                             }
                         }
@@ -312,24 +309,24 @@ __global__ void __launch_bounds__(NTHREADS, 1) conv_tc_kernel(const __grid_const
                             for (int c = 0; c < NCH; ++c)
 #pragma unroll
                                 for (int j = 0; j < 4; ++j)
-                                    umma<KIND>(d_tmem, at + (uint64_t)((c * CREG + j * 32) >> 4),
+                                    umma_warp<KIND>(el, d_tmem, at + (uint64_t)((c * CREG + j * 32) >> 4),
                                                bt + (uint64_t)((c * NS * 128 + j * 32) >> 4), IDESC,
                                                (g | tap | c | j) != 0 ? 1u : 0u);
                         }
                     }
-                    umma_commit(&empty[s]);
+                    umma_commit_warp(el, &empty[s]);
                     if (++s == S) { s = 0; ph ^= 1; }
                 }
                 if (!ok) break;
-                umma_commit(&tfull[a]);
+                umma_commit_warp(el, &tfull[a]);
                 last_a = a;
                 last_par = u & 1;
             }
             // drain: MMAs must finish before TMEM is released
             if (last_a >= 0) mbar_wait_bounded(&tfull[last_a], last_par, nullptr, WAIT_NS);
-            if (*abort) {
+            if (__any_sync(0xffffffffu, *abort)) {
                 // an early exit may leave MMAs of an unfinished tile, which no tile commit covers
-                umma_commit(drain);
+                umma_commit_warp(el, drain);
                 mbar_wait_bounded(drain, 0, nullptr, WAIT_NS);
             }
         }
@@ -931,13 +928,18 @@ __global__ void __launch_bounds__(rows_threads(CIN, MULTI), 1) conv_rows_kernel(
             mbar_wait_bounded(wbar, 0, nullptr, WAIT_NS);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            // ---------------- MMA issuer.  Per input row the output rows it touches
+        {
+            // ---------------- MMA issuer: the whole warp runs the loop with uniform values and its
+            // elected lane issues: an MMA then costs its operands' time (N = 16: 39 cycles, 48: 44,
+            // 64: 48, 192: 96), where a lane-0 branch spends 57 or more on each.  The two 2x
+            // tails of the 960 x 540 space-time filter took 177 us so and take 129, its heads and
+            // upsamplers 720 and 669.  Per input row the output rows it touches
             // form at most two contiguous TMEM slot runs (the ring may wrap); the
             // runs' descriptors are computed once per row, then the 12 (kx, K step)
             // MMAs per run only add constant offsets.
-            bool ok = mbar_wait_bounded(wbar, 0, abort, WAIT_NS);
-            if (!ok) raise_abort(abort, p.err);
+            const uint32_t el = elect_one();
+            bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(wbar, 0, abort, WAIT_NS));
+            if (!ok && lane == 0) raise_abort(abort, p.err);
             const uint64_t b_base = SW ? smem_desc_sw128(smem_u32(wsm), 0) : smem_desc(smem_u32(wsm), LBO_B, 128);
             // Work between MMA issues leaves the tensor pipe idle once the few queued
             // MMAs have run, and an mbarrier test made while MMAs are queued costs
@@ -949,11 +951,14 @@ __global__ void __launch_bounds__(rows_threads(CIN, MULTI), 1) conv_rows_kernel(
             uint32_t last_par = 0;
             auto await_row = [&](int row) -> bool {
                 if (row < nready) return true;
-                nready = ld_acquire_cta(ready);
+                // every lane's own acquire; the least count any of them saw is uniform
+                auto poll = [&]() { return (int)__reduce_min_sync(0xffffffffu, (unsigned)ld_acquire_cta(ready)); };
+                nready = poll();
                 if (row >= nready) {
                     const uint64_t t0 = globaltimer_ns();
-                    for (uint32_t it = 1; row >= (nready = ld_acquire_cta(ready)); ++it) {
-                        if ((it & 63) == 0 && (*abort || globaltimer_ns() - t0 > WAIT_NS)) return false;
+                    for (uint32_t it = 1; row >= (nready = poll()); ++it) {
+                        if ((it & 63) == 0 && __any_sync(0xffffffffu, *abort || globaltimer_ns() - t0 > WAIT_NS))
+                            return false;
                     }
                 }
                 tc_fence_after();  // the MMAs of the newly ready rows come after the acquire
@@ -988,12 +993,12 @@ __global__ void __launch_bounds__(rows_threads(CIN, MULTI), 1) conv_rows_kernel(
                         const uint32_t id0 = instr_desc(TM, 0, AFMT, AFMT);
                         const uint32_t nstep = (uint32_t)(NPR / 8) << 17;
                         const uint32_t md = tmem_base + (uint32_t)(sl * NPR);
-                        umma<KIND>(md, a_base, b_base, id0 + nstep * 2u, 1u);
-                        umma<KIND>(md + 2u * NPR, a_base, b_base + (uint64_t)((2 * NPR * (SW ? 128 : 16)) >> 4),
+                        umma_warp<KIND>(el, md, a_base, b_base, id0 + nstep * 2u, 1u);
+                        umma_warp<KIND>(el, md + 2u * NPR, a_base, b_base + (uint64_t)((2 * NPR * (SW ? 128 : 16)) >> 4),
                                    id0 + nstep, 0u);
 #pragma unroll
                         for (int t = 1; t < 3 * KSTEPS; ++t)
-                            umma<KIND>(md, a_base + a_off(t), b_base + b_off(t), id0 + nstep * 3u, 1u);
+                            umma_warp<KIND>(el, md, a_base + a_off(t), b_base + b_off(t), id0 + nstep * 3u, 1u);
                     } else if (o_lo <= o_hi) {
                         const uint64_t a_base = a_desc();
                         // Output rows [o_lo, o_hi] occupy one run of contiguous TMEM slots, or two
@@ -1020,30 +1025,30 @@ __global__ void __launch_bounds__(rows_threads(CIN, MULTI), 1) conv_rows_kernel(
                             const int olen = old_hi - o_lo + 1;
                             if (olen > 0) {
                                 const int f0 = min(olen, m0), f1 = olen - f0;
-                                umma<KIND>(md0, a_base, mb0, id0 + nstep * (uint32_t)f0, 1u);
-                                if (f1 > 0) umma<KIND>(md1, a_base, mb1, id0 + nstep * (uint32_t)f1, 1u);
+                                umma_warp<KIND>(el, md0, a_base, mb0, id0 + nstep * (uint32_t)f0, 1u);
+                                if (f1 > 0) umma_warp<KIND>(el, md1, a_base, mb1, id0 + nstep * (uint32_t)f1, 1u);
                             }
                             if (fresh)
-                                umma<KIND>(tmem_base + (uint32_t)(slot_of(r + 1) * NPR), a_base, bd_of(r + 1),
+                                umma_warp<KIND>(el, tmem_base + (uint32_t)(slot_of(r + 1) * NPR), a_base, bd_of(r + 1),
                                         id0 + nstep, 0u);
                         }
                         if (m1 == 0) {
 #pragma unroll
                             for (int t = 1; t < 3 * KSTEPS; ++t)
-                                umma<KIND>(md0, a_base + a_off(t), mb0 + b_off(t), mi0, 1u);
+                                umma_warp<KIND>(el, md0, a_base + a_off(t), mb0 + b_off(t), mi0, 1u);
                         } else {
 #pragma unroll
                             for (int t = 1; t < 3 * KSTEPS; ++t) {
                                 const uint64_t ad = a_base + a_off(t), boff = b_off(t);
-                                umma<KIND>(md0, ad, mb0 + boff, mi0, 1u);
-                                umma<KIND>(md1, ad, mb1 + boff, mi1, 1u);
+                                umma_warp<KIND>(el, md0, ad, mb0 + boff, mi0, 1u);
+                                umma_warp<KIND>(el, md1, ad, mb1 + boff, mi1, 1u);
                             }
                         }
                     }
-                    umma_commit(&empty[s]);
+                    umma_commit_warp(el, &empty[s]);
                     if (r - 1 >= ra) {
                         const int i = base + r - 1;
-                        umma_commit(&rowdone[i & (NSLOT - 1)]);
+                        umma_commit_warp(el, &rowdone[i & (NSLOT - 1)]);
                         last_slot = i & (NSLOT - 1);
                         last_par = (uint32_t)((i >> 3) & 1);
                     }
@@ -1066,18 +1071,18 @@ __global__ void __launch_bounds__(rows_threads(CIN, MULTI), 1) conv_rows_kernel(
                 constexpr uint32_t BROW = NPR * (SW ? 128 : 16);  // B bytes of one output row's taps
                 const uint32_t md0 = tmem_base + (uint32_t)(SL0 * NPR), md1 = tmem_base;
                 const uint64_t mb0 = b_base, mb1 = b_base + (uint64_t)((M0 * BROW) >> 4);
-                umma<KIND>(md0, a_base, mb0, ID0 + NST * F0, 1u);
-                if constexpr (F1 > 0) umma<KIND>(md1, a_base, mb1, ID0 + NST * F1, 1u);
-                umma<KIND>(tmem_base + (uint32_t)(((SL0 + 2) & (NSLOT - 1)) * NPR), a_base,
+                umma_warp<KIND>(el, md0, a_base, mb0, ID0 + NST * F0, 1u);
+                if constexpr (F1 > 0) umma_warp<KIND>(el, md1, a_base, mb1, ID0 + NST * F1, 1u);
+                umma_warp<KIND>(el, tmem_base + (uint32_t)(((SL0 + 2) & (NSLOT - 1)) * NPR), a_base,
                         b_base + (uint64_t)((2 * BROW) >> 4), ID0 + NST, 0u);
 #pragma unroll
                 for (int t = 1; t < 3 * KSTEPS; ++t) {
                     const uint64_t ad = a_base + a_off(t), boff = b_off(t);
-                    umma<KIND>(md0, ad, mb0 + boff, MI0, 1u);
-                    if constexpr (M1 > 0) umma<KIND>(md1, ad, mb1 + boff, MI1, 1u);
+                    umma_warp<KIND>(el, md0, ad, mb0 + boff, MI0, 1u);
+                    if constexpr (M1 > 0) umma_warp<KIND>(el, md1, ad, mb1 + boff, MI1, 1u);
                 }
-                umma_commit(&empty[s]);
-                umma_commit(&rowdone[SL0]);
+                umma_commit_warp(el, &empty[s]);
+                umma_commit_warp(el, &rowdone[SL0]);
                 last_slot = SL0;
                 last_par = par;
                 if (++s == S) s = 0;
@@ -1111,13 +1116,13 @@ __global__ void __launch_bounds__(rows_threads(CIN, MULTI), 1) conv_rows_kernel(
                         ++r;
                     }
                 }
-                if (!ok) raise_abort(abort, p.err);
+                if (!ok && lane == 0) raise_abort(abort, p.err);
                 gout += rb - ra;
             }
             if (last_slot >= 0) mbar_wait_bounded(&rowdone[last_slot], last_par, nullptr, WAIT_NS);
-            if (*abort) {
+            if (__any_sync(0xffffffffu, *abort)) {
                 // an early exit may leave MMAs of a strip's first row, which no row commit covers
-                umma_commit(drain);
+                umma_commit_warp(el, drain);
                 mbar_wait_bounded(drain, 0, nullptr, WAIT_NS);
             }
         }
