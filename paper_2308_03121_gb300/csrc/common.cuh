@@ -152,6 +152,9 @@ struct ConvArgs {
     int act;                 // 0 none, 1 LeakyReLU(0.1)
     const void *res;         // blocked residual, same layout/dtype as y, or nullptr
     void *y;                 // blocked output [cout_pad/cpc][H][W][cpc]
+    // 64 -> 64 row-kernel layers and the second conv of a residual block: write planar float32
+    // [64][H][W] (values rounded to out_dt) instead of y
+    float *y_planar;
     int in_dt, out_dt;       // dtypes of x and of y/res
     float acc_scale;         // multiplies the accumulator (FP8 dequant), 1 otherwise
     float out_scale;         // multiplies the stored value (FP8 quant of y), 1 otherwise

@@ -179,8 +179,9 @@ extern "C" nvisr_status nvisr_conv2d_static(int32_t precision, const float *x, i
     a.in_dt = dt; a.out_dt = dt; a.acc_scale = 1.f; a.out_scale = 1.f; a.y2_scale = 1.f; a.err = err;
     a.in_cpc = in_cpc; a.out_cpc = out_cpc;
     a.planar = planar; a.cin = cin;
+    if (rows) a.y_planar = y;  // x and res are copies by now
     CS_TRY(tc ? launch_conv_tc(a, st) : launch_conv_simt(a, st));
-    if (!planar) CS_TRY(launch_unpack_planar(dy, dt, cout_pad, out_cpc, cout, h, w, 1.f, y, st));
+    if (!planar && !rows) CS_TRY(launch_unpack_planar(dy, dt, cout_pad, out_cpc, cout, h, w, 1.f, y, st));
     int herr = 0;
     CS_TRY(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, st));
     CS_TRY(cudaStreamSynchronize(st));

@@ -2834,7 +2834,7 @@ nvisr_status nvisr_conv2d(int32_t precision, const float *x, int32_t cin, int32_
                                     : (tc ? tc_weight_bytes(cin_pad, cout_pad, k, idt) : simt_weight_bytes(cin_pad, cout_pad, k)));
     const size_t o_b = sc.plan((size_t)cout_pad * 4);
     const size_t o_x = planar ? 0 : sc.plan((size_t)cin_pad * px * dtype_size(idt));
-    const size_t o_y = planar ? 0 : sc.plan((size_t)cout_pad * px * dtype_size(adt));
+    const size_t o_y = planar || rows ? 0 : sc.plan((size_t)cout_pad * px * dtype_size(adt));
     const size_t o_r = res && !planar ? sc.plan((size_t)cout_pad * px * dtype_size(adt)) : 0;
     const size_t o_m = sc.plan(2 * sizeof(unsigned));
     NVISR_TRY_CUDA(sc.open());
@@ -2877,9 +2877,13 @@ nvisr_status nvisr_conv2d(int32_t precision, const float *x, int32_t cin, int32_
     a.in_dt = idt; a.out_dt = adt; a.acc_scale = sx * sw; a.out_scale = 1.f; a.y2_scale = 1.f; a.err = sc.err();
     a.in_cpc = in_cpc; a.out_cpc = out_cpc;
     a.planar = planar; a.cin = cin;
+    if (rows) {
+        a.y_planar = y;  // x and res are copies by now
+        a.y = dx;        // (only its address is used)
+    }
     cudaError_t e = tc ? launch_conv_tc(a, st) : launch_conv_simt(a, st);
     if (e != cudaSuccess) return cuda_status(e, "conv2d");
-    if (!planar) NVISR_TRY_CUDA(launch_unpack_planar(dy, adt, cout_pad, out_cpc, cout, h, w, 1.f, y, st));
+    if (!planar && !rows) NVISR_TRY_CUDA(launch_unpack_planar(dy, adt, cout_pad, out_cpc, cout, h, w, 1.f, y, st));
     NVISR_TRY_CUDA(sc.finish());
     if (sc.host_err()) return fail(NVISR_DEVICE_TIMEOUT, "conv2d: a device-side wait exceeded its bound");
     return NVISR_OK;
@@ -2899,11 +2903,11 @@ nvisr_status nvisr_resblock2d(int32_t precision, const float *x, int32_t h, int3
     const size_t abytes = plane * 2;
     const size_t o_w1 = sc.plan(tc_rows_weight_bytes()), o_w2 = sc.plan(tc_rows_weight_bytes());
     const size_t o_b1 = sc.plan(64 * 4), o_b2 = sc.plan(64 * 4);
-    const size_t o_x = sc.plan(abytes), o_y = sc.plan(abytes);
+    const size_t o_x = sc.plan(abytes);
     // the middle tensor's room: the fused form never writes it, but plans with its address
     const size_t o_h = sc.plan(fused ? 256 : abytes);
     NVISR_TRY_CUDA(sc.open());
-    void *dx = sc.at<void>(o_x), *dy = sc.at<void>(o_y), *dh = sc.at<void>(o_h);
+    void *dx = sc.at<void>(o_x), *dh = sc.at<void>(o_h);
     for (int c = 0; c < 2; ++c) {
         WeightArgs wa{};
         wa.w = c ? w2 : w1; wa.bias = c ? b2 : b1;
@@ -2919,7 +2923,8 @@ nvisr_status nvisr_resblock2d(int32_t precision, const float *x, int32_t h, int3
     a1.y = dh; a1.in_dt = dt; a1.out_dt = dt; a1.acc_scale = 1.f; a1.out_scale = 1.f; a1.y2_scale = 1.f;
     a1.err = sc.err();
     ConvArgs a2 = a1;
-    a2.x = dh; a2.w_rows = sc.at<void>(o_w2); a2.bias = sc.at<float>(o_b2); a2.act = 0; a2.res = dx; a2.y = dy;
+    a2.x = dh; a2.w_rows = sc.at<void>(o_w2); a2.bias = sc.at<float>(o_b2); a2.act = 0; a2.res = dx;
+    a2.y_planar = y;  // and a2.y, of which only the address is used, stays the middle tensor's
     cudaError_t e;
     if (fused) {
         if (!res_block_fits(a1, a2)) return fail(NVISR_UNSUPPORTED_FORMAT, "resblock2d: no fused form for these buffers");
@@ -2929,7 +2934,6 @@ nvisr_status nvisr_resblock2d(int32_t precision, const float *x, int32_t h, int3
         if (e == cudaSuccess) e = launch_conv_tc(a2, st);
     }
     if (e != cudaSuccess) return cuda_status(e, "resblock2d");
-    NVISR_TRY_CUDA(launch_unpack_planar(dy, dt, 64, 64, 64, h, w, 1.f, y, st));
     NVISR_TRY_CUDA(sc.finish());
     if (sc.host_err()) return fail(NVISR_DEVICE_TIMEOUT, "resblock2d: a device-side wait exceeded its bound");
     return NVISR_OK;

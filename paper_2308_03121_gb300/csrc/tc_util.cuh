@@ -74,5 +74,12 @@ __device__ __forceinline__ uint32_t pack2<__half>(float lo, float hi) {
     return *reinterpret_cast<const uint32_t *>(&h);
 }
 
+// A pair of floats rounded to the 16-bit type and back.
+template <typename T>
+__device__ __forceinline__ void round2(float &a, float &b) {
+    const uint32_t w = pack2<T>(a, b);
+    unpack2<T>(w, a, b);
+}
+
 }  // namespace
 }  // namespace nvisr
