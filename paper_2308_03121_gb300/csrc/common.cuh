@@ -155,6 +155,9 @@ struct ConvArgs {
     // 64 -> 64 row-kernel layers and the second conv of a residual block: write planar float32
     // [64][H][W] (values rounded to out_dt) instead of y
     float *y_planar;
+    // with y_planar, row kernel: the residual as planar float32 (rounded to out_dt on reading);
+    // apart from y_planar or equal to it
+    const float *res_planar;
     int in_dt, out_dt;       // dtypes of x and of y/res
     float acc_scale;         // multiplies the accumulator (FP8 dequant), 1 otherwise
     float out_scale;         // multiplies the stored value (FP8 quant of y), 1 otherwise
@@ -189,6 +192,11 @@ struct ConvArgs {
 inline bool planar_apart(const float *x, int64_t nx, const float *res, const float *y, int64_t ny) {
     const bool over_x = x < y + ny && y < x + nx, over_r = res && res < y + ny && y < res + ny;
     return !over_x && !over_r;
+}
+// True when a row-kernel layer writing y_planar may read its residual where it is: each thread
+// reads its elements before it writes them.
+inline bool residual_in_place(const float *res, const float *y, int64_t ny) {
+    return res == y || planar_apart(res, ny, nullptr, y, ny);
 }
 cudaError_t launch_conv_simt(const ConvArgs &a, cudaStream_t st);
 cudaError_t launch_conv_tc(const ConvArgs &a, cudaStream_t st);

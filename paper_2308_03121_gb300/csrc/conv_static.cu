@@ -163,13 +163,15 @@ extern "C" nvisr_status nvisr_conv2d_static(int32_t precision, const float *x, i
     CS_TRY(launch_weights(wa, st));
     // FP32 3x3: the kernel reads and writes the caller's tensors
     const bool planar = !tc && k == 3 && planar_apart(x, (int64_t)(cin * px), res, y, (int64_t)(cout * px));
+    const bool res_there = rows && residual_in_place(res, y, (int64_t)(cout * px));
+    if (res_there) dr = nullptr;
     if (planar) {
         dx = const_cast<float *>(x);
         dy = y;
         dr = const_cast<float *>(res);
     } else {
         CS_TRY(launch_pack_planar(x, cin, cin_pad, h, w, dt, 1.f, dx, in_cpc, st));
-        if (res) CS_TRY(launch_pack_planar(res, cout, cout_pad, h, w, dt, 1.f, dr, out_cpc, st));
+        if (res && !res_there) CS_TRY(launch_pack_planar(res, cout, cout_pad, h, w, dt, 1.f, dr, out_cpc, st));
     }
     ConvArgs a{};
     a.x = dx; a.cin_pad = cin_pad; a.H = h; a.W = w; a.nimg = 1; a.bias = db;
@@ -179,7 +181,10 @@ extern "C" nvisr_status nvisr_conv2d_static(int32_t precision, const float *x, i
     a.in_dt = dt; a.out_dt = dt; a.acc_scale = 1.f; a.out_scale = 1.f; a.y2_scale = 1.f; a.err = err;
     a.in_cpc = in_cpc; a.out_cpc = out_cpc;
     a.planar = planar; a.cin = cin;
-    if (rows) a.y_planar = y;  // x and res are copies by now
+    if (rows) {
+        a.y_planar = y;  // x is a copy by now
+        if (res_there) a.res_planar = res;
+    }
     CS_TRY(tc ? launch_conv_tc(a, st) : launch_conv_simt(a, st));
     if (!planar && !rows) CS_TRY(launch_unpack_planar(dy, dt, cout_pad, out_cpc, cout, h, w, 1.f, y, st));
     int herr = 0;

@@ -81,6 +81,7 @@ struct TcParams {
     unsigned *amax;
     // final PixelShuffle + skip
     float *y_planar;                  // row kernel, PLNO: planar float32 output [64][H][W]
+    const float *res_planar;          //   and residual (or null)
     float *ps_out;
     int64_t ps_pitch;
     ConvArgs skip;  // skip_* fields only
@@ -611,7 +612,8 @@ struct RowPlan {
 
 // PLNO (64 -> 64 layers): the output goes to planar float32, rounded to the 16-bit type, straight
 // from the registers (128 contiguous bytes per warp and channel), which saves a layout pass over
-// the output (853 x 479 layer call with a residual 165 -> 134 us, 320 x 180 52 -> 42).
+// the output (853 x 479 layer call with a residual 165 -> 134 us, 320 x 180 52 -> 42).  Its residual may
+// be planar float32 too, read a row ahead of the accumulator's arrival (134 -> 120 us: no copy of it).
 template <int IN_DT, int OUT_DT, int CBO, bool MULTI, int NPR, bool PS, int CIN, bool PLNO = false>
 __global__ void __launch_bounds__(rows_threads(CIN, MULTI), 1) conv_rows_kernel(const __grid_constant__ CUtensorMap tmap,
                                                                 const __grid_constant__ CUtensorMap ymap,
@@ -1209,6 +1211,14 @@ __global__ void __launch_bounds__(rows_threads(CIN, MULTI), 1) conv_rows_kernel(
                         const int Wl = width_of(pi);
                         rq_skip_load(p.rq, o, min(x, Wl - 1), p.H, Wl, lr);
                     }
+                // a planar residual row, rounded as a blocked one, loaded before the row's wait
+                uint32_t pr[PLNO ? 32 : 1];
+                if constexpr (PLNO)
+                    if (p.res_planar && valid) {
+                        const float *ro = p.res_planar + (int64_t)o * p.W + x;
+#pragma unroll
+                        for (int e = 0; e < 32; ++e) pr[e] = pack2<TO>(ro[(int64_t)(2 * e) * HW], ro[(int64_t)(2 * e + 1) * HW]);
+                    }
                 named_barrier(bar_id, NGRP);
                 bool w = mbar_wait_bounded(&rowdone[slot], (uint32_t)((i / NSLOT) & 1), abort, WAIT_NS);
                 w = __all_sync(0xffffffffu, w);
@@ -1481,6 +1491,11 @@ __global__ void __launch_bounds__(rows_threads(CIN, MULTI), 1) conv_rows_kernel(
                         float *yo = p.y_planar + (int64_t)o * p.W + x;
 #pragma unroll
                         for (int e = 0; e < 64; e += 2) {
+                            if (p.res_planar) {
+                                float r0, r1;
+                                unpack2<TO>(pr[e / 2], r0, r1);
+                                add_f32x2(v[e], v[e + 1], r0, r1);
+                            }
                             round2<TO>(v[e], v[e + 1]);
                             yo[(int64_t)e * HW] = v[e];
                             yo[(int64_t)(e + 1) * HW] = v[e + 1];
@@ -2050,6 +2065,7 @@ TcParams rows_params(const ConvArgs &a) {
     p.y2 = static_cast<uint8_t *>(a.y2); p.y2_scale = a.y2_scale; p.amax = a.amax;
     p.err = a.err;
     p.y_planar = a.y_planar;
+    p.res_planar = a.res_planar;
     p.starve = test_starve();
     return p;
 }
@@ -2149,7 +2165,7 @@ cudaError_t launch_conv_tc(const ConvArgs &a, cudaStream_t st) {
         if (e != cudaSuccess) return e;
         const TcParams p = rows_params(a);
         if (a.y_planar) {
-            if (a.nimg != 1 || a.y2 || a.amax) return cudaErrorInvalidValue;
+            if (a.nimg != 1 || a.y2 || a.amax || a.acc_scale != 1.f || a.out_scale != 1.f) return cudaErrorInvalidValue;
             return dt == DT_BF16 ? run_rows<DT_BF16, DT_BF16, 128, 64, false, 64, true>(map, ymap, rmap, p, st)
                                  : run_rows<DT_F16, DT_F16, 128, 64, false, 64, true>(map, ymap, rmap, p, st);
         }

@@ -2835,7 +2835,8 @@ nvisr_status nvisr_conv2d(int32_t precision, const float *x, int32_t cin, int32_
     const size_t o_b = sc.plan((size_t)cout_pad * 4);
     const size_t o_x = planar ? 0 : sc.plan((size_t)cin_pad * px * dtype_size(idt));
     const size_t o_y = planar || rows ? 0 : sc.plan((size_t)cout_pad * px * dtype_size(adt));
-    const size_t o_r = res && !planar ? sc.plan((size_t)cout_pad * px * dtype_size(adt)) : 0;
+    const bool res_there = planar || (rows && residual_in_place(res, y, (int64_t)(cout * px)));
+    const size_t o_r = res && !res_there ? sc.plan((size_t)cout_pad * px * dtype_size(adt)) : 0;
     const size_t o_m = sc.plan(2 * sizeof(unsigned));
     NVISR_TRY_CUDA(sc.open());
     float sx = 1.f, sw = 1.f;
@@ -2851,7 +2852,7 @@ nvisr_status nvisr_conv2d(int32_t precision, const float *x, int32_t cin, int32_
         sx = a[0] > 0.f ? a[0] / 448.f : 1.f;
         sw = a[1] > 0.f ? a[1] / 448.f : 1.f;
     }
-    void *dx = sc.at<void>(o_x), *dy = sc.at<void>(o_y), *dr = res ? sc.at<void>(o_r) : nullptr;
+    void *dx = sc.at<void>(o_x), *dy = sc.at<void>(o_y), *dr = res && !res_there ? sc.at<void>(o_r) : nullptr;
     if (planar) {
         dx = const_cast<float *>(x);
         dy = y;
@@ -2867,7 +2868,7 @@ nvisr_status nvisr_conv2d(int32_t precision, const float *x, int32_t cin, int32_
     NVISR_TRY_CUDA(launch_weights(wa, st));
     if (!planar) {
         NVISR_TRY_CUDA(launch_pack_planar(x, cin, cin_pad, h, w, idt, 1.f / sx, dx, in_cpc, st));
-        if (res) NVISR_TRY_CUDA(launch_pack_planar(res, cout, cout_pad, h, w, adt, 1.f, dr, out_cpc, st));
+        if (res && !res_there) NVISR_TRY_CUDA(launch_pack_planar(res, cout, cout_pad, h, w, adt, 1.f, dr, out_cpc, st));
     }
     ConvArgs a{};
     a.x = dx; a.cin_pad = cin_pad; a.H = h; a.W = w; a.nimg = 1; a.bias = wa.dst_bias;
@@ -2878,7 +2879,8 @@ nvisr_status nvisr_conv2d(int32_t precision, const float *x, int32_t cin, int32_
     a.in_cpc = in_cpc; a.out_cpc = out_cpc;
     a.planar = planar; a.cin = cin;
     if (rows) {
-        a.y_planar = y;  // x and res are copies by now
+        a.y_planar = y;  // x is a copy by now
+        if (res_there) a.res_planar = res;
         a.y = dx;        // (only its address is used)
     }
     cudaError_t e = tc ? launch_conv_tc(a, st) : launch_conv_simt(a, st);
