@@ -7,7 +7,7 @@
 //     y[o,p] = b[o] + sum_{c,k} w[o,c,k] * m[g,k](p) * bilinear(x_c, p + p_k + d[g,k](p))
 // with out-of-image bilinear corners contributing zero.
 //
-// Kernel: one CTA per SM walks 128-pixel row tiles.  For each tile and tap, sixteen producer
+// Kernel: one CTA per SM walks tiles of 32 x 4 pixels.  For each tile and tap, sixteen producer
 // warps (a warp per 8-channel chunk and half tile, a lane per pixel) read the tap's offsets and
 // mask, issue the bilinear corner loads of all their pixels before using any (so many gathers
 // are in flight at once), blend them in FP32 with the mask folded into the row weights, and
@@ -30,6 +30,12 @@ namespace nvisr {
 namespace {
 
 constexpr int TM = 128;
+// A tile's pixels: TY rows of TX.  The nine taps of neighbouring pixels read the same input, and a
+// tile of several rows keeps that window small enough for L1: with random offsets (sigma 2) the
+// 960 x 540 call takes 494, 460, 444, 446 and 463 us with rows of 128, 64, 32, 16 and 8 pixels,
+// with zero offsets 393, 377, 378, 385 and 390, and the space-time filter's two layers 684, 650, 652,
+// 668 and 685.  32 also leaves a warp's offset loads whole 128-byte lines.
+constexpr int TX = 32, TY = TM / TX;
 constexpr int NGATHER = 512;            // gather threads (a lane per pixel and chunk, two passes)
 constexpr int MMA_WARP = NGATHER / 32;  // then 4 epilogue warps, the first also loads the weights and issues the MMAs
 constexpr int NT = NGATHER + 128;       // 20 warps: 5 per SM sub-partition leaves 96 registers a thread
@@ -38,7 +44,7 @@ constexpr int SMEM_LIMIT = 232448;
 // Stages of sampled taps.  Shared memory beyond 164 KB would shrink L1, which needs a line for every
 // corner load in flight: at 960 x 540 with independent offsets of sigma 2 px a whole nvisr_dcn2d
 // call takes 492 us with 5 stages (92 KB of L1) and 798 us with 8 (28 KB); the space-time filter's
-// layer with its input copy 340 against 400 us.
+// layer with its input copy 340 against 400 us (both with one-row tiles).
 constexpr int MAX_STAGES = 5;
 
 template <typename T>
@@ -129,8 +135,8 @@ __global__ void __launch_bounds__(NT, 1) dcn_tc_kernel(const DcnArgs a, int stag
     // blocked layouts [C/cpc][H][W][cpc]: byte address of the 8-channel unit starting at channel c
     const int ycpc = a.y_cpc;
     const int64_t HW = (int64_t)H * W;
-    const int tiles_x = (W + TM - 1) / TM;
-    const int ntiles = tiles_x * H;
+    const int tiles_x = (W + TX - 1) / TX;
+    const int ntiles = tiles_x * ((H + TY - 1) / TY);
     const int S = stages;
 
     if (threadIdx.x == 0) {
@@ -193,8 +199,8 @@ __global__ void __launch_bounds__(NT, 1) dcn_tc_kernel(const DcnArgs a, int stag
         // offsets and mask of this lane's pixels for tap k of tile t: loaded one tap ahead of
         // their use, so that their DRAM latency overlaps the previous tap
         auto load_om = [&](int t, int k, float2 (&d)[NPASS], float (&lg)[NPASS]) {
-            const int y = t / tiles_x;
-            const int xb = (t - y * tiles_x) * TM;
+            const int ty = t / tiles_x;
+            const int yt = ty * TY, xt = (t - ty * tiles_x) * TX;
             // float offsets in 32 bits (the tensors are < 2^31 floats)
             uint32_t od, oms;
             if (PLANAR) {
@@ -207,7 +213,7 @@ __global__ void __launch_bounds__(NT, 1) dcn_tc_kernel(const DcnArgs a, int stag
             }
 #pragma unroll
             for (int h = 0; h < NPASS; ++h) {
-                const uint32_t pix = (uint32_t)(y * W + min(xb + pb + 32 * h, W - 1));
+                const uint32_t pix = (uint32_t)(min(yt + (pb + 32 * h) / TX, H - 1) * W + min(xt + (pb + 32 * h) % TX, W - 1));
                 if (PLANAR) {
                     d[h] = make_float2(__ldg(a.om + od + pix), __ldg(a.om + od + (uint32_t)HW + pix));
                     lg[h] = __ldg(a.om_mask + oms + pix);
@@ -221,8 +227,8 @@ __global__ void __launch_bounds__(NT, 1) dcn_tc_kernel(const DcnArgs a, int stag
         float nlg[NPASS];
         if (blockIdx.x < ntiles && !a.starve) load_om(blockIdx.x, 0, nd, nlg);
         for (int t = blockIdx.x; t < ntiles && ok && !a.starve; t += gridDim.x) {
-            const int y = t / tiles_x;
-            const int xb = (t - y * tiles_x) * TM;
+            const int ty = t / tiles_x;
+            const int yt = ty * TY, xt = (t - ty * tiles_x) * TX;
             for (int k = 0; k < 9; ++k) {
                 float2 cd[NPASS];
                 float clg[NPASS];
@@ -238,17 +244,17 @@ __global__ void __launch_bounds__(NT, 1) dcn_tc_kernel(const DcnArgs a, int stag
                 float wy[NPASS][2], wxa[NPASS], wxb[NPASS];
 #pragma unroll
                 for (int h = 0; h < NPASS; ++h) {
-                    const int px = xb + pb + 32 * h;
+                    const int px = xt + (pb + 32 * h) % TX, py = yt + (pb + 32 * h) / TX;
                     // mask = sigmoid(logit) with the fast exponential and division: a relative
                     // error near 1e-6, far below the 16-bit rounding of the sample it scales
                     // (0 and 1 at the extremes); the exact form cost 4 % of the launch
                     const float m = a.mask_logits ? __fdividef(1.f, 1.f + __expf(-clg[h])) : clg[h];
-                    const float sy = (float)(y + k / 3 - 1) + cd[h].x;
+                    const float sy = (float)(py + k / 3 - 1) + cd[h].x;
                     const float sx = (float)(px + k % 3 - 1) + cd[h].y;
                     const float fy = floorf(sy), fx = floorf(sx);
                     const int y0 = (int)fy, x0 = (int)fx;
                     const float ly = sy - fy, lx = sx - fx;
-                    const bool in = px < W;
+                    const bool in = px < W && py < H;
                     wy[h][0] = in && (unsigned)y0 < (unsigned)H ? (1.f - ly) * m : 0.f;
                     wy[h][1] = in && (unsigned)(y0 + 1) < (unsigned)H ? ly * m : 0.f;
                     const float wx0 = (unsigned)x0 < (unsigned)W ? 1.f - lx : 0.f;
@@ -369,15 +375,16 @@ __global__ void __launch_bounds__(NT, 1) dcn_tc_kernel(const DcnArgs a, int stag
                 return false;
             }
             tc_fence_after();
-            const int y = t / tiles_x;
-            const int xx = (t - y * tiles_x) * TM + m;
-            const int64_t pix = (int64_t)y * W + xx;
+            const int ty = t / tiles_x;
+            const int yy = ty * TY + m / TX, xx = (t - ty * tiles_x) * TX + m % TX;
+            const bool inside = yy < H && xx < W;
+            const int64_t pix = (int64_t)yy * W + xx;
             const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(ab * NS);
 #pragma unroll
             for (int j = 0; j < NS / 16; ++j) {
                 float v[16];
                 tmem_ld16(taddr + (uint32_t)(j * 16), v);
-                if (xx >= W) continue;
+                if (!inside) continue;
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     alignas(16) T o[CPC];
@@ -434,7 +441,7 @@ cudaError_t run(const DcnArgs &a, cudaStream_t st) {
     auto kern = dcn_tc_kernel<T, NS, C, PLANAR>;
     cudaError_t e = set_smem_limit<dcn_tc_kernel<T, NS, C, PLANAR>>(smem);
     if (e != cudaSuccess) return e;
-    const int tiles = ((a.W + TM - 1) / TM) * a.H;
+    const int tiles = ((a.W + TX - 1) / TX) * ((a.H + TY - 1) / TY);
     int grid = device_sm_count();
     if (grid > tiles) grid = tiles;
     return launch_dependent(kern, grid, NT, smem, st, a, stages);
@@ -442,7 +449,8 @@ cudaError_t run(const DcnArgs &a, cudaStream_t st) {
 
 // One thread per (pixel, 8-channel chunk), chunk fastest: a warp reads four pixels' 128-byte
 // channel lines (and their right neighbours, which L1 holds) and writes four 32-byte entries of
-// eight planes, 128 contiguous bytes each.
+// eight planes, 128 contiguous bytes each, with one 32-byte store a lane (two 16-byte stores wrote each
+// sector in halves: 7 us more at 960 x 540).
 __global__ void __launch_bounds__(256) dcn_pairs_kernel(const uint4 *__restrict__ x, int64_t HW, int W, int per,
                                                         uint4 *__restrict__ lo, uint4 *__restrict__ hi) {
     const int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -453,9 +461,7 @@ __global__ void __launch_bounds__(256) dcn_pairs_kernel(const uint4 *__restrict_
     const bool last = (int)(p % W) == W - 1;
     const uint4 v0 = __ldg(src);
     const uint4 v1 = last ? make_uint4(0u, 0u, 0u, 0u) : __ldg(src + per);
-    uint4 *d = (cc < 4 ? lo : hi) + ((int64_t)(cc & 3) * HW + p) * 2;
-    d[0] = v0;
-    d[1] = v1;
+    st_global_v8((cc < 4 ? lo : hi) + ((int64_t)(cc & 3) * HW + p) * 2, v0, v1);
 }
 
 // The same from planar float32: one lane per pixel, blockIdx.y the chunk; a lane's right
@@ -482,9 +488,7 @@ __global__ void __launch_bounds__(256) dcn_pairs_planar_kernel(const float *__re
     if ((threadIdx.x & 31) == 31) v1 = load(p + 1);
     if (p >= HW) return;
     if ((int)(p % W) == W - 1) v1 = make_uint4(0u, 0u, 0u, 0u);
-    uint4 *d = (cc < 4 ? lo : hi) + ((int64_t)(cc & 3) * HW + p) * 2;
-    d[0] = v0;
-    d[1] = v1;
+    st_global_v8((cc < 4 ? lo : hi) + ((int64_t)(cc & 3) * HW + p) * 2, v0, v1);
 }
 
 }  // namespace
