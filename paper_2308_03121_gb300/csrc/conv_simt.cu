@@ -243,18 +243,24 @@ __global__ void __launch_bounds__(16 * NB / 4) conv_simt_kernel(ConvArgs a, DcnA
 
 // ---------------------------------------------------------------- 3x3 layers
 
-// A block computes R rows x 64 pixels x NB outputs; warp = row, lane = (pixel group lane / 8,
-// output group lane % 8), a thread 16 pixels (4 runs of 4, 16 apart) x NB / 8 outputs, so 16 x 8
-// packed accumulators at NB = 64.  What bounds it is the FP32 FMA rate.  The smaller 8 x 4 thread
-// tile of conv_simt_kernel read 22 shared-memory words per 96 FMAs, with 2- to 4-way bank
-// conflicts, and staged each slice of 8 input channels between two barriers with nothing else to
-// do.  Here a (channel, ky) reads 48 words without conflicts per 384 FMAs, issued as 192 packed
-// FMAs (fma.rn.f32x2, each half an IEEE FMA), and the next slice's rows and weights arrive by
-// cp.async meanwhile.  Products are summed in the same order (channel, ky, kx), so the
-// values are the same.  960 x 540, 64 -> 64: the layer call 1162 -> 765 us (50 TFLOP/s; a chain of
-// independent FMAs runs at 79), the same with scalar FMAs.
+// A block computes 2 rows x 64 pixels x NB outputs; warp = (row, 32 pixels), lane = (pixel group
+// lane / 8, output group lane % 8), a thread 8 pixels (2 runs of 4, 16 apart) x NB / 8 outputs, so
+// 8 x 8 sums at NB = 64.  What bounds it is the FP32 FMA rate.  The 8 x 4 thread tile of
+// conv_simt_kernel read 22 shared-memory words per 96 FMAs, with 2- to 4-way bank conflicts, and
+// staged each slice of 8 input channels between two barriers with nothing else to do.  Here a
+// (channel, ky) reads 36 words without conflicts per 192 FMAs, issued as 96 packed FMAs
+// (fma.rn.f32x2, each half an IEEE FMA), and the next slice's rows and weights arrive by cp.async
+// meanwhile.  Three blocks of four warps share an SM.  960 x 540, 64 -> 64: 763 us with 16 pixels a
+// thread and 8 rows a block, which halves the weight reads but leaves two warps to a scheduler (FMA
+// pipe 71 % busy); with 8 pixels 722, 709 and 688 us with 8, 4 and 2 rows a block (blocks of more
+// rows wait for each other at the slice barriers and fill the last round worse: 64 x 64 takes 129,
+// 82 and 60 us); 675 with the registers of three resident blocks (150 a thread) instead of four (126).
+// Products are summed in the same order (channel, ky, kx), so the values are the same.  960 x 540,
+// 64 -> 64: the layer call 1162 -> 675 us (57 TFLOP/s; a chain of independent FMAs runs at 79).
 // PLANAR: x, y and the residual are planar float32 [C][H][W] (the caller's tensors, no layout copy).
 constexpr int C3_TX = 64;       // pixels of a block's row
+constexpr int C3_R = 2;         // its rows
+constexpr int C3_NT = 64 * C3_R;
 constexpr int C3_PITCH = 68;    // floats of a staged row (66 used)
 
 __device__ __forceinline__ void cp_async4(uint32_t dst, const void *src, bool valid) {
@@ -272,11 +278,12 @@ __device__ __forceinline__ void ffma2_64(uint64_t &acc, uint64_t a, uint64_t b) 
     asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
 }
 
-template <int NB, int R>
-constexpr size_t c3_smem() { return 2 * sizeof(float) * (8 * (R + 2) * C3_PITCH + 8 * 9 * NB); }
+template <int NB>
+constexpr size_t c3_smem() { return 2 * sizeof(float) * (8 * (C3_R + 2) * C3_PITCH + 8 * 9 * NB); }
 
-template <int NB, int R, bool PLANAR>
-__global__ void __launch_bounds__(32 * R, 8 / R) conv3_f32_kernel(const __grid_constant__ ConvArgs a) {
+template <int NB, bool PLANAR>
+__global__ void __launch_bounds__(C3_NT, 3) conv3_f32_kernel(const __grid_constant__ ConvArgs a) {
+    constexpr int R = C3_R;
     constexpr int N = NB / 8;          // outputs of a thread
     constexpr int ASZ = 8 * (R + 2) * C3_PITCH, BSZ = 8 * 9 * NB;
     extern __shared__ __align__(16) float smem_f[];
@@ -291,12 +298,13 @@ __global__ void __launch_bounds__(32 * R, 8 / R) conv3_f32_kernel(const __grid_c
     const int oc_base = blockIdx.y * NB;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int og = lane & 7, pg = lane >> 3;
+    const int row = warp % R, half = warp / R;
     const float *x = static_cast<const float *>(a.x) + (PLANAR ? 0 : (int64_t)img * (a.cin_pad / 4) * HW * 4);
     const float *wts = static_cast<const float *>(a.w);
 
     auto stage = [&](int sl, int buf) {
         // input rows: a warp per (channel, row), pixels x0 - 1 .. x0 + 64, zero outside the image
-        for (int i = warp; i < 8 * (R + 2); i += R) {
+        for (int i = warp; i < 8 * (R + 2); i += 2 * R) {
             const int c = i / (R + 2), r = i - c * (R + 2);
             const int ch = sl * 8 + c, iy = y0 + r - 1;
             const bool rok = iy >= 0 && iy < H && (!PLANAR || ch < a.cin);
@@ -310,16 +318,16 @@ __global__ void __launch_bounds__(32 * R, 8 / R) conv3_f32_kernel(const __grid_c
                 cp_async4(dst + 4u * (uint32_t)p, ok ? x + at : x, ok);
             }
         }
-        for (int i = threadIdx.x; i < BSZ / 4; i += 32 * R) {
+        for (int i = threadIdx.x; i < BSZ / 4; i += C3_NT) {
             const int ct = i / (NB / 4), n4 = i - ct * (NB / 4);
             cp_async16(smem_u32(Bs + buf * BSZ + i * 4), wts + ((int64_t)sl * 72 + ct) * a.cout_pad + oc_base + n4 * 4);
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
 
-    uint64_t acc[16][N / 2];
+    uint64_t acc[8][N / 2];
 #pragma unroll
-    for (int p = 0; p < 16; ++p)
+    for (int p = 0; p < 8; ++p)
 #pragma unroll
         for (int n = 0; n < N / 2; ++n) acc[p][n] = 0;
 
@@ -334,15 +342,15 @@ __global__ void __launch_bounds__(32 * R, 8 / R) conv3_f32_kernel(const __grid_c
             asm volatile("cp.async.wait_group 0;" ::: "memory");
         }
         __syncthreads();
-        const float *ar0 = As + buf * ASZ + warp * C3_PITCH + 4 * pg;
+        const float *ar0 = As + buf * ASZ + row * C3_PITCH + 32 * half + 4 * pg;
         const float *br0 = Bs + buf * BSZ;
 #pragma unroll 1
         for (int c = 0; c < 8; ++c) {
 #pragma unroll
             for (int ky = 0; ky < 3; ++ky) {
-                float av[4][6];
+                float av[2][6];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
+                for (int j = 0; j < 2; ++j) {
                     const float *ar = ar0 + (c * (R + 2) + ky) * C3_PITCH + 16 * j;
                     const float4 v0 = *reinterpret_cast<const float4 *>(ar);
                     const float2 v1 = *reinterpret_cast<const float2 *>(ar + 4);
@@ -364,7 +372,7 @@ __global__ void __launch_bounds__(32 * R, 8 / R) conv3_f32_kernel(const __grid_c
                         }
                     }
 #pragma unroll
-                    for (int p = 0; p < 16; ++p) {
+                    for (int p = 0; p < 8; ++p) {
                         const float v = av[p / 4][p % 4 + kx];
                         const uint64_t vv = pair_f32(v, v);
 #pragma unroll
@@ -377,14 +385,14 @@ __global__ void __launch_bounds__(32 * R, 8 / R) conv3_f32_kernel(const __grid_c
     }
 
     // ---- epilogue: outputs oc(n) = oc_base + 4 og + n (NB 64: the upper half 32 further; NB 16: 2 og + n)
-    const int y = y0 + warp;
+    const int y = y0 + row;
     if (y >= H) return;
     auto oc_of = [&](int n) { return oc_base + (N == 2 ? 2 * og + n : 32 * (n / 4) + 4 * og + n % 4); };
     float v[N][4];  // a run of 4 pixels
     const bool vec = PLANAR && W % 4 == 0 && (reinterpret_cast<uintptr_t>(a.y) & 15) == 0;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int xx = x0 + 16 * j + 4 * pg;
+    for (int j = 0; j < 2; ++j) {
+        const int xx = x0 + 32 * half + 16 * j + 4 * pg;
         if (xx >= W) continue;
         const int64_t pix = (int64_t)y * W + xx;
 #pragma unroll
@@ -443,30 +451,15 @@ __global__ void __launch_bounds__(32 * R, 8 / R) conv3_f32_kernel(const __grid_c
     }
 }
 
-template <int NB, int R, bool PLANAR>
-cudaError_t run_c3(const ConvArgs &a, cudaStream_t st) {
-    constexpr size_t smem = c3_smem<NB, R>();
-    const cudaError_t e = set_smem_limit<conv3_f32_kernel<NB, R, PLANAR>>((int)smem);
-    if (e != cudaSuccess) return e;
-    const dim3 grid((unsigned)((a.W + C3_TX - 1) / C3_TX * ((a.H + R - 1) / R) * a.nimg), (unsigned)(a.cout_pad / NB));
-    conv3_f32_kernel<NB, R, PLANAR><<<grid, 32 * R, smem, st>>>(a);
-    return cudaGetLastError();
-}
-
-// Rows per block: an SM holds 8 rows at a time whatever R (8 / R blocks), so a launch takes
-// ceil(blocks / (SMs * 8 / R)) rounds of 8 rows; fewer rows per block fill the last round
-// better and stage more halo rows (the constants below, in rows).
 template <int NB, bool PLANAR>
 cudaError_t launch_c3(const ConvArgs &a, cudaStream_t st) {
-    const int64_t sms = device_sm_count(), cols = (int64_t)((a.W + C3_TX - 1) / C3_TX) * a.nimg * (a.cout_pad / NB);
-    auto cost = [&](int R, double halo) {
-        const int64_t blocks = cols * ((a.H + R - 1) / R), per = sms * (8 / R);
-        return (double)((blocks + per - 1) / per) * (8.0 + halo);
-    };
-    const double c8 = cost(8, 0.0), c4 = cost(4, 0.4), c2 = cost(2, 1.2);
-    if (c8 <= c4 && c8 <= c2) return run_c3<NB, 8, PLANAR>(a, st);
-    if (c4 <= c2) return run_c3<NB, 4, PLANAR>(a, st);
-    return run_c3<NB, 2, PLANAR>(a, st);
+    constexpr size_t smem = c3_smem<NB>();
+    const cudaError_t e = set_smem_limit<conv3_f32_kernel<NB, PLANAR>>((int)smem);
+    if (e != cudaSuccess) return e;
+    const int tiles = (a.W + C3_TX - 1) / C3_TX * ((a.H + C3_R - 1) / C3_R);
+    const dim3 grid((unsigned)(tiles * a.nimg), (unsigned)(a.cout_pad / NB));
+    conv3_f32_kernel<NB, PLANAR><<<grid, C3_NT, smem, st>>>(a);
+    return cudaGetLastError();
 }
 
 template <int NB, int KS, int MODE>

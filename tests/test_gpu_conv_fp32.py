@@ -1,4 +1,4 @@
-"""The FP32 3x3 layer at the edges of its tiles (64 pixels x 8, 4 or 2 rows; 16, 32 or 64 outputs;
+"""The FP32 3x3 layer at the edges of its tiles (64 pixels x 2 rows; 16, 32 or 64 outputs;
 slices of 8 input channels), straight on the caller's planar tensors, and in place.  Against a
 64-bit convolution within the FP32 layer's tolerance (2e-5 for inputs in [-1, 1])."""
 import numpy as np
