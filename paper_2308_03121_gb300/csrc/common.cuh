@@ -265,7 +265,8 @@ struct WeightArgs {
     float *dst_bias;
     int nbias;
 };
-cudaError_t launch_weights(const WeightArgs &a, cudaStream_t st);
+// second: another layer of the same layout, type and sizes in the same launch
+cudaError_t launch_weights(const WeightArgs &a, cudaStream_t st, const WeightArgs *second = nullptr);
 // max |v| of n device values, as float bits, by atomicMax into *out.
 cudaError_t launch_absmax(const float *v, int64_t n, unsigned *out, cudaStream_t st);
 

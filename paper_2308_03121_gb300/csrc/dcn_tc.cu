@@ -486,9 +486,9 @@ __global__ void __launch_bounds__(256) dcn_pairs_planar_kernel(const float *__re
     v1.z = __shfl_down_sync(0xffffffffu, v0.z, 1);
     v1.w = __shfl_down_sync(0xffffffffu, v0.w, 1);
     if ((threadIdx.x & 31) == 31) v1 = load(p + 1);
-    if (p >= HW) return;
     if ((int)(p % W) == W - 1) v1 = make_uint4(0u, 0u, 0u, 0u);
-    st_global_v8((cc < 4 ? lo : hi) + ((int64_t)(cc & 3) * HW + p) * 2, v0, v1);
+    if (p < HW) st_global_v8((cc < 4 ? lo : hi) + ((int64_t)(cc & 3) * HW + p) * 2, v0, v1);
+    griddep_wait();  // (launched beside the weights' layout)
 }
 
 }  // namespace
@@ -505,10 +505,9 @@ cudaError_t launch_dcn_pairs_planar(const float *x, int H, int W, int dt, void *
     const int64_t HW = (int64_t)H * W;
     const dim3 grd((unsigned)((HW + 255) / 256), 8);
     uint4 *l = static_cast<uint4 *>(lo), *h = static_cast<uint4 *>(hi);
-    if (dt == DT_BF16) dcn_pairs_planar_kernel<__nv_bfloat16><<<grd, 256, 0, st>>>(x, HW, W, l, h);
-    else if (dt == DT_F16) dcn_pairs_planar_kernel<__half><<<grd, 256, 0, st>>>(x, HW, W, l, h);
-    else return cudaErrorInvalidValue;
-    return cudaGetLastError();
+    if (dt == DT_BF16) return launch_dependent(dcn_pairs_planar_kernel<__nv_bfloat16>, grd, dim3(256), 0, st, x, HW, W, l, h);
+    if (dt == DT_F16) return launch_dependent(dcn_pairs_planar_kernel<__half>, grd, dim3(256), 0, st, x, HW, W, l, h);
+    return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_dcn_tc(const DcnArgs &a0, cudaStream_t st) {

@@ -2910,14 +2910,14 @@ nvisr_status nvisr_resblock2d(int32_t precision, const float *x, int32_t h, int3
     const size_t o_h = sc.plan(fused ? 256 : abytes);
     NVISR_TRY_CUDA(sc.open());
     void *dx = sc.at<void>(o_x), *dh = sc.at<void>(o_h);
+    WeightArgs wa[2] = {};
     for (int c = 0; c < 2; ++c) {
-        WeightArgs wa{};
-        wa.w = c ? w2 : w1; wa.bias = c ? b2 : b1;
-        wa.cout = wa.cin = wa.cin_pad = wa.cout_pad = wa.nbias = 64;
-        wa.k = 3; wa.layout = WL_ROWS; wa.dt = dt; wa.scale = 1.f;
-        wa.dst = sc.at<void>(c ? o_w2 : o_w1); wa.dst_bias = sc.at<float>(c ? o_b2 : o_b1);
-        NVISR_TRY_CUDA(launch_weights(wa, st));
+        wa[c].w = c ? w2 : w1; wa[c].bias = c ? b2 : b1;
+        wa[c].cout = wa[c].cin = wa[c].cin_pad = wa[c].cout_pad = wa[c].nbias = 64;
+        wa[c].k = 3; wa[c].layout = WL_ROWS; wa[c].dt = dt; wa[c].scale = 1.f;
+        wa[c].dst = sc.at<void>(c ? o_w2 : o_w1); wa[c].dst_bias = sc.at<float>(c ? o_b2 : o_b1);
     }
+    NVISR_TRY_CUDA(launch_weights(wa[0], st, &wa[1]));
     NVISR_TRY_CUDA(launch_pack_planar(x, 64, 64, h, w, dt, 1.f, dx, 64, st));
     ConvArgs a1{};
     a1.x = dx; a1.cin_pad = 64; a1.in_cpc = 64; a1.out_cpc = 64; a1.H = h; a1.W = w; a1.nimg = 1;

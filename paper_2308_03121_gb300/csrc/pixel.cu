@@ -788,7 +788,9 @@ __global__ void __launch_bounds__(128) pack_rows_table_kernel(const PackArgs *__
 }
 
 // Layout change between a layer's planar float32 tensor [C][HW] and its blocked form, for whole
-// frames without row padding.  Both directions move each byte once (HBM-bound); what costs time
+// frames without row padding.  The packs are launched as dependents of the weights' layout (or of
+// another pack), which they do not read: they run beside it and end only when it has, so the
+// kernel after them finds both done.  Both directions move each byte once (HBM-bound); what costs time
 // is touching memory in pieces below its 32-byte sectors, so a warp covers full lines on both
 // sides.
 //
@@ -836,11 +838,13 @@ __global__ void __launch_bounds__(256) pack_lines_kernel(const float *__restrict
                 *reinterpret_cast<uint4 *>(dst + ((int64_t)blk * HW + p) * 128 + unit * 16) = pack_unit<T>(v[j]);
         }
     }
+    griddep_wait();
 }
 
 template <typename T, bool VEC>
 __global__ void __launch_bounds__(256) unpack_lines_kernel(const uint8_t *__restrict__ src, int64_t HW, int C,
                                                            int nblk, float scale, float *__restrict__ dst) {
+    griddep_wait();
     const int unit = ((threadIdx.x >> 5) & 1) * 4 + ((threadIdx.x & 31) >> 3);
     for (int blk = blockIdx.y; blk < nblk; blk += gridDim.y) {
         const int c0 = blk * 64 + unit * 8;
@@ -879,8 +883,7 @@ __global__ void __launch_bounds__(256) pack_units_kernel(const float *__restrict
                                                          float scale, uint8_t *__restrict__ dst) {
     constexpr int UPC = 16 / sizeof(T);
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= HW) return;
-    for (int u = blockIdx.y; u < nunits; u += gridDim.y) {
+    for (int u = blockIdx.y; u < nunits && p < HW; u += gridDim.y) {
         float v[UPC];
 #pragma unroll
         for (int e = 0; e < UPC; ++e) {
@@ -889,11 +892,13 @@ __global__ void __launch_bounds__(256) pack_units_kernel(const float *__restrict
         }
         *reinterpret_cast<uint4 *>(dst + ((int64_t)u * HW + p) * 16) = pack_unit<T>(v);
     }
+    griddep_wait();
 }
 
 template <typename T>
 __global__ void __launch_bounds__(256) unpack_units_kernel(const uint8_t *__restrict__ src, int64_t HW, int C,
                                                            int nunits, float scale, float *__restrict__ dst) {
+    griddep_wait();
     constexpr int UPC = 16 / sizeof(T);
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= HW) return;
@@ -1041,6 +1046,7 @@ cudaError_t launch_pack(const PackArgs &a0, cudaStream_t st) {
 cudaError_t launch_pack_planar(const float *src, int C, int cpad, int H, int W, int dt, float scale, void *dst, int cpc,
                                cudaStream_t st) {
     const int upc = chunk_channels(dt);
+    cudaError_t e = cudaSuccess;
     if (cpc == 0) cpc = upc;
     const int64_t HW = (int64_t)H * W;
     uint8_t *d = static_cast<uint8_t *>(dst);
@@ -1050,24 +1056,24 @@ cudaError_t launch_pack_planar(const float *src, int C, int cpad, int H, int W, 
         const dim3 grd((unsigned)((HW + LINE_PX - 1) / LINE_PX), (unsigned)std::min(n, 65535));
         const bool vec = HW % 4 == 0 && (reinterpret_cast<uintptr_t>(src) & 15) == 0;
         if (dt == DT_BF16) {
-            if (vec) pack_lines_kernel<__nv_bfloat16, true><<<grd, 256, 0, st>>>(src, HW, C, n, scale, d);
-            else pack_lines_kernel<__nv_bfloat16, false><<<grd, 256, 0, st>>>(src, HW, C, n, scale, d);
+            if (vec) e = launch_dependent(pack_lines_kernel<__nv_bfloat16, true>, grd, dim3(256), 0, st, src, HW, C, n, scale, d);
+            else e = launch_dependent(pack_lines_kernel<__nv_bfloat16, false>, grd, dim3(256), 0, st, src, HW, C, n, scale, d);
         } else {
-            if (vec) pack_lines_kernel<__half, true><<<grd, 256, 0, st>>>(src, HW, C, n, scale, d);
-            else pack_lines_kernel<__half, false><<<grd, 256, 0, st>>>(src, HW, C, n, scale, d);
+            if (vec) e = launch_dependent(pack_lines_kernel<__half, true>, grd, dim3(256), 0, st, src, HW, C, n, scale, d);
+            else e = launch_dependent(pack_lines_kernel<__half, false>, grd, dim3(256), 0, st, src, HW, C, n, scale, d);
         }
-        return cudaGetLastError();
+        return e;
     }
     if (cpc != upc || cpad % upc) return cudaErrorInvalidValue;
     const int n = cpad / upc;
     const dim3 grd((unsigned)((HW + 255) / 256), (unsigned)std::min(n, 65535));
     switch (dt) {
-        case DT_F32: pack_units_kernel<float><<<grd, 256, 0, st>>>(src, HW, C, n, scale, d); break;
-        case DT_BF16: pack_units_kernel<__nv_bfloat16><<<grd, 256, 0, st>>>(src, HW, C, n, scale, d); break;
-        case DT_F16: pack_units_kernel<__half><<<grd, 256, 0, st>>>(src, HW, C, n, scale, d); break;
-        default: pack_units_kernel<__nv_fp8_e4m3><<<grd, 256, 0, st>>>(src, HW, C, n, scale, d); break;
+        case DT_F32: e = launch_dependent(pack_units_kernel<float>, grd, dim3(256), 0, st, src, HW, C, n, scale, d); break;
+        case DT_BF16: e = launch_dependent(pack_units_kernel<__nv_bfloat16>, grd, dim3(256), 0, st, src, HW, C, n, scale, d); break;
+        case DT_F16: e = launch_dependent(pack_units_kernel<__half>, grd, dim3(256), 0, st, src, HW, C, n, scale, d); break;
+        default: e = launch_dependent(pack_units_kernel<__nv_fp8_e4m3>, grd, dim3(256), 0, st, src, HW, C, n, scale, d); break;
     }
-    return cudaGetLastError();
+    return e;
 }
 
 bool pack_rows_fits(const PackArgs &a) {
@@ -1101,6 +1107,7 @@ cudaError_t launch_pack_table(const PackArgs *host_tab, const PackArgs *dev_tab,
 cudaError_t launch_unpack_planar(const void *src, int dt, int cpad, int cpc, int C, int H, int W, float scale,
                                  float *dst, cudaStream_t st) {
     const int upc = chunk_channels(dt);
+    cudaError_t e = cudaSuccess;
     if (cpc == 0) cpc = upc;
     const int64_t HW = (int64_t)H * W;
     const uint8_t *s = static_cast<const uint8_t *>(src);
@@ -1110,24 +1117,24 @@ cudaError_t launch_unpack_planar(const void *src, int dt, int cpad, int cpc, int
         const dim3 grd((unsigned)((HW + LINE_PX - 1) / LINE_PX), (unsigned)std::min(n, 65535));
         const bool vec = HW % 4 == 0 && (reinterpret_cast<uintptr_t>(dst) & 15) == 0;
         if (dt == DT_BF16) {
-            if (vec) unpack_lines_kernel<__nv_bfloat16, true><<<grd, 256, 0, st>>>(s, HW, C, n, scale, dst);
-            else unpack_lines_kernel<__nv_bfloat16, false><<<grd, 256, 0, st>>>(s, HW, C, n, scale, dst);
+            if (vec) e = launch_dependent(unpack_lines_kernel<__nv_bfloat16, true>, grd, dim3(256), 0, st, s, HW, C, n, scale, dst);
+            else e = launch_dependent(unpack_lines_kernel<__nv_bfloat16, false>, grd, dim3(256), 0, st, s, HW, C, n, scale, dst);
         } else {
-            if (vec) unpack_lines_kernel<__half, true><<<grd, 256, 0, st>>>(s, HW, C, n, scale, dst);
-            else unpack_lines_kernel<__half, false><<<grd, 256, 0, st>>>(s, HW, C, n, scale, dst);
+            if (vec) e = launch_dependent(unpack_lines_kernel<__half, true>, grd, dim3(256), 0, st, s, HW, C, n, scale, dst);
+            else e = launch_dependent(unpack_lines_kernel<__half, false>, grd, dim3(256), 0, st, s, HW, C, n, scale, dst);
         }
-        return cudaGetLastError();
+        return e;
     }
     if (cpc != upc || cpad % upc) return cudaErrorInvalidValue;
     const int n = cpad / upc;
     const dim3 grd((unsigned)((HW + 255) / 256), (unsigned)std::min(n, 65535));
     switch (dt) {
-        case DT_F32: unpack_units_kernel<float><<<grd, 256, 0, st>>>(s, HW, C, n, scale, dst); break;
-        case DT_BF16: unpack_units_kernel<__nv_bfloat16><<<grd, 256, 0, st>>>(s, HW, C, n, scale, dst); break;
-        case DT_F16: unpack_units_kernel<__half><<<grd, 256, 0, st>>>(s, HW, C, n, scale, dst); break;
-        default: unpack_units_kernel<__nv_fp8_e4m3><<<grd, 256, 0, st>>>(s, HW, C, n, scale, dst); break;
+        case DT_F32: e = launch_dependent(unpack_units_kernel<float>, grd, dim3(256), 0, st, s, HW, C, n, scale, dst); break;
+        case DT_BF16: e = launch_dependent(unpack_units_kernel<__nv_bfloat16>, grd, dim3(256), 0, st, s, HW, C, n, scale, dst); break;
+        case DT_F16: e = launch_dependent(unpack_units_kernel<__half>, grd, dim3(256), 0, st, s, HW, C, n, scale, dst); break;
+        default: e = launch_dependent(unpack_units_kernel<__nv_fp8_e4m3>, grd, dim3(256), 0, st, s, HW, C, n, scale, dst); break;
     }
-    return cudaGetLastError();
+    return e;
 }
 
 // ---------------------------------------------------------------- fused requantise helpers
