@@ -234,13 +234,14 @@ __device__ __forceinline__ void chroma_pair(const uint8_t *base, int64_t pitch, 
 // 4:2:0 ingest: a lane takes 4 luma columns of rows 2j and 2j + 1.  Its two chroma columns are read
 // from chroma rows j - 1, j and j + 1, normalised and interpolated vertically, then horizontally
 // with the neighbouring lanes' (the scalar form's order).  Divisions are replaced by
-// multiplications with the reciprocal.  Bound by instruction issue (71 % busy with a lane per 4
-// columns of one row, which reads and normalises the chroma twice) and the float planes' writes:
-// 3840 x 2160 10-bit 34.0 -> 25.9 us (a lane per 8 columns wrote each plane in 16-byte halves of its
-// sectors).  LOC and XF (a transfer function) are template parameters: the code of the other
-// forms, inlined for each sample, would be fetched with it.
+// multiplications with the reciprocal.  Bound by the latency of its loads and by the float planes'
+// writes: 3840 x 2160 10-bit 34.0 us with a lane per 8 columns (which wrote each plane in 16-byte
+// halves of its sectors), 29.0 with a lane per 4 columns of one row (issue 71 % busy: the chroma
+// was read and normalised twice), 26.0 with the row pair at 54 registers, 24.8 at 48 (10 blocks an
+// SM; at 40 it spills: 26.4).  LOC and XF (a transfer function) are template parameters: the code
+// of the other forms, inlined for each sample, would be fetched with it.
 template <typename S, int LOC, bool XF>
-__global__ void __launch_bounds__(32 * Q_WARPS) ingest420_kernel(
+__global__ void __launch_bounds__(32 * Q_WARPS, 10) ingest420_kernel(
     const uint8_t *__restrict__ yp, int64_t py, const uint8_t *__restrict__ up, int64_t pu,
     const uint8_t *__restrict__ vp, int64_t pv, int H, int W, RangeConst rc, float *__restrict__ out, int64_t pitch) {
     // launched as a dependent: the ring slot may still be read by the stream's previous kernel
