@@ -399,9 +399,11 @@ void nvisr_server_destroy(nvisr_server *server);
 /* One 2-D convolution layer (Section 3.1 networks) on planar float32 tensors:
  * y[cout][H][W] = act(conv_k(x[cin][H][W]; w[cout][cin][k][k]) + b) (+ res),
  * stride 1, zero padding (k-1)/2, act 0 = none, 1 = LeakyReLU(0.1).  Runs the
- * precision's kernel (FP32 SIMT or tensor cores); the library converts x to
- * its internal layout in scratch device memory it allocates per call.
- * res may be NULL.  All pointers are device pointers. */
+ * precision's kernel (FP32 SIMT or tensor cores); where that works on the
+ * internal layout, the library converts x, and res and y where needed, in
+ * scratch device memory that it keeps from call to call (at most 1 GiB per
+ * context).  res may be NULL; y may overlap x and res.  All pointers are
+ * device pointers. */
 nvisr_status nvisr_conv2d(int32_t precision, const float *x, int32_t cin, int32_t h, int32_t w,
                           const float *weight, const float *bias, int32_t cout, int32_t k,
                           int32_t act, const float *res, float *y, void *stream);
@@ -414,8 +416,8 @@ nvisr_status nvisr_conv2d(int32_t precision, const float *x, int32_t cin, int32_
  * (device memory handed out in advance, or real-time work that cannot let
  * cudaFree synchronise the device).  Same arguments, results and error codes
  * as nvisr_conv2d, except:
- *  - every working buffer (blocked x, y and res, weight image, bias, error
- *    word) is carved from one static device array of
+ *  - every working buffer (blocked x, y and res where the kernel needs them,
+ *    weight image, bias, error word) is carved from one static device array of
  *    NVISR_CONV2D_STATIC_SCRATCH_BYTES per device, set aside when the module
  *    loads; weights are laid out by device kernels, so nothing is staged on
  *    the host.  A problem that does not fit returns NVISR_OVER_BUDGET before
@@ -444,11 +446,11 @@ nvisr_status nvisr_conv2d_static(int32_t precision, const float *x, int32_t cin,
  * (out, in, ky, kx); b1, b2: [64] or NULL (zero).  All pointers are device
  * pointers; y must not overlap x.  precision: BF16 or FP16 (activations and
  * operands in that type, FP32 accumulation; others return
- * NVISR_UNSUPPORTED_FORMAT).  fused != 0: one launch of 2-CTA clusters in
- * which one SM computes conv1 and writes its rows into the other SM's shared
- * memory, where conv2 reads them (the middle tensor never reaches device
- * memory); fused == 0: two launches of the single-layer row kernel.  Both
- * give the same values.  Scratch is allocated per call; returns after
+ * NVISR_UNSUPPORTED_FORMAT).  fused != 0: one launch of 2-CTA clusters, each a
+ * pair of SMs that runs both convs on two column tiles at once with the
+ * middle tensor's rows in shared memory (it never reaches device memory);
+ * fused == 0: two launches of the single-layer row kernel.  Both give the
+ * same values.  Scratch is kept from call to call; returns after
  * synchronising `stream` (it reads the error word back: NVISR_DEVICE_TIMEOUT
  * if a device-side wait ran out). */
 nvisr_status nvisr_resblock2d(int32_t precision, const float *x, int32_t h, int32_t w, const float *w1,
@@ -458,7 +460,7 @@ nvisr_status nvisr_resblock2d(int32_t precision, const float *x, int32_t h, int3
 /* Modulated deformable convolution 3x3, DCN v2 as in torchvision's
  * deform_conv2d (Section 3.1): offsets [2*G*9][H][W] (dy, dx per group and
  * tap), mask [G*9][H][W] (already in [0,1]), stride 1, padding 1.  Planar
- * float32 device tensors; scratch allocated per call.  x must be finite: the
+ * float32 device tensors; scratch kept from call to call.  x must be finite: the
  * tensor-core gather skips the loads of corners whose bilinear weight is zero
  * (outside the image), and a skipped corner contributes weight x an earlier
  * sample, which is zero only for a finite sample. */

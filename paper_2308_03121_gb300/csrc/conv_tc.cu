@@ -14,10 +14,10 @@
 //    of tap (ky, kx) is the same buffer addressed (ky*(128+KS-1) + kx)*16
 //    bytes further: the 9 taps share one load.
 //  * The layer's weights (or a slice of its output channels) stay resident in
-//    shared memory for the whole persistent CTA, pre-arranged on the host in
-//    the same core-matrix layout.
-//  * One thread issues tcgen05.mma (kind::f16 for BF16/FP16, kind::f8f6f4 for
-//    FP8 E4M3) into a double-buffered FP32 accumulator in TMEM; commits
+//    shared memory for the whole persistent CTA, pre-arranged in the same
+//    core-matrix layout.
+//  * One elected lane issues tcgen05.mma (kind::f16 for BF16/FP16, kind::f8f6f4
+//    for FP8 E4M3) into a double-buffered FP32 accumulator in TMEM; commits
 //    release shared-memory stages and hand finished tiles to the epilogue.
 //  * Four epilogue warps read TMEM (tcgen05.ld), apply scale, bias,
 //    LeakyReLU(0.1) and the residual add, and store the blocked output; the
@@ -115,21 +115,6 @@ __device__ __forceinline__ float from_elem<__half>(__half v) { return __half2flo
 __device__ __forceinline__ void raise_abort(volatile int *abort, int *err) {
     *abort = 1;
     if (err) atomicExch(err, DEVERR_TIMEOUT);
-}
-
-// Store 16 values as 16-bit or 8-bit elements at out (16 or 32 bytes... as
-// whole 16-byte chunks of the blocked layout).
-template <typename T>
-__device__ __forceinline__ void store_vals(uint8_t *base, int64_t chunk_stride, int chunk0, const float *v,
-                                           int n) {
-    constexpr int CPC = 16 / sizeof(T);
-    for (int c = 0; c < n / CPC; ++c) {
-        alignas(16) T o[CPC];
-#pragma unroll
-        for (int e = 0; e < CPC; ++e) o[e] = to_elem<T>(v[c * CPC + e]);
-        *reinterpret_cast<uint4 *>(base + (int64_t)(chunk0 + c) * chunk_stride) =
-            *reinterpret_cast<const uint4 *>(o);
-    }
 }
 
 // IN_DT: operand dtype; OUT_DT: dtype of y/res (16-bit, or E4M3 when the
