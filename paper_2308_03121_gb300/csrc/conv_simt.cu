@@ -254,9 +254,10 @@ __global__ void __launch_bounds__(16 * NB / 4) conv_simt_kernel(ConvArgs a, DcnA
 // thread and 8 rows a block, which halves the weight reads but leaves two warps to a scheduler (FMA
 // pipe 71 % busy); with 8 pixels 722, 709 and 688 us with 8, 4 and 2 rows a block (blocks of more
 // rows wait for each other at the slice barriers and fill the last round worse: 64 x 64 takes 129,
-// 82 and 60 us); 675 with the registers of three resident blocks (150 a thread) instead of four (126).
+// 82 and 60 us); 675 with the registers of three resident blocks (150 a thread) instead of four (126);
+// 660 with the channel loop unrolled four times (two 660, eight 662; 64 x 64 57, 60 and 60).
 // Products are summed in the same order (channel, ky, kx), so the values are the same.  960 x 540,
-// 64 -> 64: the layer call 1162 -> 675 us (57 TFLOP/s; a chain of independent FMAs runs at 79).
+// 64 -> 64: the layer call 1162 -> 660 us (58 TFLOP/s; a chain of independent FMAs runs at 79).
 // PLANAR: x, y and the residual are planar float32 [C][H][W] (the caller's tensors, no layout copy).
 constexpr int C3_TX = 64;       // pixels of a block's row
 constexpr int C3_R = 2;         // its rows
@@ -344,7 +345,7 @@ __global__ void __launch_bounds__(C3_NT, 3) conv3_f32_kernel(const __grid_consta
         __syncthreads();
         const float *ar0 = As + buf * ASZ + row * C3_PITCH + 32 * half + 4 * pg;
         const float *br0 = Bs + buf * BSZ;
-#pragma unroll 1
+#pragma unroll 4
         for (int c = 0; c < 8; ++c) {
 #pragma unroll
             for (int ky = 0; ky < 3; ++ky) {
