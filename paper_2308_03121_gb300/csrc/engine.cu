@@ -169,6 +169,7 @@ struct Step {
     int widx = -1;       // weights variant (input channels permuted), -1 = the layer's own
     int om_t = -1;       // DCN: offsets/mask tensor
     bool om_tap_major = false;  // DCN: om channels in tap-major order (its head's rows permuted)
+    void *pair_hi = nullptr;    // DCN: second half of its input's pixel pairs (tensor-core path)
     std::vector<int> skip_frames;  // final outputs: frames whose upsampled mean is added
     int in_t = -1;       // input tensor id (SRC_TENSOR)
     int src = SRC_TENSOR;
@@ -256,7 +257,7 @@ struct nvisr_filter {
     std::vector<Weights> weights;  // per layer (shared layers point to the owner)
     std::vector<int> om_tap_g;     // per layer: G when its output rows are stored tap-major, else 0
     std::vector<Tensor> tensors;
-    void *dcn_lo = nullptr, *dcn_hi = nullptr;  // DCN input in pixel pairs (tensor-core path)
+    void *dcn_lo = nullptr;        // first half of a DCN's input in pixel pairs (tensor-core path)
     std::vector<Step> steps;
     std::vector<char> blk;           // step i and i + 1 form a residual block run as one fused launch
     int pack_t = -1;               // tensor id of the packed tuple
@@ -1291,22 +1292,43 @@ nvisr_status build_plan_group(nvisr_filter *f, const float *blob) {
             f->wvar.push_back(Wv);
         }
     }
-    // the tensor-core DCN gathers from its input copied into pixel pairs.  Half of them may use
-    // the first output's float32 image where it is large enough: the run's last layers write it
-    // after every DCN, and an output of an earlier run has left it by then
-    size_t pairs = 0;
-    for (const Step &st : f->steps)
-        if (st.op == OP_DCN && f->tc)
-            pairs = std::max(pairs, (size_t)DCN_PAIR_BYTES * f->tensors[st.in_t].H * f->tensors[st.in_t].W);
-    if (pairs) {
-        nvisr_status s = dalloc(f->eng, pairs, f->owned, &f->dcn_lo, f->guard);
-        if (s != NVISR_OK) return s;
-        if (sizeof(float) * 3 * f->opitch * H * net.scale_y >= pairs) {
-            f->dcn_hi = f->out_rgb[0];
-        } else if ((s = dalloc(f->eng, pairs, f->owned, &f->dcn_hi, f->guard)) != NVISR_OK) {
-            return s;
+    // The tensor-core DCN gathers from its input copied into pixel pairs.  Half of them go to a
+    // buffer that holds nothing while their step runs: the float32 image of an output that only
+    // later steps of the run write (its values of an earlier run have left it, since a run
+    // rewrites it anyway), or a pool buffer that no live tensor has; else to one of their own.
+    auto idle_buffer = [&](int step, size_t bytes) -> void * {
+        if (sizeof(float) * 3 * f->opitch * H * net.scale_y >= bytes)
+            for (int k = 0; k < f->run_out; ++k) {
+                int first = -1;
+                for (int i = (int)f->steps.size() - 1; i >= 0; --i)
+                    if (f->steps[i].out_t < 0 && f->steps[i].out_index == k) first = i;
+                if (first > step) return f->out_rgb[k];
+            }
+        for (const Buf &b : pool) {
+            bool free = b.bytes >= bytes;
+            for (int t = 0; t < n && free; ++t)
+                free = f->tensors[t].parent >= 0 || f->tensors[t].ptr != b.p || step < first_def[t] ||
+                       step > std::max(first_def[t], last_use[t]);
+            if (free) return b.p;
         }
+        return nullptr;
+    };
+    size_t lo = 0, hi = 0;
+    for (size_t i = 0; i < f->steps.size(); ++i) {
+        Step &st = f->steps[i];
+        if (st.op != OP_DCN || !f->tc) continue;
+        const size_t bytes = (size_t)DCN_PAIR_BYTES * f->tensors[st.in_t].H * f->tensors[st.in_t].W;
+        lo = std::max(lo, bytes);
+        st.pair_hi = idle_buffer((int)i, bytes);
+        if (!st.pair_hi) hi = std::max(hi, bytes);
     }
+    void *own = nullptr;
+    for (auto [bytes, p] : {std::pair<size_t, void **>(lo, &f->dcn_lo), std::pair<size_t, void **>(hi, &own)}) {
+        nvisr_status s = bytes ? dalloc(f->eng, bytes, f->owned, p, f->guard) : NVISR_OK;
+        if (s != NVISR_OK) return s;
+    }
+    for (Step &st : f->steps)
+        if (st.op == OP_DCN && !st.pair_hi) st.pair_hi = own;
     for (Tensor &T : f->tensors)
         if (T.parent >= 0) {
             const Tensor &P = f->tensors[T.parent];
@@ -1541,10 +1563,10 @@ nvisr_status run_step(nvisr_filter *f, const Step &s, const float *const *frames
         ProfScope ps(f, NVISR_K_DCN);
         if (f->tc) {
             if (in.cpad != 64) return cuda_status(cudaErrorNotSupported, ("dcn layer " + L.name).c_str());
-            cudaError_t e = launch_dcn_pairs(in.ptr, in.H, in.W, in.cpc, f->dcn_lo, f->dcn_hi, st);
+            cudaError_t e = launch_dcn_pairs(in.ptr, in.H, in.W, in.cpc, f->dcn_lo, s.pair_hi, st);
             if (e != cudaSuccess) return cuda_status(e, ("dcn layer " + L.name + " relayout").c_str());
             d.x = f->dcn_lo;
-            d.x_hi = f->dcn_hi;
+            d.x_hi = s.pair_hi;
         }
         cudaError_t e = f->tc ? launch_dcn_tc(d, st) : launch_dcn_simt(d, st);
         if (e != cudaSuccess) return cuda_status(e, ("dcn layer " + L.name).c_str());
@@ -1751,6 +1773,7 @@ nvisr_status compute_output(nvisr_filter *f, int64_t o) {
         if (!group_locate(f, o, &loc)) return NVISR_AGAIN;
         if (loc.pass) return NVISR_OK;                   // an input frame: nothing to compute
         if (f->cached_run == loc.key) return NVISR_OK;  // an earlier output of the same run computed it
+        f->cached_run = -1;  // the run before is gone once this one has begun
         nvisr_status s = forward_group(f, loc.inputs);
         if (s == NVISR_OK) f->cached_run = loc.key;
         return s;
