@@ -285,7 +285,7 @@ __host__ __device__ inline int dcn_mask_channel(int g, int k, int G, bool tap_ma
 }
 struct DcnArgs {
     const void *x;           // SIMT: blocked; tensor cores: the pixel pairs of channels 0-31
-    const void *x_hi;        // tensor cores: the pixel pairs of channels 32-63
+    const void *x_hi;        // tensor cores: the pixel pairs of channels 32-63; null: x is planes
     int cin_pad, H, W, groups;
     int x_cpc, y_cpc;        // channels per chunk of x (SIMT) and y (0 = 16-byte units)
     const float *om;         // blocked offsets and mask, or the planar offsets
@@ -309,6 +309,10 @@ cudaError_t launch_dcn_tc(const DcnArgs &a, cudaStream_t st);
 // row's two corners.  Chunks 0-3 go to lo, 4-7 to hi (DCN_PAIR_BYTES a pixel each).
 constexpr int DCN_PAIR_BYTES = 4 * 32;
 // From a blocked 64-channel tensor (8 or 64 channels per chunk), or from planar float32 [64][H][W].
+// hi null: lo takes planes of 16-byte entries, one pixel each, for all eight chunks (the layout of a
+// tensor blocked by 8 channels).  That is half the memory, which a filter falls back on; the gather
+// then needs two loads where it has one (a filter's 960 x 540 layer of 8 groups with its copy, offsets
+// of a pixel or so: 307 us from planes, 315 from pairs).
 cudaError_t launch_dcn_pairs(const void *x, int H, int W, int x_cpc, void *lo, void *hi, cudaStream_t st);
 cudaError_t launch_dcn_pairs_planar(const float *x, int H, int W, int dt, void *lo, void *hi, cudaStream_t st);
 

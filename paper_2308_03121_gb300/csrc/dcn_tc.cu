@@ -21,7 +21,9 @@
 // 8 channels of pixels x and x + 1, so a lane fetches both corners of a sample row with one
 // aligned 32-byte load and blends all 8 channels itself.  (From 16-byte entries a lane pair
 // shared each pixel: 9 shuffles per 16 pixels for the records and the halves, and twice the
-// blend's overhead: 311 M warp instructions at 960 x 540 and 8 groups.)
+// blend's overhead: 311 M warp instructions at 960 x 540 and 8 groups.)  Where a filter's plan has
+// no memory for the second half of the pairs (see launch_dcn_pairs) the same gather reads 16-byte
+// entries, two loads a sample row.
 #include "common.cuh"
 #include "sm100_ptx.cuh"
 
@@ -105,8 +107,9 @@ __device__ __forceinline__ float2 fmul2(float s, float2 v) {
 }
 
 // T: 16-bit element type of x / y; NS: output channels (one slice); C: input channels; PLANAR:
-// planar offsets and mask.
-template <typename T, int NS, int C, bool PLANAR>
+// planar offsets and mask; PAIRS: x in pixel pairs (32-byte entries), else in 8-channel planes of
+// 16-byte entries.
+template <typename T, int NS, int C, bool PLANAR, bool PAIRS>
 __global__ void __launch_bounds__(NT, 1) dcn_tc_kernel(const DcnArgs a, int stages) {
     constexpr int CPC = 8;                 // channels per 16-byte chunk
     constexpr int NCH = C / CPC;           // chunks per tap (= K / 8)
@@ -181,9 +184,11 @@ __global__ void __launch_bounds__(NT, 1) dcn_tc_kernel(const DcnArgs a, int stag
         const int G = a.groups;
         const int g = (cc * CPC) / (a.cin_pad / G);
         const bool tapm = a.om_tap_major != 0;
-        // this chunk's plane of 32-byte pixel pairs (below 4 GiB)
-        const uint8_t *plane = static_cast<const uint8_t *>(cc < NCH / 2 ? a.x : a.x_hi) + (int64_t)(cc % (NCH / 2)) * HW * 32;
-        const uint32_t rowb = (uint32_t)W * 32u;
+        // this chunk's plane of pixel pairs, or of single pixels (below 4 GiB)
+        constexpr uint32_t ENTRY = PAIRS ? 32 : 16;
+        const uint8_t *plane = static_cast<const uint8_t *>(!PAIRS || cc < NCH / 2 ? a.x : a.x_hi) +
+                               (int64_t)(PAIRS ? cc % (NCH / 2) : cc) * HW * ENTRY;
+        const uint32_t rowb = (uint32_t)W * ENTRY;
         int s = 0;
         uint32_t ph = 0;
         bool ok = true;
@@ -263,9 +268,21 @@ __global__ void __launch_bounds__(NT, 1) dcn_tc_kernel(const DcnArgs a, int stag
                     wxa[h] = x0 < 0 ? wx1 : wx0;
                     wxb[h] = x0 < 0 ? 0.f : wx1;
                     const bool need = wxa[h] != 0.f || wxb[h] != 0.f;
-                    const uint32_t o0 = ((uint32_t)y0 * (uint32_t)W + (uint32_t)max(x0, 0)) * 32u;
-                    if (need && wy[h][0] != 0.f) ld_global_nc_v8(plane + o0, v[h][0]);
-                    if (need && wy[h][1] != 0.f) ld_global_nc_v8(plane + (o0 + rowb), v[h][1]);
+                    const uint32_t o0 = ((uint32_t)y0 * (uint32_t)W + (uint32_t)max(x0, 0)) * ENTRY;
+                    // single pixels: the row's last one has no right neighbour (its weight is zero)
+                    const uint32_t next = max(x0, 0) + 1 < W ? ENTRY : 0u;
+                    auto load = [&](uint32_t o, uint32_t (&r)[8]) {
+                        if constexpr (PAIRS) {
+                            ld_global_nc_v8(plane + o, r);
+                        } else {
+                            const uint4 p0 = __ldg(reinterpret_cast<const uint4 *>(plane + o));
+                            const uint4 p1 = __ldg(reinterpret_cast<const uint4 *>(plane + (o + next)));
+                            r[0] = p0.x; r[1] = p0.y; r[2] = p0.z; r[3] = p0.w;
+                            r[4] = p1.x; r[5] = p1.y; r[6] = p1.z; r[7] = p1.w;
+                        }
+                    };
+                    if (need && wy[h][0] != 0.f) load(o0, v[h][0]);
+                    if (need && wy[h][1] != 0.f) load(o0 + rowb, v[h][1]);
                 }
                 // the corner loads are in flight while the warp waits for a free stage
                 const bool got = mbar_wait_bounded(&empty[s], ph ^ 1, abort, WAIT_NS);
@@ -428,7 +445,7 @@ __global__ void __launch_bounds__(NT, 1) dcn_tc_kernel(const DcnArgs a, int stag
     }
 }
 
-template <typename T, int NS, int C, bool PLANAR>
+template <typename T, int NS, int C, bool PLANAR, bool PAIRS>
 cudaError_t run(const DcnArgs &a, cudaStream_t st) {
     constexpr uint32_t STAGE = (C / 8) * TM * 16;
     constexpr uint32_t wbytes = 9 * (C / 8) * NS * 16;
@@ -438,8 +455,8 @@ cudaError_t run(const DcnArgs &a, cudaStream_t st) {
     if (stages < 2) return cudaErrorInvalidConfiguration;
     int smem = 2048 + (int)wround + stages * (int)STAGE;
     if (smem < 118 * 1024) smem = 118 * 1024;
-    auto kern = dcn_tc_kernel<T, NS, C, PLANAR>;
-    cudaError_t e = set_smem_limit<dcn_tc_kernel<T, NS, C, PLANAR>>(smem);
+    auto kern = dcn_tc_kernel<T, NS, C, PLANAR, PAIRS>;
+    cudaError_t e = set_smem_limit<dcn_tc_kernel<T, NS, C, PLANAR, PAIRS>>(smem);
     if (e != cudaSuccess) return e;
     const int tiles = ((a.W + TX - 1) / TX) * ((a.H + TY - 1) / TY);
     int grid = device_sm_count();
@@ -450,7 +467,9 @@ cudaError_t run(const DcnArgs &a, cudaStream_t st) {
 // One thread per (pixel, 8-channel chunk), chunk fastest: a warp reads four pixels' 128-byte
 // channel lines (and their right neighbours, which L1 holds) and writes four 32-byte entries of
 // eight planes, 128 contiguous bytes each, with one 32-byte store a lane (two 16-byte stores wrote each
-// sector in halves: 7 us more at 960 x 540).
+// sector in halves: 7 us more at 960 x 540).  PAIRS = false writes 16-byte entries, all eight planes
+// to lo.
+template <bool PAIRS>
 __global__ void __launch_bounds__(256) dcn_pairs_kernel(const uint4 *__restrict__ x, int64_t HW, int W, int per,
                                                         uint4 *__restrict__ lo, uint4 *__restrict__ hi) {
     const int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -460,6 +479,10 @@ __global__ void __launch_bounds__(256) dcn_pairs_kernel(const uint4 *__restrict_
     const uint4 *src = x + ((int64_t)(cc / per) * HW + p) * per + cc % per;  // per: chunks per pixel line
     const bool last = (int)(p % W) == W - 1;
     const uint4 v0 = __ldg(src);
+    if (!PAIRS) {
+        lo[(int64_t)cc * HW + p] = v0;
+        return;
+    }
     const uint4 v1 = last ? make_uint4(0u, 0u, 0u, 0u) : __ldg(src + per);
     st_global_v8((cc < 4 ? lo : hi) + ((int64_t)(cc & 3) * HW + p) * 2, v0, v1);
 }
@@ -496,8 +519,11 @@ __global__ void __launch_bounds__(256) dcn_pairs_planar_kernel(const float *__re
 cudaError_t launch_dcn_pairs(const void *x, int H, int W, int x_cpc, void *lo, void *hi, cudaStream_t st) {
     if (x_cpc != 8 && x_cpc != 64) return cudaErrorInvalidValue;
     const int64_t HW = (int64_t)H * W;
-    dcn_pairs_kernel<<<(unsigned)((HW * 8 + 255) / 256), 256, 0, st>>>(static_cast<const uint4 *>(x), HW, W, x_cpc / 8,
-                                                                       static_cast<uint4 *>(lo), static_cast<uint4 *>(hi));
+    const unsigned grid = (unsigned)((HW * 8 + 255) / 256);
+    const uint4 *xs = static_cast<const uint4 *>(x);
+    uint4 *l = static_cast<uint4 *>(lo), *h = static_cast<uint4 *>(hi);
+    if (h) dcn_pairs_kernel<true><<<grid, 256, 0, st>>>(xs, HW, W, x_cpc / 8, l, h);
+    else dcn_pairs_kernel<false><<<grid, 256, 0, st>>>(xs, HW, W, x_cpc / 8, l, h);
     return cudaGetLastError();
 }
 
@@ -515,16 +541,19 @@ cudaError_t launch_dcn_tc(const DcnArgs &a0, cudaStream_t st) {
     a.starve = test_starve();
     if (a.y_cpc == 0) a.y_cpc = 8;
     if (a.cin_pad != 64 || a.cout_pad != 64 || (a.cin_pad / a.groups) % 8) return cudaErrorNotSupported;
-    if (!a.x_hi || (a.y_cpc != 8 && a.y_cpc != 64)) return cudaErrorNotSupported;
+    const bool planar = a.om_mask != nullptr, pairs = a.x_hi != nullptr;
+    if ((planar && !pairs) || (a.y_cpc != 8 && a.y_cpc != 64)) return cudaErrorNotSupported;
     if (a.om_tap_major && a.groups % 2) return cudaErrorNotSupported;
     // 32-bit gather offsets into a plane of x and into the offsets and mask
     if ((int64_t)a.H * a.W * 32 >= (int64_t(1) << 32) || (int64_t)a.H * a.W * a.om_cpad >= (int64_t(1) << 31))
         return cudaErrorNotSupported;
-    const bool planar = a.om_mask != nullptr;
-    if (a.in_dt == DT_BF16 && a.out_dt == DT_BF16)
-        return planar ? run<__nv_bfloat16, 64, 64, true>(a, st) : run<__nv_bfloat16, 64, 64, false>(a, st);
-    if (a.in_dt == DT_F16 && a.out_dt == DT_F16)
-        return planar ? run<__half, 64, 64, true>(a, st) : run<__half, 64, 64, false>(a, st);
+    auto go = [&](auto elem) {
+        using T = decltype(elem);
+        if (planar) return run<T, 64, 64, true, true>(a, st);
+        return pairs ? run<T, 64, 64, false, true>(a, st) : run<T, 64, 64, false, false>(a, st);
+    };
+    if (a.in_dt == DT_BF16 && a.out_dt == DT_BF16) return go(__nv_bfloat16{});
+    if (a.in_dt == DT_F16 && a.out_dt == DT_F16) return go(__half{});
     return cudaErrorNotSupported;
 }
 

@@ -169,7 +169,9 @@ struct Step {
     int widx = -1;       // weights variant (input channels permuted), -1 = the layer's own
     int om_t = -1;       // DCN: offsets/mask tensor
     bool om_tap_major = false;  // DCN: om channels in tap-major order (its head's rows permuted)
-    void *pair_hi = nullptr;    // DCN: second half of its input's pixel pairs (tensor-core path)
+    // DCN (tensor-core path): its input's pixel pairs; without pair_hi its planes, in pair_lo unless
+    // the input is laid out so
+    void *pair_lo = nullptr, *pair_hi = nullptr;
     std::vector<int> skip_frames;  // final outputs: frames whose upsampled mean is added
     int in_t = -1;       // input tensor id (SRC_TENSOR)
     int src = SRC_TENSOR;
@@ -257,7 +259,6 @@ struct nvisr_filter {
     std::vector<Weights> weights;  // per layer (shared layers point to the owner)
     std::vector<int> om_tap_g;     // per layer: G when its output rows are stored tap-major, else 0
     std::vector<Tensor> tensors;
-    void *dcn_lo = nullptr;        // first half of a DCN's input in pixel pairs (tensor-core path)
     std::vector<Step> steps;
     std::vector<char> blk;           // step i and i + 1 form a residual block run as one fused launch
     int pack_t = -1;               // tensor id of the packed tuple
@@ -1292,20 +1293,23 @@ nvisr_status build_plan_group(nvisr_filter *f, const float *blob) {
             f->wvar.push_back(Wv);
         }
     }
-    // The tensor-core DCN gathers from its input copied into pixel pairs.  Half of them go to a
-    // buffer that holds nothing while their step runs: the float32 image of an output that only
-    // later steps of the run write (its values of an earlier run have left it, since a run
-    // rewrites it anyway), or a pool buffer that no live tensor has; else to one of their own.
-    auto idle_buffer = [&](int step, size_t bytes) -> void * {
+    // The tensor-core DCN gathers from its input copied into pixel pairs, or, at half the memory,
+    // into 8-channel planes, which a tensor blocked by 8 channels is already.  The plan has memory
+    // of its own for planes only.  The pairs' second half goes to a buffer that holds nothing while
+    // their step runs: the float32 image of an output that only later steps of the run write (its
+    // values of an earlier run have left it, since a run rewrites it anyway), or a pool buffer that
+    // no live tensor has.  Most networks have one (a 4x output image, or a tensor of the layers
+    // after the alignment); a step without one gathers from planes.
+    auto idle_buffer = [&](int step, size_t bytes, const void *taken) -> void * {
         if (sizeof(float) * 3 * f->opitch * H * net.scale_y >= bytes)
             for (int k = 0; k < f->run_out; ++k) {
                 int first = -1;
                 for (int i = (int)f->steps.size() - 1; i >= 0; --i)
                     if (f->steps[i].out_t < 0 && f->steps[i].out_index == k) first = i;
-                if (first > step) return f->out_rgb[k];
+                if (first > step && f->out_rgb[k] != taken) return f->out_rgb[k];
             }
         for (const Buf &b : pool) {
-            bool free = b.bytes >= bytes;
+            bool free = b.bytes >= bytes && b.p != taken;
             for (int t = 0; t < n && free; ++t)
                 free = f->tensors[t].parent >= 0 || f->tensors[t].ptr != b.p || step < first_def[t] ||
                        step > std::max(first_def[t], last_use[t]);
@@ -1313,22 +1317,23 @@ nvisr_status build_plan_group(nvisr_filter *f, const float *blob) {
         }
         return nullptr;
     };
-    size_t lo = 0, hi = 0;
+    size_t planes = 0;
+    for (const Step &st : f->steps)
+        if (st.op == OP_DCN && f->tc && f->tensors[st.in_t].cpc != 8)
+            planes = std::max(planes, (size_t)DCN_PAIR_BYTES * f->tensors[st.in_t].H * f->tensors[st.in_t].W);
+    void *own = nullptr;
+    if (planes) {
+        nvisr_status s = dalloc(f->eng, planes, f->owned, &own, f->guard);
+        if (s != NVISR_OK) return s;
+    }
     for (size_t i = 0; i < f->steps.size(); ++i) {
         Step &st = f->steps[i];
         if (st.op != OP_DCN || !f->tc) continue;
         const size_t bytes = (size_t)DCN_PAIR_BYTES * f->tensors[st.in_t].H * f->tensors[st.in_t].W;
-        lo = std::max(lo, bytes);
-        st.pair_hi = idle_buffer((int)i, bytes);
-        if (!st.pair_hi) hi = std::max(hi, bytes);
+        st.pair_hi = idle_buffer((int)i, bytes, nullptr);
+        st.pair_lo = planes >= bytes ? own : idle_buffer((int)i, bytes, st.pair_hi);
+        if (!st.pair_lo) st.pair_hi = nullptr;
     }
-    void *own = nullptr;
-    for (auto [bytes, p] : {std::pair<size_t, void **>(lo, &f->dcn_lo), std::pair<size_t, void **>(hi, &own)}) {
-        nvisr_status s = bytes ? dalloc(f->eng, bytes, f->owned, p, f->guard) : NVISR_OK;
-        if (s != NVISR_OK) return s;
-    }
-    for (Step &st : f->steps)
-        if (st.op == OP_DCN && !st.pair_hi) st.pair_hi = own;
     for (Tensor &T : f->tensors)
         if (T.parent >= 0) {
             const Tensor &P = f->tensors[T.parent];
@@ -1563,9 +1568,11 @@ nvisr_status run_step(nvisr_filter *f, const Step &s, const float *const *frames
         ProfScope ps(f, NVISR_K_DCN);
         if (f->tc) {
             if (in.cpad != 64) return cuda_status(cudaErrorNotSupported, ("dcn layer " + L.name).c_str());
-            cudaError_t e = launch_dcn_pairs(in.ptr, in.H, in.W, in.cpc, f->dcn_lo, s.pair_hi, st);
-            if (e != cudaSuccess) return cuda_status(e, ("dcn layer " + L.name + " relayout").c_str());
-            d.x = f->dcn_lo;
+            if (s.pair_hi || in.cpc != 8) {
+                cudaError_t e = launch_dcn_pairs(in.ptr, in.H, in.W, in.cpc, s.pair_lo, s.pair_hi, st);
+                if (e != cudaSuccess) return cuda_status(e, ("dcn layer " + L.name + " relayout").c_str());
+                d.x = s.pair_lo;
+            }
             d.x_hi = s.pair_hi;
         }
         cudaError_t e = f->tc ? launch_dcn_tc(d, st) : launch_dcn_simt(d, st);

@@ -4,8 +4,10 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
 import paper_2308_03121_gb300 as nv
 import synth
+from gpu_util import fmt_dict, lsb_stats, prequant
 from test_gpu_filter import run_gpu
 
 pytestmark = pytest.mark.gpu
@@ -58,3 +60,74 @@ def test_output_described_before_the_alignment():
     for t, (a, b) in enumerate(zip(want, got)):
         for k in "YUV":
             assert np.array_equal(a[k], b[k]), (t, k)
+
+
+def _two_frame_net(scale, nres, dead_end=False):
+    """Two frames -> one output: extract, offset/mask head, deformable layer, nres residual blocks,
+    output layer.  dead_end adds two layers after the deformable one that nothing reads: the
+    second needs a buffer that is idle before."""
+    rng = np.random.default_rng(synth.BASE_SEED + 92)
+    C, G = 64, 8
+    spec = synth.NetSpec("group", 2, scale, "bilinear", flags="extra")
+    spec.conv(rng, "f0", "frame0", 3, C, act="lrelu")
+    spec.conv(rng, "f1", "frame1", 3, C, act="lrelu", share="f0")
+    rows = np.ones(27 * G)
+    rows[: 18 * G] = synth.OFFSET_GAIN
+    spec.conv(rng, "om", "f0,f1", 2 * C, 27 * G, row_gains=rows)
+    spec.dcn(rng, "al", "f0", "om", C, C, G)
+    prev = "al"
+    for i in range(nres):
+        spec.conv(rng, f"r{i}a", prev, C, C, act="lrelu")
+        spec.conv(rng, f"r{i}b", f"r{i}a", C, C, add=prev, gain=synth.RES_GAIN)
+        prev = f"r{i}b"
+    if dead_end:
+        for k in range(2):
+            spec.conv(np.random.default_rng(k), f"dead{k}", "al", C, C)
+    spec.conv(rng, "tail", prev, C, 3 * scale * scale, ps=2 if scale == 2 else None, gain=synth.TAIL_GAIN)
+    spec.out("tail", skip="frame0")
+    return spec.build()
+
+
+# scale, residual blocks, layers nothing reads, device memory of the 70 x 38 filter with one copy of
+# the deformable layer's input (128 bytes a pixel)
+FORMS = [(1, 0, False, 6632960), (1, 0, True, 7268864), (2, 1, False, 7250688), (2, 0, False, 6614784)]
+
+
+@pytest.mark.parametrize("prec", ["bf16", "fp16"])
+@pytest.mark.parametrize("scale,nres,dead_end,need", FORMS)
+def test_deformable_layer_needs_one_copy_of_its_input(scale, nres, dead_end, need, prec):
+    """Networks at scale 1 and 2, whose output images are too small for half of the pixel pairs, with
+    and without an idle tensor that is not: the filter fits a budget of what it needs with one copy
+    of the layer's input, and its outputs are the oracle's within one code."""
+    W, H, N = 70, 38, 3
+    frames = synth.frames_textured(synth.BASE_SEED + 93, N, W, H, 8, "420", "limited")
+    flags = np.zeros(N, bool)
+    text, blob = _two_frame_net(scale, nres, dead_end)
+    fi, fo = nv.fmt(W, H, 8), nv.fmt(scale * W, scale * H, 8)
+    eng = nv.Engine(hbm_budget_bytes=need)
+    eng.filter(text, blob, fi, fo, prec, scale)
+    eng.close()
+    fdo = fmt_dict(scale * W, scale * H, 8)
+    ref = oracle.run_filter(frames, flags, text, blob, fmt_dict(W, H, 8), fdo, keep_float=True)
+    outs, _ = run_gpu(text, blob, frames, flags, fi, fo, prec, scale=scale, options=nv.OPT_GUARD_BANDS)
+    assert len(outs) == len(ref) > 0
+    for got, r in zip(outs, ref):
+        pq = prequant(r, fdo)
+        mx, _ = lsb_stats(got, {k: oracle.quantise(pq[k], 8) for k in "YUV"})
+        assert mx <= 1, mx
+
+
+@pytest.mark.parametrize("prec", ["bf16", "fp16"])
+def test_gather_from_planes_equals_gather_from_pairs(prec):
+    """The same network with and without the idle buffer that layers nothing reads bring, bit for bit:
+    pixel pairs against 8-channel planes."""
+    W, H, N = 70, 38, 3
+    frames = synth.frames_textured(synth.BASE_SEED + 93, N, W, H, 10, "444", "full")
+    flags = np.zeros(N, bool)
+    fm = nv.fmt(W, H, 10, "444", "full")
+    a, _ = run_gpu(*_two_frame_net(1, 0, False), frames, flags, fm, fm, prec, scale=1)
+    b, _ = run_gpu(*_two_frame_net(1, 0, True), frames, flags, fm, fm, prec, scale=1)
+    assert len(a) == len(b) > 0
+    for x, y in zip(a, b):
+        for k in "YUV":
+            assert np.array_equal(x[k], y[k]), k
