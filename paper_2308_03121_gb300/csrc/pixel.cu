@@ -1034,7 +1034,7 @@ cudaError_t launch_pack(const PackArgs &a0, cudaStream_t st) {
     const int upc = chunk_channels(a.dt);
     if (a.cpc == 0) a.cpc = upc;
     if (!pack_rows_fits(a)) return cudaErrorInvalidValue;
-    dim3 blk(128), grd((a.W / 4 + 127) / 128, a.H);
+    dim3 blk(128), grd(((a.W + 3) / 4 + 127) / 128, a.H);
     switch (a.dt) {
         case DT_F32: pack_rows_kernel<float><<<grd, blk, 0, st>>>(a); break;
         case DT_BF16: pack_rows_kernel<__nv_bfloat16><<<grd, blk, 0, st>>>(a); break;
@@ -1095,7 +1095,7 @@ cudaError_t launch_pack_table(const PackArgs *host_tab, const PackArgs *dev_tab,
         maxw = std::max(maxw, a.W);
         maxh = std::max(maxh, a.H);
     }
-    dim3 blk(128), grd((maxw / 4 + 127) / 128, maxh, n);
+    dim3 blk(128), grd(((maxw + 3) / 4 + 127) / 128, maxh, n);
     switch (host_tab[0].dt) {
         case DT_F32: pack_rows_table_kernel<float><<<grd, blk, 0, st>>>(dev_tab); break;
         case DT_BF16: pack_rows_table_kernel<__nv_bfloat16><<<grd, blk, 0, st>>>(dev_tab); break;
