@@ -33,7 +33,7 @@ __global__ void __launch_bounds__(256) weights_kernel(WeightArgs a0, WeightArgs 
     const WeightArgs &a = blockIdx.y ? a1 : a0;
     constexpr int UPC = 16 / (int)sizeof(T);  // elements of a 16-byte unit
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
-    if (t0 < a.nbias) a.dst_bias[t0] = a.bias && t0 < a.cout ? a.bias[t0] : 0.f;
+    for (int64_t i = t0; i < a.nbias; i += step) a.dst_bias[i] = a.bias && i < a.cout ? a.bias[i] : 0.f;
     const int kk = a.k * a.k;
     T *dst = static_cast<T *>(a.dst);
     for (int64_t i = t0; i < total; i += step) {
