@@ -90,6 +90,7 @@ struct BlockParams {
     const uint8_t *w1, *w2;    // stacked weights of conv1 and conv2
     const float *b1, *b2;      // biases [64]
     int *err;
+    int w_fresh;               // wait for the previous kernels before the weights and biases too
     int starve;                // test drill: no input is loaded, the pipeline waits run out
     float *yp;                 // PLANAR: the output [64][H][W] float32
 };
@@ -187,6 +188,7 @@ __global__ void __launch_bounds__(BTHREADS, 1)
     // barrier `bar` of CTA 0, for arrivals from either CTA
     auto lead_bar = [&](uint64_t *bar) { return mapa_shared(smem_u32(bar), 0u); };
 
+    if (p.w_fresh) griddep_wait();
     if (threadIdx.x == 0) {
         for (int k = 0; k < XST; ++k) {
             mbar_init(&full[k], 1);
@@ -207,7 +209,8 @@ __global__ void __launch_bounds__(BTHREADS, 1)
         mbar_init(drain, 1);
         *abort = 0;
         fence_mbarrier_init();
-        // weights are written once at filter creation: loaded before the wait on the previous kernel
+        // a filter's weights are written once at its creation: loaded before the wait on the previous
+        // kernel (a layer call's after the one above)
         mbar_arrive_expect_tx(wbar, 2 * WB);
         for (int c = 0; c < 2; ++c)
             for (int kx = 0; kx < 3; ++kx)
@@ -621,6 +624,7 @@ BlockParams block_params(const ConvArgs &c1, const ConvArgs &c2) {
     p.b1 = c1.bias;
     p.b2 = c2.bias;
     p.err = c1.err ? c1.err : c2.err;
+    p.w_fresh = c1.w_fresh | c2.w_fresh;
     p.starve = test_starve();
     p.yp = c2.y_planar;
     return p;

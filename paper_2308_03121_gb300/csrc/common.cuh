@@ -183,6 +183,7 @@ struct ConvArgs {
     int64_t ring_pitch;
     int tslot[8];
     int *err;                // device error word (tensor-core kernels), may be null
+    int w_fresh;             // w, w_rows and bias come from a kernel (launch_weights), see launch_dependent
     // FP32 3x3 layers without a shuffle: x, y and res are planar float32 [C][H][W] with cin
     // real input channels
     int planar, cin;
@@ -300,6 +301,7 @@ struct DcnArgs {
     int in_dt, out_dt;
     float acc_scale, out_scale;
     int *err;
+    int w_fresh;             // w and bias come from a kernel (launch_weights), see launch_dependent
     int starve;              // test drill: the gather loads nothing, the pipeline waits run out
 };
 cudaError_t launch_dcn_simt(const DcnArgs &a, cudaStream_t st);
@@ -357,7 +359,12 @@ int test_starve();
 // start (barriers, TMEM, weights) while the stream's previous kernel drains; the kernel waits
 // (griddepcontrol.wait) for that kernel's completion before it touches activations.  Under
 // stream capture the attribute becomes a programmatic edge of the graph.  Such a kernel reads
-// nothing before that wait but data no kernel writes (weights and biases uploaded by copies).
+// nothing before that wait but data no kernel writes: a filter's weights and biases, uploaded by
+// copies.  Those of a layer call come from launch_weights two launches earlier, with a layout kernel
+// between them, and are written only for certain once the kernel's own wait is over: w_fresh puts
+// that wait before their loads.  It covers launch_weights because every layout kernel launched so
+// (pack_lines_kernel, pack_units_kernel, dcn_pairs_planar_kernel) waits for its predecessor in turn
+// before it ends.
 template <typename... P, typename... A>
 cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, dim3 threads, int smem, cudaStream_t st, A &&...args) {
     cudaLaunchAttribute at[1];

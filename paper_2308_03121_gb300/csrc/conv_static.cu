@@ -180,7 +180,7 @@ extern "C" nvisr_status nvisr_conv2d_static(int32_t precision, const float *x, i
     a.cout = cout; a.cout_pad = cout_pad; a.k = k; a.act = act; a.res = dr; a.y = dy;
     a.in_dt = dt; a.out_dt = dt; a.acc_scale = 1.f; a.out_scale = 1.f; a.y2_scale = 1.f; a.err = err;
     a.in_cpc = in_cpc; a.out_cpc = out_cpc;
-    a.planar = planar; a.cin = cin;
+    a.planar = planar; a.cin = cin; a.w_fresh = 1;
     if (rows) {
         a.y_planar = y;  // x is a copy by now
         if (res_there) a.res_planar = res;

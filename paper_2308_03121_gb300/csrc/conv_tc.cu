@@ -90,6 +90,7 @@ struct TcParams {
     int ntup;                         // row kernel, 16-channel head: > 0 = read the tuple's ntup float32
     int tslot[8];                     //   frames from the ring (slots tslot[]) instead of a packed tensor
     int *err;
+    int w_fresh;                      // wait for the previous kernels before the weights and biases too
     int starve;                       // test drill: the producer loads no input, the pipeline waits run out
     FusedRq rq;                       // 2 x 2 shuffle tail: requantise in the epilogue
 };
@@ -166,6 +167,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) conv_tc_kernel(const __grid_const
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int slice = blockIdx.x % p.nslice;
+    if (p.w_fresh) griddep_wait();
     if (threadIdx.x >= 64 && threadIdx.x < 64 + NS) sbias[threadIdx.x - 64] = p.bias[slice * NS + threadIdx.x - 64];
     const int cta_stride = gridDim.x / p.nslice;
     const int cta0 = blockIdx.x / p.nslice;
@@ -186,7 +188,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) conv_tc_kernel(const __grid_const
         mbar_init(drain, 1);
         *abort = 0;
         fence_mbarrier_init();
-        // the weights are not the previous kernel's: they load before the wait below
+        // the weights are not the previous kernel's: they load before the wait below (or after the
+        // one above)
         mbar_arrive_expect_tx(wbar, p.wbytes);
         const uint8_t *wsrc = p.wts + (size_t)slice * p.wbytes;
         for (uint32_t off = 0; off < p.wbytes; off += 32768u)
@@ -715,6 +718,7 @@ __global__ void __launch_bounds__(rows_threads(CIN, MULTI), 1) conv_rows_kernel(
     auto ymap_of = [&](int pi) { return MULTI ? &probs[pi].ymap : &ymap; };
     auto rmap_of = [&](int pi) { return MULTI ? &probs[pi].rmap : &rmap; };
     auto width_of = [&](int pi) { return MULTI ? probs[pi].W : p.W; };
+    if (p.w_fresh) griddep_wait();
     if (threadIdx.x >= 64 && threadIdx.x < 64 + NPR)
         sbias[threadIdx.x - 64] = p.bias[PSB ? 4 * (threadIdx.x - 64) + slice : slice * NPR + threadIdx.x - 64];
     // 16-channel head reading the tuple's float32 frames (ntup > 0): warps 0 and 11 convert
@@ -751,8 +755,8 @@ __global__ void __launch_bounds__(rows_threads(CIN, MULTI), 1) conv_rows_kernel(
         grp_stop[1] = 0;
         *ready = 0;
         fence_mbarrier_init();
-        // the weights are written once at filter creation, so they load before the wait
-        // below, while the previous layer may still be running
+        // a filter's weights are written once at its creation, so they load before the wait
+        // below, while the previous layer may still be running (a layer call's after the one above)
         mbar_arrive_expect_tx(wbar, 3 * WKX);
         const uint8_t *wsrc = p.wts + (size_t)slice * 3 * WKX;
         for (uint32_t off = 0; off < 3 * WKX; off += 32768u)
@@ -2051,6 +2055,7 @@ TcParams rows_params(const ConvArgs &a) {
     p.err = a.err;
     p.y_planar = a.y_planar;
     p.res_planar = a.res_planar;
+    p.w_fresh = a.w_fresh;
     p.starve = test_starve();
     return p;
 }
@@ -2347,6 +2352,7 @@ cudaError_t launch_conv_tc(const ConvArgs &a, cudaStream_t st) {
     p.y2 = static_cast<uint8_t *>(a.y2); p.y2_scale = a.y2_scale; p.amax = a.amax;
     p.ps_out = a.ps_out; p.ps_pitch = a.ps_pitch; p.skip = a; p.ps_act = a.ps_act;
     p.err = a.err;
+    p.w_fresh = a.w_fresh;
     p.starve = test_starve();
     return v->fn(map, p, st);
 }

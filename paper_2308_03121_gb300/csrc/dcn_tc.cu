@@ -142,6 +142,7 @@ __global__ void __launch_bounds__(NT, 1) dcn_tc_kernel(const DcnArgs a, int stag
     const int ntiles = tiles_x * ((H + TY - 1) / TY);
     const int S = stages;
 
+    if (a.w_fresh) griddep_wait();
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
             mbar_init(&full[s], NGATHER);
@@ -154,7 +155,8 @@ __global__ void __launch_bounds__(NT, 1) dcn_tc_kernel(const DcnArgs a, int stag
         mbar_init(wbar, 1);
         *abort = 0;
         fence_mbarrier_init();
-        // the weights are not the previous kernel's: they load before the wait below
+        // the weights are not the previous kernel's: they load before the wait below (or after the
+        // one above)
         mbar_arrive_expect_tx(wbar, wbytes);
         for (uint32_t off = 0; off < wbytes; off += 32768u)
             bulk_load(wsm + off, static_cast<const uint8_t *>(a.w) + off, min(32768u, wbytes - off), wbar);

@@ -2907,7 +2907,7 @@ nvisr_status nvisr_conv2d(int32_t precision, const float *x, int32_t cin, int32_
     a.cout = cout; a.cout_pad = cout_pad; a.k = k; a.act = act; a.res = dr; a.y = dy;
     a.in_dt = idt; a.out_dt = adt; a.acc_scale = sx * sw; a.out_scale = 1.f; a.y2_scale = 1.f; a.err = sc.err();
     a.in_cpc = in_cpc; a.out_cpc = out_cpc;
-    a.planar = planar; a.cin = cin;
+    a.planar = planar; a.cin = cin; a.w_fresh = 1;
     if (rows) {
         a.y_planar = y;  // x is a copy by now
         if (res_there) a.res_planar = res;
@@ -2953,7 +2953,7 @@ nvisr_status nvisr_resblock2d(int32_t precision, const float *x, int32_t h, int3
     a1.x = dx; a1.cin_pad = 64; a1.in_cpc = 64; a1.out_cpc = 64; a1.H = h; a1.W = w; a1.nimg = 1;
     a1.w_rows = sc.at<void>(o_w1); a1.bias = sc.at<float>(o_b1); a1.cout = 64; a1.cout_pad = 64; a1.k = 3; a1.act = 1;
     a1.y = dh; a1.in_dt = dt; a1.out_dt = dt; a1.acc_scale = 1.f; a1.out_scale = 1.f; a1.y2_scale = 1.f;
-    a1.err = sc.err();
+    a1.err = sc.err(); a1.w_fresh = 1;
     ConvArgs a2 = a1;
     a2.x = dh; a2.w_rows = sc.at<void>(o_w2); a2.bias = sc.at<float>(o_b2); a2.act = 0; a2.res = dx;
     a2.y_planar = y;  // and a2.y, of which only the address is used, stays the middle tensor's
@@ -3013,7 +3013,7 @@ nvisr_status nvisr_dcn2d(int32_t precision, const float *x, int32_t cin, int32_t
     d.x_hi = tc ? sc.at<void>(o_xh) : nullptr;
     d.w = wa.dst; d.bias = wa.dst_bias; d.cout = cout; d.cout_pad = cout_pad; d.y = dy;
     d.in_dt = adt; d.out_dt = adt; d.acc_scale = 1.f; d.out_scale = 1.f; d.err = sc.err();
-    d.y_cpc = y_cpc;
+    d.y_cpc = y_cpc; d.w_fresh = 1;
     cudaError_t e = tc ? launch_dcn_tc(d, st) : launch_dcn_simt(d, st);
     if (e != cudaSuccess) return cuda_status(e, "dcn2d");
     NVISR_TRY_CUDA(launch_unpack_planar(dy, adt, cout_pad, y_cpc, cout, h, w, 1.f, y, st));

@@ -790,8 +790,9 @@ __global__ void __launch_bounds__(128) pack_rows_table_kernel(const PackArgs *__
 
 // Layout change between a layer's planar float32 tensor [C][HW] and its blocked form, for whole
 // frames without row padding.  The packs are launched as dependents of the weights' layout (or of
-// another pack), which they do not read: they run beside it and end only when it has, so the
-// kernel after them finds both done.  Both directions move each byte once (HBM-bound); what costs time
+// another pack), which they do not read: they run beside it, and every thread waits for it before
+// it ends, so the kernel after them, once it has waited for them, finds both done (launch_dependent).
+// Both directions move each byte once (HBM-bound); what costs time
 // is touching memory in pieces below its 32-byte sectors, so a warp covers full lines on both
 // sides.
 //

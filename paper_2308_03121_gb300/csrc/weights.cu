@@ -27,6 +27,7 @@ __device__ __forceinline__ __nv_fp8_e4m3 to_elem<__nv_fp8_e4m3>(float v) { retur
 // of a layer call changes the input's layout and needs nothing of this one: it may start at
 // once, and itself ends only when this one has (with a residual block's two layers in one launch
 // 357 -> 351 us at 1080p, 444 -> 441 for a 540p deformable layer, 127 -> 124 for a 853 x 479 layer).
+// The layer's own kernel loads this one's results only after its wait (w_fresh, launch_dependent).
 template <typename T>
 __global__ void __launch_bounds__(256) weights_kernel(WeightArgs a0, WeightArgs a1, int64_t total) {
     griddep_launch_dependents();
