@@ -168,13 +168,15 @@ typedef struct nvisr_filter nvisr_filter;
  * Errors: INVALID_ARG (NULL pointers, bad device), CUDA_ERROR. */
 nvisr_status nvisr_engine_create(const nvisr_engine_desc *desc, nvisr_engine **out);
 
-/* Destroy the engine and every filter it still owns. NULL is ignored. */
+/* Destroy the engine and every filter it still owns, and release the kept
+ * scratch of the layer calls (nvisr_release_scratch). NULL is ignored. */
 void nvisr_engine_destroy(nvisr_engine *engine);
 
 /* The cudaStream_t the engine's work is enqueued on. */
 void *nvisr_engine_stream(nvisr_engine *engine);
 
-/* Device bytes currently held by the engine's filters. */
+/* Device bytes currently held by the engine's filters (the layer calls' kept
+ * scratch belongs to no engine and is not counted). */
 int64_t nvisr_engine_bytes_in_use(nvisr_engine *engine);
 
 /* Create a filter: parse and check the network description (Section 3.1: the
@@ -402,11 +404,18 @@ void nvisr_server_destroy(nvisr_server *server);
  * precision's kernel (FP32 SIMT or tensor cores); where that works on the
  * internal layout, the library converts x, and res and y where needed, in
  * scratch device memory that it keeps from call to call (at most 1 GiB per
- * context).  res may be NULL; y may overlap x and res.  All pointers are
+ * context; see nvisr_release_scratch).  res may be NULL; y may overlap x and res.  All pointers are
  * device pointers. */
 nvisr_status nvisr_conv2d(int32_t precision, const float *x, int32_t cin, int32_t h, int32_t w,
                           const float *weight, const float *bias, int32_t cout, int32_t k,
                           int32_t act, const float *res, float *y, void *stream);
+
+/* Frees the scratch device memory that nvisr_conv2d, nvisr_resblock2d and
+ * nvisr_dcn2d keep between calls in the current device's context; calls in
+ * flight on other threads keep theirs.  The next call allocates again (about a
+ * millisecond).  For a program whose other allocations need the memory: this
+ * library's own release it by themselves before they fail. */
+nvisr_status nvisr_release_scratch(void);
 
 /* Size of the fixed device area behind nvisr_conv2d_static (32 MiB per device). */
 #define NVISR_CONV2D_STATIC_SCRATCH_BYTES (32 * 1024 * 1024)

@@ -21,7 +21,7 @@ __all__ = [
     "Batch", "Engine", "Filter", "NvisrError", "Server", "PREC", "Status", "fmt", "lib", "load",
     "nvisr_conv2d", "nvisr_conv2d_static", "nvisr_dcn2d", "nvisr_resblock2d", "nvisr_fig1_layout", "nvisr_group_outputs",
     "nvisr_group_runs",
-    "nvisr_ingest", "nvisr_network_check", "nvisr_requant", "nvisr_selftest",
+    "nvisr_ingest", "nvisr_network_check", "nvisr_release_scratch", "nvisr_requant", "nvisr_selftest",
     "nvisr_tuple_map",
 ]
 
@@ -130,6 +130,7 @@ _SIGS = {
     "nvisr_resblock2d": (_I32, [_I32, _VP, _I32, _I32, _VP, _VP, _VP, _VP, _VP, _I32, _VP]),
     "nvisr_dcn2d": (_I32, [_I32, _VP, _I32, _I32, _I32, _VP, _VP, _I32, _VP, _VP, _I32, _VP, _VP]),
     "nvisr_selftest": (_I32, [_I32P, _I32P]),
+    "nvisr_release_scratch": (_I32, []),
     "nvisr_test_starve": (_I32, [_I32]),
     "nvisr_selftest_swizzle": (_I32, [_I32P]),
     "nvisr_batch_create": (_I32, [_VP, ctypes.POINTER(_VP), _I32, ctypes.POINTER(_VP)]),
@@ -287,6 +288,12 @@ def nvisr_dcn2d(precision, x, offsets, mask, weight, bias, groups, stream=None):
                             bias.data_ptr() if bias is not None else None, cout, y.data_ptr(),
                             _stream_ptr(stream)), "nvisr_dcn2d")
     return y
+
+
+def nvisr_release_scratch():
+    """Free the device memory that the layer calls keep between calls."""
+    load()
+    _check(_LIB.nvisr_release_scratch(), "nvisr_release_scratch")
 
 
 def nvisr_tuple_map(flags, T):

@@ -115,12 +115,7 @@ nvisr_status dalloc(nvisr_engine *e, size_t bytes, std::vector<DevBuf> &owned, v
         return fail(NVISR_OVER_BUDGET, "HBM budget exceeded: need " + std::to_string(bytes) + " more bytes, " +
                                            std::to_string(e->budget - e->used) + " left");
     void *p = nullptr;
-    cudaError_t ce = cudaMalloc(&p, bytes);
-    if (ce == cudaErrorMemoryAllocation) {
-        cudaGetLastError();
-        scratch_trim();  // the per-call entry points' kept working memory
-        ce = cudaMalloc(&p, bytes);
-    }
+    cudaError_t ce = device_malloc(&p, bytes);
     if (ce != cudaSuccess) {
         cudaGetLastError();
         return fail(NVISR_OUT_OF_MEMORY, std::string("cudaMalloc: ") + cudaGetErrorString(ce));
@@ -2039,7 +2034,7 @@ int tune_rps(nvisr_batch *b, nvisr_batch::Plan &P, const PartFrames &pf, cudaStr
 
 nvisr_status build_batch_plan(nvisr_batch *b, nvisr_batch::Plan &P, const PartFrames &pf, cudaStream_t st) {
     const int n = (int)P.parts.size();
-    NVISR_TRY_CUDA(cudaMalloc(&P.pack_dev, sizeof(PackArgs) * n));
+    NVISR_TRY_CUDA(device_malloc((void **)&P.pack_dev, sizeof(PackArgs) * n));
     const size_t nsteps = b->members[0]->steps.size();
     P.tab_host.assign(nsteps, nullptr);
     P.tab_dev.assign(nsteps, nullptr);
@@ -2060,7 +2055,7 @@ nvisr_status build_batch_plan(nvisr_batch *b, nvisr_batch::Plan &P, const PartFr
         }
         if (!blk) continue;
         NVISR_TRY_CUDA(cudaMallocHost(&P.btab_host[si], sizeof(BlockProblem) * n));
-        NVISR_TRY_CUDA(cudaMalloc(&P.btab_dev[si], sizeof(BlockProblem) * n));
+        NVISR_TRY_CUDA(device_malloc((void **)&P.btab_dev[si], sizeof(BlockProblem) * n));
         cudaError_t e = launch_res_block_multi(args.data(), args2.data(), n, P.btab_host[si], P.btab_dev[si], st,
                                                true, false);
         if (e != cudaSuccess) return cuda_status(e, "batched residual block table");
@@ -2075,7 +2070,7 @@ nvisr_status build_batch_plan(nvisr_batch *b, nvisr_batch::Plan &P, const PartFr
         }
         if (!rows) continue;
         NVISR_TRY_CUDA(cudaMallocHost(&P.tab_host[si], sizeof(RowProblem) * n));
-        NVISR_TRY_CUDA(cudaMalloc(&P.tab_dev[si], sizeof(RowProblem) * n));
+        NVISR_TRY_CUDA(device_malloc((void **)&P.tab_dev[si], sizeof(RowProblem) * n));
     }
     P.rps = tune_rps(b, P, pf, st);
     for (size_t si = 0; si < nsteps; ++si) {
@@ -2150,7 +2145,7 @@ nvisr_status nvisr_engine_create(const nvisr_engine_desc *desc, nvisr_engine **o
         }
         e->own_stream = true;
     }
-    if (cudaMalloc(&e->err_word, sizeof(int)) != cudaSuccess || cudaMemset(e->err_word, 0, sizeof(int)) != cudaSuccess ||
+    if (device_malloc((void **)&e->err_word, sizeof(int)) != cudaSuccess || cudaMemset(e->err_word, 0, sizeof(int)) != cudaSuccess ||
         cudaHostAlloc(&e->err_host, sizeof(int), cudaHostAllocDefault) != cudaSuccess ||
         cudaStreamCreateWithFlags(&e->copy_stream, cudaStreamNonBlocking) != cudaSuccess) {
         cudaFree(e->err_word);
@@ -2193,6 +2188,7 @@ void nvisr_engine_destroy(nvisr_engine *e) {
     if (e->own_stream) cudaStreamDestroy(e->stream);
     cudaStreamDestroy(e->copy_stream);
     delete e;
+    scratch_trim();
 }
 
 void *nvisr_engine_stream(nvisr_engine *e) { return e ? (void *)e->stream : nullptr; }
@@ -3022,6 +3018,11 @@ nvisr_status nvisr_dcn2d(int32_t precision, const float *x, int32_t cin, int32_t
     return NVISR_OK;
 }
 
+nvisr_status nvisr_release_scratch(void) {
+    scratch_trim();
+    return NVISR_OK;
+}
+
 nvisr_status nvisr_test_starve(int32_t on) {
     g_test_starve = on ? 1 : 0;
     return NVISR_OK;
@@ -3030,7 +3031,7 @@ nvisr_status nvisr_test_starve(int32_t on) {
 nvisr_status nvisr_selftest(int32_t *mismatches_bf16, int32_t *mismatches_fp8) {
     if (!mismatches_bf16 || !mismatches_fp8) return fail(NVISR_INVALID_ARG, "selftest: NULL argument");
     int *d;
-    NVISR_TRY_CUDA(cudaMalloc(&d, 2 * sizeof(int)));
+    NVISR_TRY_CUDA(device_malloc((void **)&d, 2 * sizeof(int)));
     cudaMemset(d, 0, 2 * sizeof(int));
     int e1 = tc_selftest(0, d, 0);
     int e2 = tc_selftest(1, d + 1, 0);
@@ -3048,7 +3049,7 @@ nvisr_status nvisr_selftest(int32_t *mismatches_bf16, int32_t *mismatches_fp8) {
 nvisr_status nvisr_selftest_swizzle(int32_t *out16) {
     if (!out16) return fail(NVISR_INVALID_ARG, "selftest_swizzle: NULL argument");
     int *d;
-    NVISR_TRY_CUDA(cudaMalloc(&d, 16 * sizeof(int)));
+    NVISR_TRY_CUDA(device_malloc((void **)&d, 16 * sizeof(int)));
     cudaMemset(d, 0, 16 * sizeof(int));
     const int e = tc_probe_sw128(d, 0);
     const cudaError_t se = cudaDeviceSynchronize();

@@ -63,10 +63,15 @@ void free_slab(const Slab &s) {
 }  // namespace
 
 void scratch_trim() {
-    const uint64_t ctx = context_id();
     std::vector<Slab> out;
+    Kept &k = kept();
     {
-        Kept &k = kept();
+        std::lock_guard<std::mutex> lock(k.mu);
+        if (k.slabs.empty()) return;
+    }
+    (void)cudaFree(nullptr);  // binds the device's context to a thread new to it
+    const uint64_t ctx = context_id();
+    {
         std::lock_guard<std::mutex> lock(k.mu);
         for (size_t i = 0; i < k.slabs.size();)
             if (k.slabs[i].ctx == ctx) {
@@ -77,6 +82,16 @@ void scratch_trim() {
             }
     }
     for (const Slab &s : out) free_slab(s);
+}
+
+cudaError_t device_malloc(void **p, size_t bytes) {
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation) {
+        (void)cudaGetLastError();
+        scratch_trim();
+        e = cudaMalloc(p, bytes);
+    }
+    return e;
 }
 
 cudaError_t Scratch::open() {
@@ -105,12 +120,7 @@ cudaError_t Scratch::open() {
     }
     if (!dev_) {
         void *p = nullptr, *h = nullptr, *hd = nullptr;
-        e = cudaMalloc(&p, want);
-        if (e == cudaErrorMemoryAllocation) {
-            (void)cudaGetLastError();
-            scratch_trim();
-            e = cudaMalloc(&p, want);
-        }
+        e = device_malloc(&p, want);
         if (e == cudaSuccess) e = cudaHostAlloc(&h, sizeof(int), cudaHostAllocMapped | cudaHostAllocPortable);
         if (e == cudaSuccess) e = cudaHostGetDevicePointer(&hd, h, 0);
         if (e != cudaSuccess) {
