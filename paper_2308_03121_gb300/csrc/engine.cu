@@ -1726,7 +1726,7 @@ nvisr_status forward_group(nvisr_filter *f, const std::vector<int64_t> &idx) {
             pa.cpad = t.cpad;
             pa.dt = t.dt;
             pa.cpc = t.cpc;
-                    cudaError_t e;
+            cudaError_t e;
             {
                 ProfScope ps(f, NVISR_K_PACK);
                 e = launch_pack(pa, f->eng->stream);
@@ -2642,7 +2642,7 @@ nvisr_status nvisr_batch_step(nvisr_batch *b, int32_t *produced) {
             pa.cpad = pk.cpad;
             pa.dt = pk.dt;
             pa.cpc = pk.cpc ? pk.cpc : chunk_channels(pk.dt);
-                    if (!pack_rows_fits(pa)) return fail(NVISR_INTERNAL, "batch_step: tuple pack layout not supported");
+            if (!pack_rows_fits(pa)) return fail(NVISR_INTERNAL, "batch_step: tuple pack layout not supported");
             for (const Step &s : f->steps)
                 if (s.op == OP_CONV && s.out_t < 0) set_final_skip(f, s, pf.frames[i].data());
         }

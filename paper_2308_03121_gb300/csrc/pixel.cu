@@ -117,59 +117,23 @@ __device__ __forceinline__ float chroma_at(const uint8_t *base, int64_t pitch, i
     return (ld_sample(row, i) - off) / den;
 }
 
-// Vertically interpolated chroma column i for luma row y (4:2:0).
-template <typename S>
-__device__ __forceinline__ float chroma_v(const uint8_t *base, int64_t pitch, int Hc, int Wc,
-                                          int y, int i, int loc, float off, float den) {
-    const int j = y >> 1;
-    const float c0 = chroma_at<S>(base, pitch, Hc, Wc, j, i, off, den);
-    if (loc == NVISR_CHROMA_POINT) return c0;
-    const int jn = (y & 1) ? j + 1 : j - 1;
-    const float c1 = chroma_at<S>(base, pitch, Hc, Wc, jn, i, off, den);
-    return 0.75f * c0 + 0.25f * c1;
-}
-
-// Full-resolution chroma at luma (y, x) for 4:2:0, given the format siting.
-template <typename S>
-__device__ __forceinline__ float chroma_up(const uint8_t *base, int64_t pitch, int Hc, int Wc,
-                                           int y, int x, int loc, float off, float den) {
-    const int i = x >> 1;
-    const float v0 = chroma_v<S>(base, pitch, Hc, Wc, y, i, loc, off, den);
-    if (loc == NVISR_CHROMA_POINT) return v0;
-    if (loc == NVISR_CHROMA_LEFT) {
-        if ((x & 1) == 0) return v0;
-        const float v1 = chroma_v<S>(base, pitch, Hc, Wc, y, i + 1, loc, off, den);
-        return 0.5f * (v0 + v1);
-    }
-    const int in = (x & 1) ? i + 1 : i - 1;  // CENTER
-    const float v1 = chroma_v<S>(base, pitch, Hc, Wc, y, in, loc, off, den);
-    return 0.75f * v0 + 0.25f * v1;
-}
-
+// 4:4:4 ingest, one thread per 4 pixels of a row.
 template <typename S, bool XF>
 __global__ void __launch_bounds__(256) ingest_kernel(
     const uint8_t *__restrict__ yp, int64_t py, const uint8_t *__restrict__ up, int64_t pu,
-    const uint8_t *__restrict__ vp, int64_t pv, int H, int W, int sub420, int loc, RangeConst rc,
-    float *__restrict__ out, int64_t pitch) {
+    const uint8_t *__restrict__ vp, int64_t pv, int H, int W, RangeConst rc, float *__restrict__ out, int64_t pitch) {
     const int qx = blockIdx.x * blockDim.x + threadIdx.x;  // quad of 4 pixels
     const int y = blockIdx.y;
     const int x0 = qx * 4;
     if (x0 >= W) return;
-    const int Hc = sub420 ? H / 2 : H, Wc = sub420 ? W / 2 : W;
     const S *yrow = reinterpret_cast<const S *>(yp + (int64_t)y * py);
     float r[4], g[4], b[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
         const int x = min(x0 + e, W - 1);
         const float Y = (ld_sample(yrow, x) - rc.y_off) / rc.y_den;
-        float cb, cr;
-        if (sub420) {
-            cb = chroma_up<S>(up, pu, Hc, Wc, y, x, loc, rc.c_off, rc.c_den);
-            cr = chroma_up<S>(vp, pv, Hc, Wc, y, x, loc, rc.c_off, rc.c_den);
-        } else {
-            cb = chroma_at<S>(up, pu, Hc, Wc, y, x, rc.c_off, rc.c_den);
-            cr = chroma_at<S>(vp, pv, Hc, Wc, y, x, rc.c_off, rc.c_den);
-        }
+        const float cb = chroma_at<S>(up, pu, H, W, y, x, rc.c_off, rc.c_den);
+        const float cr = chroma_at<S>(vp, pv, H, W, y, x, rc.c_off, rc.c_den);
         if (rc.yuv) {
             r[e] = Y;
             g[e] = cb;
@@ -969,10 +933,9 @@ cudaError_t launch_ingest(const nvisr_format &f, const void *y, int64_t py, cons
     }
     dim3 block(64);
     dim3 grid((f.width / 4 + 1 + block.x - 1) / block.x, f.height);
-    const int sub = f.subsampling == NVISR_SUB_420;
     auto run = [&](auto kern) {
         kern<<<grid, block, 0, st>>>((const uint8_t *)y, py, (const uint8_t *)u, pu, (const uint8_t *)v, pv, f.height,
-                                     f.width, sub, f.chroma_loc, rc, out, out_pitch);
+                                     f.width, rc, out, out_pitch);
     };
     if (f.bit_depth <= 8) rc.transfer ? run(ingest_kernel<uint8_t, true>) : run(ingest_kernel<uint8_t, false>);
     else rc.transfer ? run(ingest_kernel<uint16_t, true>) : run(ingest_kernel<uint16_t, false>);
