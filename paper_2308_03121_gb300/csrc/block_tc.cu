@@ -47,6 +47,9 @@
 // then holds the clock near 1.5 GHz (1.55 PFLOP/s, 0.93 of the sustained cuBLAS rate), so what
 // is left is the arithmetic itself, with 5 % of it in the last, 30-pixel column tile.
 //
+// What the SMs hand each other are signals: h rows, x rows, weights and accumulators are written
+// and read in one SM's memory, whichever CTA's thread issues the MMA (mbar_arrive_cluster).
+//
 // Every wait is bounded in time; a CTA that gives up raises the abort flags of both CTAs and
 // the error word.  Both CTAs end with two cluster barriers: between them each waits for the
 // last MMA commit onto its barriers, so neither leaves while the other may still write into
