@@ -62,27 +62,45 @@ def test_output_described_before_the_alignment():
             assert np.array_equal(a[k], b[k]), (t, k)
 
 
-def _two_frame_net(scale, nres, dead_end=False):
+def _two_frame_net(scale, nres, dead_end=False, narrow=""):
     """Two frames -> one output: extract, offset/mask head, deformable layer, nres residual blocks,
-    output layer.  dead_end adds two layers after the deformable one that nothing reads: the
-    second needs a buffer that is idle before."""
+    output layer.  dead_end adds layers after the deformable one that nothing reads: the last needs a
+    buffer that is idle before.  narrow: a deformable layer's input is also concatenated with 16
+    channels of frame 1, so that it is blocked by 8 channels: that of a second layer ("chain", which
+    without the dead ends gathers from the input itself), or that of the only layer, at half size
+    ("pool", whose pixel pairs lie in two idle buffers)."""
     rng = np.random.default_rng(synth.BASE_SEED + 92)
     C, G = 64, 8
     spec = synth.NetSpec("group", 2, scale, "bilinear", flags="extra")
     spec.conv(rng, "f0", "frame0", 3, C, act="lrelu")
-    spec.conv(rng, "f1", "frame1", 3, C, act="lrelu", share="f0")
+    spec.conv(rng, "f1", "frame1", 3, 16 if narrow == "pool" else C, act="lrelu", share=None if narrow == "pool" else "f0")
     rows = np.ones(27 * G)
     rows[: 18 * G] = synth.OFFSET_GAIN
-    spec.conv(rng, "om", "f0,f1", 2 * C, 27 * G, row_gains=rows)
-    spec.dcn(rng, "al", "f0", "om", C, C, G)
-    prev = "al"
+    if narrow == "pool":
+        spec.pool("p0", "f0", C)
+        spec.pool("p1", "f1", 16)
+        spec.conv(rng, "mix", "p0,p1", C + 16, C)
+        spec.conv(rng, "om", "mix", C, 27 * G, row_gains=rows)
+        spec.dcn(rng, "al", "p0", "om", C, C, G)
+        spec.up("ua", "al", C)
+        prev = "ua"
+    else:
+        spec.conv(rng, "om", "f0,f1", 2 * C, 27 * G, row_gains=rows)
+        spec.dcn(rng, "al", "f0", "om", C, C, G)
+        prev = "al"
+    if narrow == "chain":
+        spec.conv(rng, "g1", "frame1", 3, 16, act="lrelu")
+        spec.conv(rng, "mix", "al,g1", C + 16, C)
+        spec.conv(rng, "om2", "mix", C, 27 * G, row_gains=rows)
+        spec.dcn(rng, "al2", "al", "om2", C, C, G)
+        prev = "al2"
     for i in range(nres):
         spec.conv(rng, f"r{i}a", prev, C, C, act="lrelu")
         spec.conv(rng, f"r{i}b", f"r{i}a", C, C, add=prev, gain=synth.RES_GAIN)
         prev = f"r{i}b"
     if dead_end:
-        for k in range(2):
-            spec.conv(np.random.default_rng(k), f"dead{k}", "al", C, C)
+        for k in range(3 if narrow else 2):
+            spec.conv(np.random.default_rng(k), f"dead{k}", prev, C, C)
     spec.conv(rng, "tail", prev, C, 3 * scale * scale, ps=2 if scale == 2 else None, gain=synth.TAIL_GAIN)
     spec.out("tail", skip="frame0")
     return spec.build()
@@ -118,16 +136,22 @@ def test_deformable_layer_needs_one_copy_of_its_input(scale, nres, dead_end, nee
 
 
 @pytest.mark.parametrize("prec", ["bf16", "fp16"])
-def test_gather_from_planes_equals_gather_from_pairs(prec):
-    """The same network with and without the idle buffer that layers nothing reads bring, bit for bit:
-    pixel pairs against 8-channel planes."""
+@pytest.mark.parametrize("narrow", ["", "chain", "pool"])
+def test_gather_from_planes_equals_gather_from_pairs(prec, narrow):
+    """The same network with and without the idle buffers that layers nothing reads bring, bit for bit:
+    pixel pairs against 8-channel planes or the input itself; and the oracle's codes within one."""
     W, H, N = 70, 38, 3
     frames = synth.frames_textured(synth.BASE_SEED + 93, N, W, H, 10, "444", "full")
     flags = np.zeros(N, bool)
     fm = nv.fmt(W, H, 10, "444", "full")
-    a, _ = run_gpu(*_two_frame_net(1, 0, False), frames, flags, fm, fm, prec, scale=1)
-    b, _ = run_gpu(*_two_frame_net(1, 0, True), frames, flags, fm, fm, prec, scale=1)
-    assert len(a) == len(b) > 0
-    for x, y in zip(a, b):
+    a, _ = run_gpu(*_two_frame_net(1, 0, False, narrow), frames, flags, fm, fm, prec, scale=1)
+    b, _ = run_gpu(*_two_frame_net(1, 0, True, narrow), frames, flags, fm, fm, prec, scale=1)
+    fd = fmt_dict(W, H, 10, "444", "full")
+    ref = oracle.run_filter(frames, flags, *_two_frame_net(1, 0, False, narrow), fd, fd, keep_float=True)
+    assert len(a) == len(b) == len(ref) > 0
+    for x, y, r in zip(a, b, ref):
         for k in "YUV":
             assert np.array_equal(x[k], y[k]), k
+        pq = prequant(r, fd)
+        mx, _ = lsb_stats(x, {k: oracle.quantise(pq[k], 10) for k in "YUV"})
+        assert mx <= 1, mx
